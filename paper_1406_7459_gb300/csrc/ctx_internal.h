@@ -35,6 +35,7 @@ struct mm_ctx {
     cudaStream_t cap;          // private stream used only for graph capture
     int device;
     Geom g;
+    Geom gf;                   // geometry of the two-kernel step: g, or a ragged film's carrier lengths
     Launch l;
     float* Kt = nullptr;
     float* Kd = nullptr;       // 2-D spectrum per z offset, exchange folded in (two-kernel step)
@@ -57,6 +58,7 @@ struct mm_ctx {
     FastStepFns fs;            // two-kernel step (power-of-two grids)
     FastSplitFns fsplit;       // compile-time split pass 2 (thick power-of-two samples)
     bool has_fs = false;
+    bool rag = false;          // has_fs through the ragged kernels; Kt is formed on demand
     bool has_ss = false;       // thick power-of-two samples: split pass 2 + the x-step kernel
     bool has_gx = false;       // generic x passes: the step's pass 3 also forms the next x spectrum
     float* Kt_ex = nullptr;    // tensor spectrum with the exchange stencil folded in (has_ss)

@@ -59,9 +59,76 @@ template <> __device__ __forceinline__ void dftp<4>(float2* a) { dft4(a); }
 template <> __device__ __forceinline__ void dftp<8>(float2* a) { dft8(a); }
 template <> __device__ __forceinline__ void dftp<16>(float2* a) { dft16(a); }
 template <> __device__ __forceinline__ void dftp<32>(float2* a) { dft32(a); }
+template <> __device__ __forceinline__ void dftp<3>(float2* a) { dft3(a); }
+template <> __device__ __forceinline__ void dftp<5>(float2* a) { dft5(a); }
 
-// Split of n into P x Q for the two register steps.
+// W_N^k = exp(-2 pi i k / N), k < N, evaluated at compile time in double by
+// the Taylor series of cos and sin on |x| <= pi / 4 and the symmetries of
+// the circle.  Used with compile-time k only.
+template <int N> struct WTab {
+    float c[N] = {}, s[N] = {};
+    constexpr WTab() {
+        for (int k = 0; k < N; ++k) {
+            const int oct = (8 * k) / N;                  // eighth of the circle that 2 pi k / N lies in
+            // angle as quarter q plus x in (-pi/4, pi/4]
+            const int q = (oct + 1) / 2;
+            const double x = 6.28318530717958647692 * k / N - 1.57079632679489661923 * q;
+            double cx = 0, sx = 0, t = 1;
+            for (int i = 0; i < 24; ++i) {                // t = x^i / i!
+                if (i % 4 == 0) cx += t;
+                if (i % 4 == 1) sx += t;
+                if (i % 4 == 2) cx -= t;
+                if (i % 4 == 3) sx -= t;
+                t = t * x / (i + 1);
+            }
+            const double cc = q % 4 == 0 ? cx : (q % 4 == 1 ? -sx : (q % 4 == 2 ? -cx : sx));
+            const double ss = q % 4 == 0 ? sx : (q % 4 == 1 ? cx : (q % 4 == 2 ? -sx : -cx));
+            c[k] = (float)cc;
+            s[k] = (float)-ss;
+        }
+    }
+};
+
+// Forward DFT of length A B in registers (Cooley-Tukey): B DFTs of length A
+// over every B-th input, the twiddles W_AB^{r q}, A DFTs of length B.
+template <int A, int B> __device__ __forceinline__ void dft_ab(float2* a) {
+    constexpr WTab<A * B> w{};
+    float2 c[B][A];
+#pragma unroll
+    for (int r = 0; r < B; ++r) {
+#pragma unroll
+        for (int i = 0; i < A; ++i) c[r][i] = a[r + B * i];
+        dftp<A>(c[r]);
+#pragma unroll
+        for (int q = 1; q < A; ++q)
+            if (r > 0) c[r][q] = cmul(c[r][q], make_float2(w.c[r * q], w.s[r * q]));
+    }
+#pragma unroll
+    for (int q = 0; q < A; ++q) {
+        float2 t[B];
+#pragma unroll
+        for (int r = 0; r < B; ++r) t[r] = c[r][q];
+        dftp<B>(t);
+#pragma unroll
+        for (int r = 0; r < B; ++r) a[q + A * r] = t[r];
+    }
+}
+template <> __device__ __forceinline__ void dftp<6>(float2* a) { dft_ab<2, 3>(a); }
+template <> __device__ __forceinline__ void dftp<12>(float2* a) { dft_ab<4, 3>(a); }
+template <> __device__ __forceinline__ void dftp<20>(float2* a) { dft_ab<4, 5>(a); }
+template <> __device__ __forceinline__ void dftp<24>(float2* a) { dft_ab<8, 3>(a); }
+
+// Split of n into P x Q for the two register steps.  The lengths between
+// the powers of two (ragged samples, film_ragged) keep P even and the group
+// of max(P, Q) threads within 8, 16 or 32 lanes (Fft2::G).
 template <int N> struct Split;
+template <> struct Split<48> { static constexpr int P = 8, Q = 6; };
+template <> struct Split<96> { static constexpr int P = 16, Q = 6; };
+template <> struct Split<192> { static constexpr int P = 16, Q = 12; };
+template <> struct Split<320> { static constexpr int P = 16, Q = 20; };
+template <> struct Split<384> { static constexpr int P = 16, Q = 24; };
+template <> struct Split<640> { static constexpr int P = 32, Q = 20; };
+template <> struct Split<768> { static constexpr int P = 32, Q = 24; };
 template <> struct Split<8> { static constexpr int P = 4, Q = 2; };
 template <> struct Split<16> { static constexpr int P = 4, Q = 4; };
 template <> struct Split<32> { static constexpr int P = 8, Q = 4; };
@@ -95,7 +162,8 @@ template <int R> __device__ __forceinline__ float2 wpi(int q) {
 template <int N> struct Fft2 {
     static constexpr int P = Split<N>::P;
     static constexpr int Q = Split<N>::Q;
-    static constexpr int G = P > Q ? P : Q;        // threads per transform
+    static constexpr int M = P > Q ? P : Q;
+    static constexpr int G = M <= 4 ? M : (M <= 8 ? 8 : (M <= 16 ? 16 : 32));   // threads per transform
     static constexpr int EXS = Q + 1;              // padded exchange row
     static constexpr int EX = P * EXS;             // exchange buffer (complex)
 

@@ -25,7 +25,10 @@ __host__ __device__ constexpr int pzlen(int L) { return L + L / 16 + 1; }
 // one complex line).  Groups of G threads: (pair, half).
 // Mcopy (may be null): a second copy of the rows read, e.g. the device copy
 // of a state that M points to in host memory.
-template <int N, int R>
+// RAG: a ragged sample, g.nx <= N cells per row and g.ny rows of a spectrum
+// row stride g.Jst (ny rounded up): cells past nx and rows past ny are zeros,
+// and the zero rows' spectra (up to Jst) are written like the others.
+template <int N, int R, bool RAG = false>
 __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const float* __restrict__ M,
                                                                 float2* __restrict__ S, float* __restrict__ Mcopy) {
     using F = Fft2<N>;
@@ -33,9 +36,11 @@ __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const flo
     constexpr int T = R * G;                              // the launch's block size
     extern __shared__ float2 sm[];
     float2* tw = sm;
-    float2* ex = tw + L;
+    float2* ta = tw + L;                  // RAG: every twiddle from a table, rounded once (N entries)
+    float2* ex = tw + L + (RAG ? N : 0);
     float2* zb = ex + R * F::EX;
-    const int ntj = g.ny / R;
+    const int ntj = RAG ? (g.Jst + R - 1) / R : g.ny / R;
+    const int nx = RAG ? g.nx : N;
     int b = blockIdx.x;
     const int jt = b % ntj;
     b /= ntj;
@@ -44,31 +49,44 @@ __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const flo
     const int j0 = jt * R;
 #pragma unroll
     for (int i = threadIdx.x; i < L; i += T) tw[i] = __ldg(g.twx + i);
+    if constexpr (RAG) {
+#pragma unroll
+        for (int i = threadIdx.x; i < N; i += T) ta[i] = __ldg(g.twx + 2 * (i / Q) * (i % Q));
+    }
     pdl_wait();                           // M and S may belong to the previous kernel
     __syncthreads();
 
     const int grp = threadIdx.x / G, t = threadIdx.x % G;
     const int p = grp >> 1, h = grp & 1;
     if (t < Q) {
-        const float* ra = M + (size_t)c * g.N + ((size_t)k * g.ny + j0 + 2 * p) * N;
-        const float* rb = ra + N;
+        const float* ra = M + (size_t)c * g.N + ((size_t)k * g.ny + j0 + 2 * p) * nx;
+        const float* rb = ra + nx;
+        const int na = !RAG || j0 + 2 * p < g.ny ? nx : 0, nb = !RAG || j0 + 2 * p + 1 < g.ny ? nx : 0;
         float2 v[P];
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             const int j = t + Q * q;
-            v[q] = make_float2(__ldg(ra + j), __ldg(rb + j));
+            if constexpr (RAG)
+                v[q] = make_float2(j < na ? __ldg(ra + j) : 0.f, j < nb ? __ldg(rb + j) : 0.f);
+            else
+                v[q] = make_float2(__ldg(ra + j), __ldg(rb + j));
         }
         if (Mcopy && h == 0) {
             float* ca = Mcopy + (ra - M);
 #pragma unroll
             for (int q = 0; q < P; ++q) {
                 const int j = t + Q * q;
-                ca[j] = v[q].x;
-                ca[N + j] = v[q].y;
+                if (!RAG || j < na) ca[j] = v[q].x;
+                if (!RAG || j < nb) ca[nx + j] = v[q].y;
             }
         }
-        if (h) F::odd_input(v, t, tw);
-        F::stepA(v, t, tw, ex + grp * F::EX, false);
+        if constexpr (RAG) {
+            if (h) F::odd_input_tab(v, t, tw);
+            F::stepA_tab(v, t, ta, ex + grp * F::EX, false);
+        } else {
+            if (h) F::odd_input(v, t, tw);
+            F::stepA(v, t, tw, ex + grp * F::EX, false);
+        }
     }
     __syncthreads();
     if (t < P) {
@@ -83,9 +101,10 @@ __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const flo
     for (int idx = threadIdx.x; idx < (N + 1) * R; idx += T) {
         const int r = idx % R;
         const int kx = idx / R;
+        if (RAG && j0 + r >= g.Jst) continue;
         const float2* line = zb + (r >> 1) * ZS;
         const float2 zk = line[pz(kx)];
-        const float2 zm = line[pz((L - kx) & (L - 1))];
+        const float2 zm = line[pz(kx == 0 ? 0 : L - kx)];
         float2 o;
         if ((r & 1) == 0) o = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
         else o = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
@@ -379,8 +398,8 @@ __global__ void __launch_bounds__(256) k_pass3_fast(Geom g, LlgCoef cf, const fl
 }
 
 // shared-memory bytes of each fast kernel
-template <int N, int R> constexpr size_t pass1_fast_smem() {
-    return sizeof(float2) * (2 * N + R * Fft2<N>::EX + (R / 2) * pzlen(2 * N));
+template <int N, int R, bool RAG = false> constexpr size_t pass1_fast_smem() {
+    return sizeof(float2) * ((RAG ? 3 : 2) * N + R * Fft2<N>::EX + (R / 2) * pzlen(2 * N));
 }
 template <int NY, int NZ> constexpr size_t plane_fast_smem() {
     return sizeof(float2) * (2 * NY + 6 * NZ * Fft2<NY>::EX + 3 * NZ * pzlen(2 * NY));

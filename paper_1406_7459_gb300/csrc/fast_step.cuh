@@ -144,7 +144,8 @@ __device__ __forceinline__ void zdirect_task(const float2 (&m)[3][NZ], Coef coef
 // transforms, the z sum (which reads all lines of a column) and the inverse
 // transforms.  Returns false, uniformly over the block, when a copy wait gave
 // up (or ok_in is false); nothing is written to Sh then.
-template <int NY, int NZ, int T>
+// RAG: a ragged sample, lines of g.Jst <= NY values (zero past them).
+template <int NY, int NZ, int T, bool RAG = false>
 __device__ __forceinline__ bool plane_body(const Geom& g, int kx, bool ok_in, const float2* tw, const float2* ta,
                                            const float* Ks, float2* zb, uint32_t b_s, uint32_t par, uint32_t b_k,
                                            float2* __restrict__ Sh) {
@@ -172,7 +173,12 @@ __device__ __forceinline__ bool plane_body(const Geom& g, int kx, bool ok_in, co
     if (ok && act && t < Q) {
         const float2* src = zb + lf * ZS;                 // both halves' groups read the line
 #pragma unroll
-        for (int q = 0; q < P; ++q) v[q] = src[t + Q * q];
+        for (int q = 0; q < P; ++q) {
+            if constexpr (RAG)
+                v[q] = t + Q * q < g.Jst ? src[t + Q * q] : make_float2(0.f, 0.f);
+            else
+                v[q] = src[t + Q * q];
+        }
     }
     if (__syncthreads_or(!ok)) return false;
     // forward y (pruned input): odd half pre-multiplied by W_LY^j; the
@@ -257,7 +263,8 @@ __device__ __forceinline__ bool plane_body(const Geom& g, int kx, bool ok_in, co
         for (int q = 0; q < Q; ++q) {
             const float ox = __shfl_down_sync(0xffffffffu, w[q].x, 16);
             const float oy = __shfl_down_sync(0xffffffffu, w[q].y, 16);
-            if (act && h == 0) outp[(size_t)line * g.Jst + t + P * q] = make_float2(w[q].x + ox, w[q].y + oy);
+            if (act && h == 0 && t < P && (!RAG || t + P * q < g.Jst))
+                outp[(size_t)line * g.Jst + t + P * q] = make_float2(w[q].x + ox, w[q].y + oy);
         }
     } else {
         // halves in different warps: through the shared lines
@@ -270,14 +277,14 @@ __device__ __forceinline__ bool plane_body(const Geom& g, int kx, bool ok_in, co
 #pragma unroll
         for (int idx = threadIdx.x; idx < NL * NY; idx += T) {
             const int l = idx / NY, n = idx % NY;
-            outp[(size_t)l * g.Jst + n] = cadd(zb[l * ZS + n], zb[l * ZS + HALF + n]);
+            if (!RAG || n < g.Jst) outp[(size_t)l * g.Jst + n] = cadd(zb[l * ZS + n], zb[l * ZS + HALF + n]);
         }
     }
     return true;
 }
 
 // K_A as a kernel: one kx plane per CTA.
-template <int NY, int NZ>
+template <int NY, int NZ, bool RAG = false>
 __global__ void __launch_bounds__(PlaneLayout<NY, NZ>::THREADS, (PlaneLayout<NY, NZ>::THREADS <= 512) ? 2 : 1)
     k_plane_pdl(const __grid_constant__ Geom g, const float* __restrict__ Kd, const float2* __restrict__ S,
                 float2* __restrict__ Sh, int* __restrict__ flag, int early_trigger) {
@@ -316,15 +323,16 @@ __global__ void __launch_bounds__(PlaneLayout<NY, NZ>::THREADS, (PlaneLayout<NY,
     if (threadIdx.x == 0) {
         proxy_fence_global();                             // S came from ordinary stores
         const float2* plane = S + (size_t)kx * NL * g.Jst;
-        mbar_expect_tx(b_s, NL * NY * sizeof(float2));
+        const uint32_t ln = (uint32_t)((RAG ? g.Jst : NY) * sizeof(float2));   // Jst: a multiple of 4
+        mbar_expect_tx(b_s, NL * ln);
 #pragma unroll 1
-        for (int l = 0; l < NL; ++l) bulk_g2s(smem_addr(zb + l * ZS), plane + (size_t)l * g.Jst, NY * sizeof(float2), b_s);
+        for (int l = 0; l < NL; ++l) bulk_g2s(smem_addr(zb + l * ZS), plane + (size_t)l * g.Jst, ln, b_s);
         mbar_expect_tx(b_k, Lay::KT_FLOATS * sizeof(float));
         bulk_g2s(smem_addr(Ks), Kd + (size_t)kx * Lay::KT_FLOATS, Lay::KT_FLOATS * sizeof(float), b_k);
     }
     const bool ok = mbar_wait(b_tw, 0);
     if (ok) fill_ta<NY, Q, T>(ta, tw);
-    if (!plane_body<NY, NZ, T>(g, kx, ok, tw, ta, Ks, zb, b_s, 0, b_k, Sh)) {
+    if (!plane_body<NY, NZ, T, RAG>(g, kx, ok, tw, ta, Ks, zb, b_s, 0, b_k, Sh)) {
         // a wait gave up: every thread leaves together, once the copies in
         // flight have landed (bounded again)
         if (threadIdx.x == 0) {
@@ -379,6 +387,12 @@ struct XTma {
     uint32_t bar = 0;
 };
 
+// A thread's cells of a ragged x-step tile (its trips of the field loop):
+// M and the exchange field of Eq. (4), formed before the spectrum arrives.
+template <int CPT> struct RagCells {
+    float m[CPT][3], ex[CPT][3];
+};
+
 // MODE kModeStep: the Euler step (M^{n+1} replaces M^n in Mt and goes to
 // Mout when Mout is given; Snext = its x spectrum); kModeHeff: Mout = H_eff
 // of M (Sh from the spectrum with the exchange stencil folded in);
@@ -391,26 +405,36 @@ struct XTma {
 // (floats [c][row][i]) are in shared memory or on their way there as
 // 16-byte asynchronous copies of this thread (the gather below waits for
 // all of them).  sb stages the tile's rows of Sh, wk the transforms.
-template <int N, int R, int MODE, int T>
+//
+// RAG: a ragged sample of g.nx <= N cells per row and g.Jst (a multiple of
+// R) rows of spectrum of which g.ny are the sample's; Mt is zero past both
+// and M^n itself comes in rc (load_rag_cells).
+// The exchange stays the stencil of Eq. (4), as on the general path (the
+// spectrum is the plain one): on samples of any shape its rounding is that
+// of neighbouring differences, where the folded form's is that of the
+// transforms.
+template <int N, int R, int MODE, int T, bool RAG = false>
 __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int tile, const float2* tw,
                                            const float2* ta, float* Mt, float2* sb, float2* wk,
                                            const float2* __restrict__ Sh, float2* __restrict__ Snext,
                                            float* __restrict__ Mout, int* __restrict__ flag,
-                                           float* __restrict__ Mcopy = nullptr, const XTma& xt = XTma{}) {
+                                           float* __restrict__ Mcopy = nullptr, const XTma& xt = XTma{},
+                                           const RagCells<(R * N + T - 1) / T>* rc = nullptr) {
     using Lay = XstepLayout<N, R>;
     using F = Fft2<N>;
     constexpr int P = F::P, Q = F::Q, G = F::G, L = Lay::L, H = Lay::H, NL = Lay::NL, ZS = Lay::ZS;
     constexpr int HM = Lay::HM, HP = Lay::HP, HOFF = Lay::HOFF;
     constexpr int RP = R / 2;                             // row pairs of the tile
     static_assert(T >= 2 * NL * G, "block smaller than the tile's transform groups");
-    const int ntj = g.ny / R;
+    const int ntj = (RAG ? g.Jst : g.ny) / R;
+    const int nx = RAG ? g.nx : N;
     const int jt = tile % ntj;
     const int k = tile / ntj;
     const int j0 = jt * R;
     // 32-bit offsets: the plan admits this kernel only when 3 (nx + 1) nz ny
     // complex values and 3 nx ny nz floats index below 2^31
     const int Nc = g.N;
-    const int plane_xy = N * g.ny;
+    const int plane_xy = nx * g.ny;
     const int s_c = g.nz * g.Jst, s_kx = 3 * s_c;            // spectrum strides of c and kx
     const int s_base = k * g.Jst + j0;
 
@@ -489,7 +513,7 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
         for (int q = 0; q < Q; ++q) {
             const float ox = __shfl_down_sync(0xffffffffu, w[q].x, 16);
             const float oy = __shfl_down_sync(0xffffffffu, w[q].y, 16);
-            if (fft_thread && h == 0) wk[line * L + t + P * q] = make_float2(w[q].x + ox, w[q].y + oy);
+            if (fft_thread && h == 0 && t < P) wk[line * L + t + P * q] = make_float2(w[q].x + ox, w[q].y + oy);
         }
     } else {
         if (fft_thread && t < P) {
@@ -510,30 +534,41 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
     // (zero change), so each missing neighbour adds pexch M(i) / delta^2.
     const float bz = cf.pexch * (float)((g.nz > 1) * ((k == 0) + (k == g.nz - 1))) * cf.idz2;
 #pragma unroll
-    for (int idx = threadIdx.x; idx < R * N; idx += T) {
+    for (int u = 0; u < (R * N + T - 1) / T; ++u) {
+        const int idx = u * T + threadIdx.x;
+        if (R * N % T != 0 && idx >= R * N) break;
         const int r = idx / N;
         const int i = idx % N;
         const int j = j0 + r;
+        if (RAG && (i >= nx || j >= g.ny)) continue;            // Mt stays zero there
         float hd[3];
 #pragma unroll
         for (int cc = 0; cc < 3; ++cc) {
             const float2 z = wk[(cc * RP + (r >> 1)) * L + i];   // pair line of rows (r & ~1, r | 1)
             hd[cc] = (r & 1) ? z.y : z.x;
         }
-        const int cell = i + N * (j0 + r) + plane_xy * k;
+        const int cell = i + nx * (j0 + r) + plane_xy * k;
         if constexpr (MODE == kModeDemag) {
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc) Mout[cc * Nc + cell] = hd[cc];
             continue;
         }
-        const float bnd = bz + cf.pexch * ((float)((i == 0) + (i == N - 1)) * cf.idx2 +
-                                           (float)((g.ny > 1) * ((j == 0) + (j == g.ny - 1))) * cf.idy2);
         float m[3], hh[3];
+        if constexpr (RAG) {
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc) {
-            const float m0 = Mt[(cc * R + r) * N + i];
-            m[cc] = m0;
-            hh[cc] = hd[cc] + bnd * m0;
+            for (int cc = 0; cc < 3; ++cc) {
+                m[cc] = rc->m[u][cc];
+                hh[cc] = hd[cc] + rc->ex[u][cc];
+            }
+        } else {
+            const float bnd = bz + cf.pexch * ((float)((i == 0) + (i == N - 1)) * cf.idx2 +
+                                               (float)((g.ny > 1) * ((j == 0) + (j == g.ny - 1))) * cf.idy2);
+#pragma unroll
+            for (int cc = 0; cc < 3; ++cc) {
+                const float m0 = Mt[(cc * R + r) * N + i];
+                m[cc] = m0;
+                hh[cc] = hd[cc] + bnd * m0;
+            }
         }
         hh[0] += cf.hx;
         hh[1] += cf.panis * m[1] + cf.hy;
@@ -552,7 +587,8 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
         const float n0 = m[0] + cf.dt * (cf.c1 * p0 + cf.c2 * q0);
         const float n1 = m[1] + cf.dt * (cf.c1 * p1 + cf.c2 * q1);
         const float n2 = m[2] + cf.dt * (cf.c1 * p2 + cf.c2 * q2);
-        const float s = cf.Ms * rsqrtf(n0 * n0 + n1 * n1 + n2 * n2);
+        const float s = RAG ? cf.Ms / sqrtf(n0 * n0 + n1 * n1 + n2 * n2)
+                            : cf.Ms * rsqrtf(n0 * n0 + n1 * n1 + n2 * n2);
         const float o0 = n0 * s, o1 = n1 * s, o2 = n2 * s;
         if (!isfinite(o0 + o1 + o2)) atomicOr(flag, kFlagNonFinite);   // |o| <= Ms when finite
         if (Mout) {
@@ -601,7 +637,7 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
             const int p2 = idx % RP, ck = idx / RP;
             const int c = ck / H, kx = ck - c * H;
             const float2* ln = wk + (c * RP + p2) * ZS;
-            const int km = (L - kx) & (L - 1);
+            const int km = kx == 0 ? 0 : L - kx;
             const float2 zk = ln[(kx & 1) * HOFF + (kx >> 1)];
             const float2 zm = ln[(km & 1) * HOFF + (km >> 1)];
             const float4 o = make_float4(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y),
@@ -623,6 +659,44 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
     }
 }
 
+// Ragged tiles: this thread's cells of M with their exchange field, by the
+// stencil with free boundaries (a missing neighbour is the cell itself), in
+// registers; the tile's cells past nx and ny are zeroed in Mt (the update
+// writes the others).  Run before the wait for the plane kernel, which does
+// not write M, so the 7-point loads overlap it.
+template <int N, int R, int T>
+__device__ __forceinline__ void load_rag_cells(const Geom& g, const LlgCoef& cf, int tile, const float* __restrict__ M,
+                                               float* Mt, RagCells<(R * N + T - 1) / T>& rc) {
+    const int ntj = g.Jst / R;
+    const int k = tile / ntj, j0 = (tile % ntj) * R;
+    const int nx = g.nx, Nc = g.N, plane_xy = nx * g.ny;
+#pragma unroll
+    for (int u = 0; u < (R * N + T - 1) / T; ++u) {
+        const int idx = u * T + threadIdx.x;
+        if (R * N % T != 0 && idx >= R * N) break;
+        const int r = idx / N, i = idx % N, j = j0 + r;
+        if (i >= nx || j >= g.ny) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) Mt[(c * R + r) * N + i] = 0.f;
+            continue;
+        }
+        const int cell = i + nx * j + plane_xy * k;
+        const int xm = i > 0 ? cell - 1 : cell, xp = i + 1 < nx ? cell + 1 : cell;
+        const int ym = j > 0 ? cell - nx : cell, yp = j + 1 < g.ny ? cell + nx : cell;
+        const int zm = k > 0 ? cell - plane_xy : cell, zp = k + 1 < g.nz ? cell + plane_xy : cell;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float* Mc = M + (size_t)c * Nc;
+            const float m0 = __ldg(Mc + cell);
+            float lap = (__ldg(Mc + xp) - 2.f * m0 + __ldg(Mc + xm)) * cf.idx2 +
+                        (__ldg(Mc + yp) - 2.f * m0 + __ldg(Mc + ym)) * cf.idy2;
+            if (g.nz > 1) lap += (__ldg(Mc + zp) - 2.f * m0 + __ldg(Mc + zm)) * cf.idz2;
+            rc.m[u][c] = m0;
+            rc.ex[u][c] = cf.pexch * lap;
+        }
+    }
+}
+
 // Fill the tile's M^n rows (floats [c][row][i]) with 16-byte asynchronous
 // copies (committed with the caller's next group).
 template <int N, int R, int T>
@@ -640,7 +714,7 @@ __device__ __forceinline__ void load_mtile(const Geom& g, int tile, const float*
 }
 
 // K_B as a kernel: one (layer, R rows) tile per CTA.
-template <int N, int R, int MODE>
+template <int N, int R, int MODE, bool RAG = false>
 __global__ void __launch_bounds__(XstepLayout<N, R>::THREADS)
     k_xstep_pdl(const __grid_constant__ Geom g, const __grid_constant__ LlgCoef cf, const float2* __restrict__ Sh,
                 float2* __restrict__ Snext, const float* __restrict__ M, float* __restrict__ Mout,
@@ -663,6 +737,17 @@ __global__ void __launch_bounds__(XstepLayout<N, R>::THREADS)
 #pragma unroll
     for (int i = threadIdx.x; i < L / 2; i += T) copy16(tw + 2 * i, g.twx + 2 * i);
     F::template load_ta<T>(ta, g.twx);
+    if constexpr (RAG) {
+        __pipeline_commit();
+        RagCells<(R * N + T - 1) / T> rc;
+        if constexpr (MODE != kModeDemag) load_rag_cells<N, R, T>(g, cf, blockIdx.x, M, Mt, rc);
+        pdl_wait();
+        xstep_body<N, R, MODE, T, true>(g, cf, blockIdx.x, tw, ta, Mt, sb, wk, Sh, Snext, Mout, flag, Mcopy, XTma{},
+                                        &rc);
+        __syncthreads();
+        pdl_trigger();
+        return;
+    }
     if constexpr (MODE != kModeDemag) load_mtile<N, R, T>(g, blockIdx.x, M, Mt);
     __pipeline_commit();
     pdl_wait();

@@ -65,6 +65,30 @@ static bool make_axis_plan(int L, AxisPlan* p) {
     return n == 1 && p->nst <= kMaxStages;
 }
 
+// Ragged films: the two-kernel step on carrier lengths (ragged.cuh), its
+// geometry in c->gf.  False, with c unchanged but for c->fs and c->gf, where
+// no kernels exist for the size.
+static bool plan_ragged(mm_ctx* c) {
+    const Geom& g = c->g;
+    Geom& f = c->gf;
+    FastStepFns fs;
+    int NX = 0, NY = 0;
+    const int jst = (g.ny + 3) & ~3;          // whole tiles of four rows; 16-byte lines for the bulk copies
+    if (!ragged_lookup(g.nx, g.ny, g.nz, &fs, &NX, &NY)) return false;
+    f = g;
+    f.Lx = 2 * NX;
+    f.Ly = 2 * NY;
+    f.Lz = 1;                                 // the z sum is direct
+    f.Hx = NX + 1;
+    f.Hy = NY + 1;
+    f.Hz = 1;
+    f.Jst = jst;
+    // the x-step kernel indexes the spectrum and M with 32-bit offsets
+    if (!(3.0 * f.Hx * f.nz * f.Jst < (double)INT_MAX && 3.0 * f.N < (double)INT_MAX)) return false;
+    c->fs = fs;
+    return true;
+}
+
 static int build_plan(mm_ctx* c) {
     Geom& g = c->g;
     Launch& l = c->l;
@@ -165,6 +189,12 @@ static int build_plan(mm_ctx* c) {
                     3.0 * g.Hx * g.nz * g.Jst < (double)INT_MAX && 3.0 * g.N < (double)INT_MAX;
         if (c->has_ss) s.ka = nullptr;
         c->has_persist = ok && persist_lookup(g.nx, g.ny, g.nz, s.rb, &c->pf);
+    }
+    c->gf = g;
+    c->rag = allow_fast && !c->has_fs && !c->has_ss && plan_ragged(c);
+    if (c->rag) {
+        c->has_fs = true;
+        c->has_persist = false;
     }
     if (!c->has_fs && !c->has_ss && !l.fx) {
         c->has_gx = true;
@@ -278,18 +308,20 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
         CU(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking));
         Geom& g = c->g;
         const size_t N = (size_t)g.N;
-        CU(cudaMalloc(&c->Kt, sizeof(float) * 6 * (size_t)g.Hx * g.Hy * g.Hz));
+        Geom& gf = c->gf;
+        if (!c->rag) CU(cudaMalloc(&c->Kt, sizeof(float) * 6 * (size_t)g.Hx * g.Hy * g.Hz));
         // the two-kernel step's spectra carry one pad kx plane (the tiled
         // copies of the x-step touch it; nothing reads it)
-        const size_t plane = (size_t)3 * g.nz * g.Jst;
-        const size_t nS = (size_t)(g.Hx + (c->has_fs ? 1 : 0)) * plane;
+        const size_t plane = (size_t)3 * gf.nz * gf.Jst;
+        const size_t nS = (size_t)(gf.Hx + (c->has_fs ? 1 : 0)) * plane;
         CU(cudaMalloc(&c->S, sizeof(float2) * nS));
         if (c->has_fs) {
             CU(cudaMalloc(&c->Sh, sizeof(float2) * nS));
-            CU(cudaMemset(c->S + (size_t)g.Hx * plane, 0, sizeof(float2) * plane));
-            CU(cudaMemset(c->Sh + (size_t)g.Hx * plane, 0, sizeof(float2) * plane));
-            CU(cudaMalloc(&c->Kd, sizeof(float) * 6 * (size_t)g.Hx * kd_row(g.Hy) * g.nz));
-            CU(cudaMalloc(&c->Kd0, sizeof(float) * 6 * (size_t)g.Hx * kd_row(g.Hy) * g.nz));
+            CU(cudaMemset(c->S + (size_t)gf.Hx * plane, 0, sizeof(float2) * plane));
+            CU(cudaMemset(c->Sh + (size_t)gf.Hx * plane, 0, sizeof(float2) * plane));
+            // ragged films keep the exchange stencil: no folded spectrum
+            if (!c->rag) CU(cudaMalloc(&c->Kd, sizeof(float) * 6 * (size_t)gf.Hx * kd_row(gf.Hy) * gf.nz));
+            CU(cudaMalloc(&c->Kd0, sizeof(float) * 6 * (size_t)gf.Hx * kd_row(gf.Hy) * gf.nz));
         }
         if (c->has_ss) CU(cudaMalloc(&c->Kt_ex, sizeof(float) * 6 * (size_t)g.Hx * g.Hy * g.Hz));
         CU(cudaMalloc(&c->Mbuf[0], sizeof(float) * 3 * N));
@@ -298,31 +330,33 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
         CU(cudaMalloc(&c->flag, sizeof(int)));
         CU(cudaMalloc(&c->partials, sizeof(double) * energy_partials_elems(g.N)));
         CU(cudaMalloc(&c->Edev, sizeof(double) * 5));
-        CU(cudaMalloc(&c->tw, sizeof(float2) * (size_t)(g.Lx + g.Ly + g.Lz)));
+        const size_t ntw = (size_t)gf.Lx + gf.Ly + gf.Lz;
+        CU(cudaMalloc(&c->tw, sizeof(float2) * ntw));
         {
-            float2* h = (float2*)malloc(sizeof(float2) * (size_t)(g.Lx + g.Ly + g.Lz));
+            float2* h = (float2*)malloc(sizeof(float2) * ntw);
             if (!h) return fail(MM_ENOMEM, "host allocation failed");
-            host_twiddles(g.Lx, h);
-            host_twiddles(g.Ly, h + g.Lx);
-            host_twiddles(g.Lz, h + g.Lx + g.Ly);
-            cudaError_t e = cudaMemcpy(c->tw, h, sizeof(float2) * (size_t)(g.Lx + g.Ly + g.Lz),
-                                       cudaMemcpyHostToDevice);
+            host_twiddles(gf.Lx, h);
+            host_twiddles(gf.Ly, h + gf.Lx);
+            host_twiddles(gf.Lz, h + gf.Lx + gf.Ly);
+            cudaError_t e = cudaMemcpy(c->tw, h, sizeof(float2) * ntw, cudaMemcpyHostToDevice);
             free(h);
             CU(e);
         }
-        g.twx = c->tw;
-        g.twy = c->tw + g.Lx;
-        g.twz = c->tw + g.Lx + g.Ly;
-        g.Kt = c->Kt;
-        g.Kd = c->Kd;
-        g.Kd0 = c->Kd0;
-        CU(configure_pass_kernels(g, c->l));
+        for (Geom* q : {&g, &gf}) {           // a ragged film's own lengths have no kernels: only gf's are read
+            q->twx = c->tw;
+            q->twy = c->tw + gf.Lx;
+            q->twz = c->tw + gf.Lx + gf.Ly;
+            q->Kt = c->Kt;
+            q->Kd = c->rag ? c->Kd0 : c->Kd;
+            q->Kd0 = c->Kd0;
+        }
+        if (!c->rag) CU(configure_pass_kernels(g, c->l));
         if (c->has_fs || c->has_ss) CU(configure_step_kernels(c->fs));
         if (c->has_fs) {
             int sms = 0;
             CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
-            c->fs.early = fast_step_early_trigger(g, sms);
-            encode_xstep_maps(g, &c->fs, c->Sh, c->S);   // per-thread copies where no map applies
+            c->fs.early = c->rag ? ragged_early_trigger(gf, c->fs, sms) : fast_step_early_trigger(gf, sms);
+            if (!c->rag) encode_xstep_maps(g, &c->fs, c->Sh, c->S);   // per-thread copies where no map applies
         }
         if (c->has_persist) {
             bool usable = false;
@@ -332,7 +366,7 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
         }
 
         // tensor set-up in FP64
-        const int L[3] = {g.Lx, g.Ly, g.Lz};
+        const int L[3] = {gf.Lx, gf.Ly, gf.Lz};
         double *Nd = nullptr, *w1 = nullptr, *w2 = nullptr;
         const size_t wn = tensor_work_elems(c->grid, L);
         cudaError_t e = cudaMalloc(&Nd, sizeof(double) * 6 * N);
@@ -349,7 +383,10 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
         exf.idx2 = 1.0 / (c->cell[0] * c->cell[0]);
         exf.idy2 = 1.0 / (c->cell[1] * c->cell[1]);
         exf.idz2 = 1.0 / (c->cell[2] * c->cell[2]);
-        if (e == cudaSuccess) e = tensor_spectrum(c->grid, L, Nd, c->Kt, w1, w2, c->stream, c->Kd, exf, c->Kd0);
+        if (e == cudaSuccess && c->rag)
+            e = tensor_spectrum(c->grid, L, Nd, nullptr, w1, w2, c->stream, c->Kd0);
+        else if (e == cudaSuccess)
+            e = tensor_spectrum(c->grid, L, Nd, c->Kt, w1, w2, c->stream, c->Kd, exf, c->Kd0);
         if (e == cudaSuccess && c->has_ss) {
             ExchangeFold ex3 = exf;
             ex3.on = 1;
@@ -444,19 +481,26 @@ extern "C" int mm_get_m(mm_ctx* c, float* M) {
     return MM_OK;
 }
 
+// x R2C of M into the spectrum workspace S; Mcopy (has_fs, may be null): also
+// copy M there.
+static cudaError_t form_spectrum(mm_ctx* c, const float* M, cudaStream_t s, float* Mcopy = nullptr) {
+    if (c->rag) return launch_ragged_pass1(c->gf, c->fs, M, c->S, s, Mcopy);
+    return launch_pass1(c->g, c->l, M, c->S, s, Mcopy);
+}
+
 // The three-pass evaluation on the spectrum workspace S (which also holds
 // the two-kernel step's spectrum, so it invalidates a pending one).
 int mmk::run_passes(mm_ctx* c, int mode, const float* M, float* out, double dt, cudaStream_t s) {
     const LlgCoef cf = make_coef(c, dt);
     c->spec_valid = false;
-    CU(launch_pass1(c->g, c->l, M, c->S, s));
-    if (c->has_fs && c->fs.ta <= 512 && (mode == kModeDemag || mode == kModeHeff)) {
+    CU(form_spectrum(c, M, s));
+    if (c->has_fs && (c->rag || c->fs.ta <= 512) && (mode == kModeDemag || mode == kModeHeff)) {
         // power-of-two films: the step's plane kernel and the field-only
         // variant of its x-step kernel (where the plane kernel runs at most
         // 512 threads: larger ones are register-starved, and the three-pass
         // plane kernel serves them better)
-        CU(launch_field_pdl(c->g, c->fs, cf, mode, mode == kModeDemag ? c->Kd0 : c->Kd, c->S, c->Sh, M, out, c->flag,
-                            s));
+        CU(launch_field_pdl(c->gf, c->fs, cf, mode, mode == kModeDemag ? c->gf.Kd0 : c->gf.Kd, c->S, c->Sh, M, out,
+                            c->flag, s));
         return MM_OK;
     }
     if (c->has_ss && (mode == kModeDemag || mode == kModeHeff)) {
@@ -510,7 +554,7 @@ static int enqueue_rk_step(mm_ctx* c, int p, double dt, cudaStream_t s) {
 static int enqueue_step(mm_ctx* c, int p, double dt, cudaStream_t s) {
     if (c->method != MM_INTEGRATOR_EULER) return enqueue_rk_step(c, p, dt, s);
     if (c->has_fs) {
-        CU(launch_step_pdl(c->g, c->fs, make_coef(c, dt), c->S, c->Sh, c->Mbuf[p], c->Mbuf[1 - p],
+        CU(launch_step_pdl(c->gf, c->fs, make_coef(c, dt), c->S, c->Sh, c->Mbuf[p], c->Mbuf[1 - p],
                            c->flag, s, true));
         return MM_OK;
     }
@@ -564,7 +608,7 @@ static int capture_step(mm_ctx* c, int kind, int p, double dt) {
 // Form S[cur] from M[cur] when the two-kernel step needs it.
 static int ensure_spectrum(mm_ctx* c) {
     if (!(c->has_fs || c->has_ss || c->has_gx) || c->spec_valid || c->method != MM_INTEGRATOR_EULER) return MM_OK;
-    CU(launch_pass1(c->g, c->l, c->Mbuf[c->cur], c->S, c->stream));
+    CU(form_spectrum(c, c->Mbuf[c->cur], c->stream));
     c->spec_valid = true;
     return MM_OK;
 }
@@ -632,7 +676,7 @@ extern "C" int mm_step(mm_ctx* c, int n, double dt) {
         for (int s = 0; s < n;) {
             const int m = std::min(n - s, kPersistChunk);
             const int p = c->cur, q = (p + m) & 1;
-            CU(launch_persist(c->g, c->pf, cf, c->Kd, c->S, c->Sh, c->Mbuf[p], c->Mbuf[q], m, c->flag, c->gbar,
+            CU(launch_persist(c->gf, c->pf, cf, c->Kd, c->S, c->Sh, c->Mbuf[p], c->Mbuf[q], m, c->flag, c->gbar,
                               c->wait_limit, c->stream));
             c->cur = q;
             s += m;
@@ -725,13 +769,13 @@ extern "C" int mm_step_host(mm_ctx* c, const float* M_in, int n, double dt, floa
     // leaves a device copy for the updates; the last step's update writes
     // the new state to the context and to the caller's buffer
     float* cp = in == c->Mbuf[c->cur] ? nullptr : c->Mbuf[c->cur];
-    CU(launch_pass1(c->g, c->l, in, c->S, c->stream, cp));
+    CU(form_spectrum(c, in, c->stream, cp));
     const LlgCoef cf = make_coef(c, dt);
     int p = c->cur;
     for (int s = 0; s < n; ++s) {
         const float* Mn = c->Mbuf[p];
         float* copy = (s == n - 1) ? out : nullptr;
-        CU(launch_step_pdl(c->g, c->fs, cf, c->S, c->Sh, Mn, c->Mbuf[1 - p], c->flag, c->stream, true, copy));
+        CU(launch_step_pdl(c->gf, c->fs, cf, c->S, c->Sh, Mn, c->Mbuf[1 - p], c->flag, c->stream, true, copy));
         p = 1 - p;
     }
     c->cur = p;
@@ -796,9 +840,36 @@ extern "C" int mm_tensor_octant(mm_ctx* c, double* out) {
     return MM_OK;
 }
 
+// The tensor spectrum on the padded lengths of c->g, for the contexts whose
+// steps do not read it (ragged films); kept afterwards.
+static int form_kt(mm_ctx* c) {
+    const int L[3] = {c->g.Lx, c->g.Ly, c->g.Lz};
+    const size_t wn = tensor_work_elems(c->grid, L);
+    double *Nd = nullptr, *w1 = nullptr, *w2 = nullptr;
+    float* Kt = nullptr;
+    cudaError_t e = cudaMalloc(&Kt, sizeof(float) * 6 * (size_t)c->g.Hx * c->g.Hy * c->g.Hz);
+    if (e == cudaSuccess) e = cudaMalloc(&Nd, sizeof(double) * 6 * (size_t)c->g.N);
+    if (e == cudaSuccess) e = cudaMalloc(&w1, sizeof(double) * wn);
+    if (e == cudaSuccess) e = cudaMalloc(&w2, sizeof(double) * wn);
+    if (e == cudaSuccess) e = tensor_octant_fp64(c->grid, c->cell, Nd, c->stream);
+    if (e == cudaSuccess) e = tensor_spectrum(c->grid, L, Nd, Kt, w1, w2, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    cudaFree(Nd);
+    cudaFree(w1);
+    cudaFree(w2);
+    if (e != cudaSuccess) cudaFree(Kt);
+    CU(e);
+    c->Kt = Kt;
+    return MM_OK;
+}
+
 extern "C" int mm_kernel_spectrum(mm_ctx* c, float* out) {
     if (!c || !out) return fail(MM_EINVAL, "null argument");
     const size_t n = (size_t)6 * c->g.Hx * c->g.Hy * c->g.Hz;
+    if (!c->Kt) {
+        int rc = form_kt(c);
+        if (rc != MM_OK) return rc;
+    }
     CU(cudaMemcpyAsync(out, c->Kt, sizeof(float) * n, cudaMemcpyDefault, c->stream));
     CU(cudaStreamSynchronize(c->stream));
     return MM_OK;
@@ -820,16 +891,16 @@ extern "C" int mm_time_passes(mm_ctx* c, int reps, double dt, void* flush, unsig
             CU(cudaEventRecord(ev[0], c->stream));
             if (c->has_fs) {
                 // pass 1 alone (the two-kernel step folds it into K_B), then K_A, K_B
-                CU(launch_pass1(c->g, c->l, c->Mbuf[p], c->S, c->stream));
+                CU(form_spectrum(c, c->Mbuf[p], c->stream));
                 CU(cudaEventRecord(ev[1], c->stream));
-                CU(launch_step_a(c->g, c->fs, c->Kd, c->S, c->Sh, c->flag, c->stream, false, 0));
+                CU(launch_step_a(c->gf, c->fs, c->gf.Kd, c->S, c->Sh, c->flag, c->stream, false, 0));
                 CU(cudaEventRecord(ev[2], c->stream));
-                CU(launch_step_b(c->g, c->fs, cf, c->Sh, c->S, c->Mbuf[p], c->Mbuf[1 - p], c->flag,
+                CU(launch_step_b(c->gf, c->fs, cf, c->Sh, c->S, c->Mbuf[p], c->Mbuf[1 - p], c->flag,
                                  c->stream, false));
                 c->spec_valid = true;
             } else {
                 c->spec_valid = false;            // S no longer holds a step's x spectrum
-                CU(launch_pass1(c->g, c->l, c->Mbuf[p], c->S, c->stream));
+                CU(form_spectrum(c, c->Mbuf[p], c->stream));
                 CU(cudaEventRecord(ev[1], c->stream));
                 CU(launch_plane(c->g, c->l, c->S, c->stream));
                 CU(cudaEventRecord(ev[2], c->stream));

@@ -167,6 +167,10 @@ struct FastStepFns {
                    CUtensorMap, int) = {nullptr, nullptr, nullptr};
     int rb = 0, tb = 0;
     size_t sb = 0;
+    // ragged films: their row transform (the exact sizes use FastFns::p1)
+    void (*p1)(Geom, const float*, float2*, float*) = nullptr;
+    int r1 = 0, t1 = 0;
+    size_t s1 = 0;
     bool tma = false;
     int tma_use = 0;                           // bit 0: tiled gather, bit 1: tiled scatter (opt-in:
                                                // measured slower than the per-thread copies)
@@ -183,6 +187,12 @@ bool encode_xstep_maps(const Geom& g, FastStepFns* f, const float2* Sh, const fl
 bool fast_step_lookup_x(int nx, FastStepFns* f);
 bool fast_step_lookup_plane_a(int ny, int nz, FastStepFns* f);
 bool fast_step_lookup_plane_b(int ny, int nz, FastStepFns* f);
+// Ragged films (ragged.cuh): the kernels and the carrier lengths NX >= nx,
+// NY >= ny; whether the plane kernel triggers the x-step early.
+bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY);
+int ragged_early_trigger(const Geom& g, const FastStepFns& f, int sms);
+cudaError_t launch_ragged_pass1(const Geom& g, const FastStepFns& f, const float* M, float2* S, cudaStream_t s,
+                                float* Mcopy = nullptr);
 // K_A reads the x half-spectrum S and writes its output to Sh; K_B reads Sh
 // and writes the next step's S.
 cudaError_t launch_step_pdl(const Geom& g, const FastStepFns& f, const LlgCoef& c, float2* S, float2* Sh,
@@ -277,6 +287,7 @@ struct ExchangeFold {
     int nx, ny, Lx, Ly;
     double pexch, idx2, idy2, idz2;
 };
+// (Kt_dev null: only the 2-D spectra)
 cudaError_t tensor_spectrum(const int grid[3], const int L[3], const double* N_dev, float* Kt_dev,
                             double* work1, double* work2, cudaStream_t s, float* Kd_dev = nullptr,
                             ExchangeFold ex = ExchangeFold{}, float* Kd0_dev = nullptr);

@@ -1,0 +1,10 @@
+// ragged_plane_nz2.cu -- the plane kernel of ragged films of 2 layers.
+#include "ragged.cuh"
+
+namespace mmk {
+
+bool ragged_lookup_plane_nz2(int NY, FastStepFns* f) {
+    return rag_lookup_plane_lo<2>(NY, f) || rag_lookup_plane_hi<2>(NY, f);
+}
+
+}  // namespace mmk

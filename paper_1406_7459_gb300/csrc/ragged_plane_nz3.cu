@@ -1,0 +1,10 @@
+// ragged_plane_nz3.cu -- the plane kernel of ragged films of 3 layers.
+#include "ragged.cuh"
+
+namespace mmk {
+
+bool ragged_lookup_plane_nz3(int NY, FastStepFns* f) {
+    return rag_lookup_plane_lo<3>(NY, f) || rag_lookup_plane_hi<3>(NY, f);
+}
+
+}  // namespace mmk

@@ -1,0 +1,58 @@
+// ragged_select.cu -- picks the kernels and carrier lengths of a ragged film
+// (ragged.cuh) and launches its row transform.
+#include "ragged.cuh"
+
+namespace mmk {
+
+bool ragged_lookup_x_a(int N, FastStepFns* f);
+bool ragged_lookup_x_b(int N, FastStepFns* f);
+bool ragged_lookup_x_c(int N, FastStepFns* f);
+bool ragged_lookup_x_d(int N, FastStepFns* f);
+bool ragged_lookup_plane_nz1(int NY, FastStepFns* f);
+bool ragged_lookup_plane_nz2(int NY, FastStepFns* f);
+bool ragged_lookup_plane_nz3(int NY, FastStepFns* f);
+bool ragged_lookup_plane_nz4(int NY, FastStepFns* f);
+bool ragged_lookup_plane_nz5(int NY, FastStepFns* f);
+bool ragged_lookup_plane_nz6(int NY, FastStepFns* f);
+bool ragged_lookup_plane_nz7(int NY, FastStepFns* f);
+bool ragged_lookup_plane_nz8(int NY, FastStepFns* f);
+
+bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY) {
+    *NX = ragged_len(nx);
+    *NY = ragged_len(ny);
+    if (!*NX || !*NY) return false;
+    bool ok = false;
+    switch (nz) {
+        case 1: ok = ragged_lookup_plane_nz1(*NY, f); break;
+        case 2: ok = ragged_lookup_plane_nz2(*NY, f); break;
+        case 3: ok = ragged_lookup_plane_nz3(*NY, f); break;
+        case 4: ok = ragged_lookup_plane_nz4(*NY, f); break;
+        case 5: ok = ragged_lookup_plane_nz5(*NY, f); break;
+        case 6: ok = ragged_lookup_plane_nz6(*NY, f); break;
+        case 7: ok = ragged_lookup_plane_nz7(*NY, f); break;
+        case 8: ok = ragged_lookup_plane_nz8(*NY, f); break;
+        default: break;
+    }
+    return ok && (ragged_lookup_x_a(*NX, f) || ragged_lookup_x_b(*NX, f) ||
+                  ragged_lookup_x_c(*NX, f) || ragged_lookup_x_d(*NX, f));
+}
+
+// The plane kernel's trigger (fast_step.cuh), per L2-resident step, early
+// against late: where the x tiles cover the SMs early wins (250x250x4 18.9
+// against 20.2 us, 600x400x1 28.5 against 30.6, 50x200x2 6.9 against 7.2), as
+// it does where planes and tiles together leave each SM one block (30x30x1
+// 4.4 against 4.9); in between the early tiles share a few SMs with planes
+// and hold those up (200x60x3 12.3 against 9.6, 100x100x1 7.1 against 6.7).
+int ragged_early_trigger(const Geom& g, const FastStepFns& f, int sms) {
+    const int tiles = g.nz * (g.Jst / f.rb);
+    return tiles >= sms || tiles + g.Hx <= sms;
+}
+
+cudaError_t launch_ragged_pass1(const Geom& g, const FastStepFns& f, const float* M, float2* S, cudaStream_t s,
+                                float* Mcopy) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = launch_config(dim3(3 * g.nz * ((g.Jst + f.r1 - 1) / f.r1)), f.t1, f.s1, s, attr);
+    return cudaLaunchKernelEx(&cfg, f.p1, g, M, S, Mcopy);
+}
+
+}  // namespace mmk

@@ -369,9 +369,11 @@ cudaError_t tensor_spectrum(const int grid[3], const int L[3], const double* N_d
             k_pack2d<<<(unsigned)((nd + T - 1) / T), T, 0, s>>>(nz, Hx, Hy, Hyp, 1.0 / ((double)L[0] * L[1]), work2,
                                                                 Kd0_dev, ExchangeFold{});
     }
-    size_t n3 = (size_t)6 * Hx * Hy * Hz;
-    const double scale = 1.0 / ((double)L[0] * L[1] * L[2]);
-    k_tz<<<(unsigned)((n3 + T - 1) / T), T, 0, s>>>(nz, Hx, Hy, L[2], Hz, scale, work2, Kt_dev, csz);
+    if (Kt_dev) {
+        const size_t n3 = (size_t)6 * Hx * Hy * Hz;
+        const double scale = 1.0 / ((double)L[0] * L[1] * L[2]);
+        k_tz<<<(unsigned)((n3 + T - 1) / T), T, 0, s>>>(nz, Hx, Hy, L[2], Hz, scale, work2, Kt_dev, csz);
+    }
     e = cudaGetLastError();
     cudaError_t e2 = cudaFreeAsync(cs, s);
     return e != cudaSuccess ? e : e2;
