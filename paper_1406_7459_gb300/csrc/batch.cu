@@ -1,5 +1,11 @@
 // batch.cu -- many independent samples of uneven size stepped together.
 //
+// Samples with sides in the carrier lengths of the ragged-film kernels
+// (ragged_batch.cuh) step on those, one launch per class of lengths and pass,
+// the classes side by side; the others on the general mixed-radix kernels
+// described next.  512 samples of 16..256 x 16..64 x 1..2 cells: see
+// ragged_batch.cuh for both sides' times.
+//
 // Each sample is a complete problem of its own (grid, cell, material, field)
 // with its own tensor spectrum; the step of every sample is the paper's
 // three phases (Sec. 3: forward FFTs, member-wise product, inverse FFTs,
@@ -16,6 +22,7 @@
 // itself.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -24,54 +31,19 @@
 #include <vector>
 
 #include "../../include/mm.h"
+#include "batch_kernels.cuh"
 #include "bulk_copy.cuh"
 #include "grid_sync.cuh"
-#include "pass_bodies.cuh"
-#include "plane_kernel.cuh"
 
 using namespace mmk;
 
 namespace mmk {
-
-struct BatchDesc {
-    Geom g;
-    LlgCoef cf;
-    float* M0;
-    float* M1;
-    float2* S;
-    int r1, r3;
-    int r2;                                   // kx planes per plane-pass CTA
-};
-
-__device__ __forceinline__ int find_sample(const int* __restrict__ pre, int ns, int b) {
-    int lo = 0, hi = ns - 1;                  // largest s with pre[s] <= b
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(pre + mid) <= b) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
 
 __global__ void __launch_bounds__(256) k_batch_pass1(const BatchDesc* __restrict__ d, const int* __restrict__ pre,
                                                       int ns, int par) {
     const int s = find_sample(pre, ns, blockIdx.x);
     const BatchDesc& b = d[s];
     pass1_body(b.g, b.r1, b.r1 / 2, par ? b.M1 : b.M0, b.S, blockIdx.x - __ldg(pre + s));
-}
-
-// plane-pass tile `tile` of a sample: r2 consecutive kx planes (fewer at
-// the end), all their lines transformed together
-__device__ __forceinline__ void batch_plane_tile(const BatchDesc& b, int tile) {
-    const int kx0 = tile * b.r2;
-    const int np = min(b.r2, b.g.Hx - kx0);
-    const int nl = 3 * b.g.nz * np;
-    switch (b.g.Lz) {
-        case 1: plane_body_multi<1>(b.g, nl, b.S, kx0, np); break;
-        case 4: plane_body_multi<4>(b.g, nl, b.S, kx0, np); break;
-        case 5: plane_body_multi<5>(b.g, nl, b.S, kx0, np); break;
-        default: plane_body_multi<8>(b.g, nl, b.S, kx0, np); break;
-    }
 }
 
 __global__ void __launch_bounds__(256) k_batch_plane(const BatchDesc* __restrict__ d, const int* __restrict__ pre,
@@ -91,51 +63,6 @@ __global__ void __launch_bounds__(256) k_batch_pass3(const BatchDesc* __restrict
     cf.dt = dt;
     pass3_body<kModeStepX>(b.g, b.r3, 3 * b.r3 / 2, cf, b.S, par ? b.M1 : b.M0, par ? b.M0 : b.M1, flag,
                            blockIdx.x - __ldg(pre + s), b.S);
-}
-
-// n steps of every sample in one cooperative launch.  Work queue 0 holds
-// the pass-1 tiles (the x R2C of the starting state; only when the spectra
-// are not already those of that state), queue 1 the plane tiles, queue 2
-// the update tiles, which also form the next step's x spectra (kModeStepX,
-// in place: a tile reads exactly the spectrum entries it writes).  The
-// state goes M[par0] -> M[par0 ^ 1] -> ...  A grid-barrier wait that runs
-// out of polls sets kFlagTimeout.
-__global__ void __launch_bounds__(256) k_batch_persist(const BatchDesc* __restrict__ d, const int* __restrict__ pre,
-                                                        int ns, int t1, int t2, int t3, int par0, int nsteps,
-                                                        float dt, int first_x, int* __restrict__ flag,
-                                                        GridBar* __restrict__ gb, long long limit) {
-    __shared__ int slot;
-    const int P = ns + 1;
-    unsigned bar = 0;
-    bool ok = true;
-    if (first_x) {
-        for (int i; (i = queue_next(gb, 0, t1, 0, &slot)) >= 0;) {
-            const int s = find_sample(pre, ns, i);
-            const BatchDesc& b = d[s];
-            pass1_body(b.g, b.r1, b.r1 / 2, par0 ? b.M1 : b.M0, b.S, i - __ldg(pre + s));
-        }
-        ok = grid_sync(gb, bar++, limit);
-    }
-    for (int st = 0; ok && st < nsteps; ++st) {
-        const int par = (par0 + st) & 1;
-        for (int i; (i = queue_next(gb, 1, t2, st, &slot)) >= 0;) {
-            const int s = find_sample(pre + P, ns, i);
-            batch_plane_tile(d[s], i - __ldg(pre + P + s));
-        }
-        ok = grid_sync(gb, bar++, limit);
-        if (!ok) break;
-        for (int i; (i = queue_next(gb, 2, t3, st, &slot)) >= 0;) {
-            const int s = find_sample(pre + 2 * P, ns, i);
-            const BatchDesc& b = d[s];
-            LlgCoef cf = b.cf;
-            cf.dt = dt;
-            pass3_body<kModeStepX>(b.g, b.r3, 3 * b.r3 / 2, cf, b.S, par ? b.M1 : b.M0, par ? b.M0 : b.M1, flag,
-                                   i - __ldg(pre + 2 * P + s), b.S);
-        }
-        if (st + 1 < nsteps) ok = grid_sync(gb, bar++, limit);
-    }
-    if (!ok && threadIdx.x == 0) atomicOr(flag, kFlagTimeout);
-    grid_exit(gb);
 }
 
 }  // namespace mmk
@@ -161,8 +88,21 @@ struct mm_batch {
     BatchDesc* d_desc = nullptr;
     int* d_pre = nullptr;                      // 3 prefix arrays of ns + 1
     int* flag = nullptr;
-    int tiles[3] = {0, 0, 0};
+    int tiles[3] = {0, 0, 0};                  // of the samples on the general kernels
     size_t smem[3] = {0, 0, 0};
+    // samples on the ragged-film kernels, grouped by class (ragged_batch.cuh)
+    struct Group {
+        int first = 0, count = 0;              // of its items
+    };
+    std::vector<RagDesc> rag;
+    RagDesc* d_rag = nullptr;
+    RagItem* d_items = nullptr;
+    Group g1[kRagXClasses], g2[kRagPlaneClasses], g3[kRagXClasses];   // row transform, plane, update
+    int n_items[3] = {0, 0, 0}, off_items[3] = {0, 0, 0};
+    size_t rag_smem = 0;                       // largest tile, for the persistent launch
+    static constexpr int kSide = 3;            // streams beside the batch's own
+    cudaStream_t side[kSide] = {};
+    cudaEvent_t fork = nullptr, join[kSide] = {};
     int threads = 256, r1 = 4, r3 = 2, r2 = 1;
     int par = 0;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
@@ -216,6 +156,17 @@ static LlgCoef batch_coef(const mm_batch* b, int s) {
     return f;
 }
 
+// Let a kernel have all the dynamic shared memory its static part leaves.
+// The attribute belongs to the kernel, not to a batch: every batch of the
+// process sets the same value, so that none takes it away from another.
+template <typename F> static cudaError_t allow_smem(F* k) {
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, k);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(227 * 1024 - at.sharedSizeBytes));
+}
+
 // Tile counts, prefix tables, shared-memory sizes and descriptors for the
 // current shape choice (r1, r3, threads); uploads them.
 static int batch_layout(mm_batch* b) {
@@ -229,12 +180,12 @@ static int batch_layout(mm_batch* b) {
         d.r3 = b->r3;
         d.r2 = b->r2;
         d.cf = batch_coef(b, s);
+        b->rag[s].cf = d.cf;
+        for (int q = 0; q < 3; ++q) pre[q * (b->ns + 1) + s] = acc[q];
+        if (b->rag[s].xcls >= 0) continue;
         const int t1 = 3 * g.nz * ((g.ny + b->r1 - 1) / b->r1);
         const int t2 = (g.Hx + b->r2 - 1) / b->r2;
         const int t3 = g.nz * ((g.ny + b->r3 - 1) / b->r3);
-        pre[0 * (b->ns + 1) + s] = acc[0];
-        pre[1 * (b->ns + 1) + s] = acc[1];
-        pre[2 * (b->ns + 1) + s] = acc[2];
         acc[0] += t1;
         acc[1] += t2;
         acc[2] += t3;
@@ -251,30 +202,66 @@ static int batch_layout(mm_batch* b) {
         b->smem[q] = sm[q];
         if (sm[q] > 227 * 1024) return set_error(MM_EUNSUPPORTED, "batch sample exceeds shared memory");
     }
-    BCU(cudaFuncSetAttribute(k_batch_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm[0]));
-    BCU(cudaFuncSetAttribute(k_batch_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm[1]));
-    BCU(cudaFuncSetAttribute(k_batch_pass3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm[2]));
+    BCU(allow_smem(k_batch_pass1));
+    BCU(allow_smem(k_batch_plane));
+    BCU(allow_smem(k_batch_pass3));
     {
         size_t ps = sm[0] > sm[1] ? sm[0] : sm[1];
         ps = ps > sm[2] ? ps : sm[2];
+        ps = ps > b->rag_smem ? ps : b->rag_smem;
         b->psmem = ps;
-        BCU(cudaFuncSetAttribute(k_batch_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps));
+        BCU(allow_smem(batch_persist_fn()));
         int dev = 0, sms = 0, per_sm = 0;
         BCU(cudaGetDevice(&dev));
         BCU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        BCU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_persist, b->threads, ps));
+        BCU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_persist_fn(), kRagBatchThreads, ps));
         b->pgrid = per_sm * sms;
     }
+    BCU(cudaMemcpy(b->d_rag, b->rag.data(), sizeof(RagDesc) * b->ns, cudaMemcpyHostToDevice));
     BCU(cudaMemcpy(b->d_desc, b->desc.data(), sizeof(BatchDesc) * b->ns, cudaMemcpyHostToDevice));
     BCU(cudaMemcpy(b->d_pre, pre.data(), sizeof(int) * pre.size(), cudaMemcpyHostToDevice));
     b->ver++;
     return MM_OK;
 }
 
+// The class launches of a pass run side by side: fork the side streams off
+// s, deal the launches out over s and them, join back into s.
+struct Lanes {
+    mm_batch* b;
+    cudaStream_t s;
+    int next = 0;
+    cudaError_t begin() {
+        cudaError_t e = cudaEventRecord(b->fork, s);
+        for (int q = 0; q < mm_batch::kSide && e == cudaSuccess; ++q) e = cudaStreamWaitEvent(b->side[q], b->fork, 0);
+        return e;
+    }
+    cudaStream_t lane() {
+        const int q = next++ % (mm_batch::kSide + 1);
+        return q == 0 ? s : b->side[q - 1];
+    }
+    cudaError_t end() {
+        cudaError_t e = cudaGetLastError();
+        for (int q = 0; q < mm_batch::kSide; ++q) {
+            cudaError_t r = cudaEventRecord(b->join[q], b->side[q]);
+            if (r == cudaSuccess) r = cudaStreamWaitEvent(s, b->join[q], 0);
+            if (e == cudaSuccess) e = r;
+        }
+        return e;
+    }
+};
+
 // x R2C of every sample's state M[par] into its spectrum
 static int batch_pass1(mm_batch* b, int par, cudaStream_t s) {
-    k_batch_pass1<<<b->tiles[0], b->threads, b->smem[0], s>>>(b->d_desc, b->d_pre, b->ns, par);
-    BCU(cudaGetLastError());
+    Lanes l{b, s};
+    BCU(l.begin());
+    if (b->tiles[0])
+        k_batch_pass1<<<b->tiles[0], b->threads, b->smem[0], l.lane()>>>(b->d_desc, b->d_pre, b->ns, par);
+    for (int c = 0; c < kRagXClasses; ++c)
+        if (b->g1[c].count) {
+            const RagXFns f = rag_x_fns(c);
+            f.p1<<<b->g1[c].count, f.t1, f.s1, l.lane()>>>(b->d_rag, b->d_items + b->g1[c].first, par);
+        }
+    BCU(l.end());
     return MM_OK;
 }
 
@@ -282,11 +269,28 @@ static int batch_pass1(mm_batch* b, int par, cudaStream_t s) {
 // pass, then the update, which leaves the x transforms of M[par ^ 1].
 static int batch_enqueue(mm_batch* b, int par, double dt, cudaStream_t s) {
     const int P = b->ns + 1;
-    k_batch_plane<<<b->tiles[1], b->threads, b->smem[1], s>>>(b->d_desc, b->d_pre + P, b->ns);
-    BCU(cudaGetLastError());
-    k_batch_pass3<<<b->tiles[2], b->threads, b->smem[2], s>>>(b->d_desc, b->d_pre + 2 * P, b->ns, par, (float)dt,
-                                                              b->flag);
-    BCU(cudaGetLastError());
+    Lanes l{b, s};
+    BCU(l.begin());
+    if (b->tiles[1])
+        k_batch_plane<<<b->tiles[1], b->threads, b->smem[1], l.lane()>>>(b->d_desc, b->d_pre + P, b->ns);
+    for (int c = 0; c < kRagPlaneClasses; ++c)
+        if (b->g2[c].count) {
+            const RagPlaneFns f = rag_plane_fns(c);
+            f.k<<<b->g2[c].count, f.t, f.smem, l.lane()>>>(b->d_rag, b->d_items + b->g2[c].first, b->flag);
+        }
+    BCU(l.end());
+    Lanes u{b, s};
+    BCU(u.begin());
+    if (b->tiles[2])
+        k_batch_pass3<<<b->tiles[2], b->threads, b->smem[2], u.lane()>>>(b->d_desc, b->d_pre + 2 * P, b->ns, par,
+                                                                         (float)dt, b->flag);
+    for (int c = kRagXClasses - 1; c >= 0; --c)               // the long rows first
+        if (b->g3[c].count) {
+            const RagXFns f = rag_x_fns(c);
+            f.xs<<<b->g3[c].count, f.tx, f.sx, u.lane()>>>(b->d_rag, b->d_items + b->g3[c].first, par, (float)dt,
+                                                           b->flag);
+        }
+    BCU(u.end());
     return MM_OK;
 }
 
@@ -303,7 +307,64 @@ static void batch_release(mm_batch* b) {
     cudaFree(b->d_pre);
     cudaFree(b->flag);
     cudaFree(b->gb);
+    cudaFree(b->d_rag);
+    cudaFree(b->d_items);
+    for (int q = 0; q < mm_batch::kSide; ++q) {
+        if (b->side[q]) cudaStreamDestroy(b->side[q]);
+        if (b->join[q]) cudaEventDestroy(b->join[q]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
     if (b->cap) cudaStreamDestroy(b->cap);
+}
+
+// The carrier lengths and classes of a sample the ragged-film kernels take.
+static bool batch_classes(const Geom& g, int* NX, int* NY, int* xc, int* pc) {
+    *NX = plan_ragged_len(g.nx);
+    *NY = plan_ragged_len(g.ny);
+    *xc = rag_x_class(*NX);
+    *pc = rag_plane_class(*NY, g.nz);
+    return *xc >= 0 && *pc >= 0;
+}
+
+// Item lists per class (they depend on the grids only) and the kernels'
+// shared memory.
+static int batch_items(mm_batch* b) {
+    std::vector<RagItem> items;
+    auto fill = [&](mm_batch::Group* g, int ncls, int pass) {
+        b->off_items[pass] = (int)items.size();
+        for (int c = 0; c < ncls; ++c) {
+            g[c].first = (int)items.size();
+            for (int s = 0; s < b->ns; ++s) {
+                const RagDesc& d = b->rag[s];
+                if (d.xcls < 0 || (pass == 1 ? d.pcls : d.xcls) != c) continue;
+                const int n = pass == 0   ? 3 * d.nz * ((d.Jst + kRagRows1 - 1) / kRagRows1)
+                              : pass == 1 ? b->desc[s].g.Hx
+                                          : d.nz * (d.Jst / rag_x_fns(c).rows);
+                for (int t = 0; t < n; ++t) items.push_back(RagItem{s, t});
+            }
+            g[c].count = (int)items.size() - g[c].first;
+        }
+        b->n_items[pass] = (int)items.size() - b->off_items[pass];
+    };
+    fill(b->g1, kRagXClasses, 0);
+    fill(b->g2, kRagPlaneClasses, 1);
+    fill(b->g3, kRagXClasses, 2);
+    for (int c = 0; c < kRagXClasses; ++c)
+        if (b->g1[c].count) {
+            const RagXFns f = rag_x_fns(c);
+            BCU(allow_smem(f.p1));
+            BCU(allow_smem(f.xs));
+            b->rag_smem = std::max(b->rag_smem, std::max(f.s1, f.sx));
+        }
+    for (int c = 0; c < kRagPlaneClasses; ++c)
+        if (b->g2[c].count) {
+            const RagPlaneFns f = rag_plane_fns(c);
+            BCU(allow_smem(f.k));
+            b->rag_smem = std::max(b->rag_smem, f.smem);
+        }
+    BCU(cudaMalloc(&b->d_items, sizeof(RagItem) * (items.empty() ? 1 : items.size())));
+    BCU(cudaMemcpy(b->d_items, items.data(), sizeof(RagItem) * items.size(), cudaMemcpyHostToDevice));
+    return MM_OK;
 }
 
 extern "C" int mm_batch_create(mm_batch** out, int n, const int* grids, const double* cells, const double* Ms,
@@ -327,6 +388,7 @@ extern "C" int mm_batch_create(mm_batch** out, int n, const int* grids, const do
     b->Hext.assign(3 * n, 0.0);
     b->desc.resize(n);
     b->moff.resize(n);
+    b->rag.resize(n);
     int rc = [&]() -> int {
         size_t mt = 0, st = 0, kt = 0, tt = 0, wmax = 0, nmax = 0;
         std::vector<size_t> soff(n), koff(n), toff(n);
@@ -354,12 +416,29 @@ extern "C" int mm_batch_create(mm_batch** out, int n, const int* grids, const do
             g.Jst = ny;
             if (!plan_axis(g.Lx, &g.px) || !plan_axis(g.Ly, &g.py) || !plan_axis(g.Lz, &g.pz))
                 return set_error(MM_EUNSUPPORTED, "no radix plan");
+            RagDesc& rd = b->rag[s];
+            memset(&rd, 0, sizeof(rd));
+            int NX = 0, NY = 0;
+            if (batch_classes(g, &NX, &NY, &rd.xcls, &rd.pcls)) {
+                g.Lx = 2 * NX;
+                g.Ly = 2 * NY;
+                g.Lz = 1;                                     // the z sum is direct
+                g.Hx = NX + 1;
+                g.Hy = NY + 1;
+                g.Hz = 1;
+                g.Jst = (ny + 3) & ~3;
+            } else {
+                rd.xcls = rd.pcls = -1;
+            }
             b->moff[s] = mt;
             mt += 3 * (size_t)g.N;
+            // every sample's spectra start on 16 bytes (bulk copies)
             soff[s] = st;
-            st += (size_t)g.Hx * 3 * nz * ny;
+            st += ((size_t)g.Hx * 3 * nz * g.Jst + 1) & ~(size_t)1;
             koff[s] = kt;
-            kt += (size_t)6 * g.Hx * g.Hy * g.Hz;
+            kt += rd.xcls >= 0 ? (size_t)6 * g.Hx * kd_row(g.Hy) * nz
+                               : ((size_t)6 * g.Hx * g.Hy * g.Hz + 3) & ~(size_t)3;
+            tt += tt & 1;
             toff[s] = tt;
             tt += (size_t)(g.Lx + g.Ly + g.Lz);
             const int L[3] = {g.Lx, g.Ly, g.Lz};
@@ -377,6 +456,12 @@ extern "C" int mm_batch_create(mm_batch** out, int n, const int* grids, const do
         BCU(cudaMalloc(&b->tw, sizeof(float2) * tt));
         BCU(cudaMalloc(&b->d_desc, sizeof(BatchDesc) * n));
         BCU(cudaMalloc(&b->d_pre, sizeof(int) * 3 * (n + 1)));
+        BCU(cudaMalloc(&b->d_rag, sizeof(RagDesc) * n));
+        BCU(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
+        for (int q = 0; q < mm_batch::kSide; ++q) {
+            BCU(cudaStreamCreateWithFlags(&b->side[q], cudaStreamNonBlocking));
+            BCU(cudaEventCreateWithFlags(&b->join[q], cudaEventDisableTiming));
+        }
         BCU(cudaMalloc(&b->flag, sizeof(int)));
         BCU(cudaMemset(b->flag, 0, sizeof(int)));
         BCU(cudaMalloc(&b->gb, sizeof(GridBar)));
@@ -398,6 +483,18 @@ extern "C" int mm_batch_create(mm_batch** out, int n, const int* grids, const do
             b->desc[s].M0 = b->M0 + b->moff[s];
             b->desc[s].M1 = b->M1 + b->moff[s];
             b->desc[s].S = b->S + soff[s];
+            RagDesc& rd = b->rag[s];
+            rd.nx = g.nx;
+            rd.ny = g.ny;
+            rd.nz = g.nz;
+            rd.N = g.N;
+            rd.Jst = g.Jst;
+            rd.twx = g.twx;
+            rd.twy = g.twy;
+            rd.Kd = g.Kt;
+            rd.M[0] = b->desc[s].M0;
+            rd.M[1] = b->desc[s].M1;
+            rd.S = b->desc[s].S;
             for (int i = 0; i < g.N; ++i) {
                 hm[b->moff[s] + i] = (float)Ms[s];
                 hm[b->moff[s] + g.N + i] = 0.f;
@@ -415,14 +512,18 @@ extern "C" int mm_batch_create(mm_batch** out, int n, const int* grids, const do
             const Geom& g = b->desc[s].g;
             const int L[3] = {g.Lx, g.Ly, g.Lz};
             e = tensor_octant_fp64(&grids[3 * s], &cells[3 * s], Nd, b->stream);
-            if (e == cudaSuccess) e = tensor_spectrum(&grids[3 * s], L, Nd, b->Kt + koff[s], w1, w2, b->stream);
+            float* Ks = b->Kt + koff[s];
+            if (e == cudaSuccess)
+                e = b->rag[s].xcls >= 0 ? tensor_spectrum(&grids[3 * s], L, Nd, nullptr, w1, w2, b->stream, Ks)
+                                        : tensor_spectrum(&grids[3 * s], L, Nd, Ks, w1, w2, b->stream);
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
         cudaFree(Nd);
         cudaFree(w1);
         cudaFree(w2);
         BCU(e);
-        return batch_layout(b);
+        const int rc2 = batch_items(b);
+        return rc2 != MM_OK ? rc2 : batch_layout(b);
     }();
     if (rc != MM_OK) {
         batch_release(b);
@@ -494,14 +595,16 @@ static cudaError_t batch_launch_persist(const mm_batch* b, int m, double dt, int
     attr[0].val.cooperative = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(b->pgrid);
-    cfg.blockDim = dim3(b->threads);
+    cfg.blockDim = dim3(kRagBatchThreads);
     cfg.dynamicSmemBytes = b->psmem;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_batch_persist, (const BatchDesc*)b->d_desc, (const int*)b->d_pre, b->ns,
-                              b->tiles[0], b->tiles[1], b->tiles[2], b->par, m, (float)dt, first, b->flag, b->gb,
-                              b->wait_limit);
+    BatchPass q[3];
+    for (int i = 0; i < 3; ++i)
+        q[i] = BatchPass{b->d_items + b->off_items[i], b->d_pre + i * (b->ns + 1), b->n_items[i], b->tiles[i]};
+    return cudaLaunchKernelEx(&cfg, batch_persist_fn(), (const BatchDesc*)b->d_desc, (const RagDesc*)b->d_rag, q[0],
+                              q[1], q[2], b->ns, b->par, m, (float)dt, first, b->flag, b->gb, b->wait_limit);
 }
 
 // The launch of m steps as a graph replay: captured (on the capture stream)

@@ -28,12 +28,14 @@ __host__ __device__ constexpr int pzlen(int L) { return L + L / 16 + 1; }
 // RAG: a ragged sample, g.nx <= N cells per row and g.ny rows of a spectrum
 // row stride g.Jst (ny rounded up): cells past nx and rows past ny are zeros,
 // and the zero rows' spectra (up to Jst) are written like the others.
-template <int N, int R, bool RAG = false>
-__global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const float* __restrict__ M,
-                                                                float2* __restrict__ S, float* __restrict__ Mcopy) {
+// T: the block size (threads past the R G of the transforms only help with
+// the copies and the split).
+template <int N, int R, int T, bool RAG>
+__device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float* __restrict__ M,
+                                           float2* __restrict__ S, float* __restrict__ Mcopy) {
     using F = Fft2<N>;
     constexpr int P = F::P, Q = F::Q, G = F::G, L = 2 * N, ZS = pzlen(2 * N);
-    constexpr int T = R * G;                              // the launch's block size
+    static_assert(T >= R * G, "block smaller than the tile's transform groups");
     extern __shared__ float2 sm[];
     float2* tw = sm;
     float2* ta = tw + L;                  // RAG: every twiddle from a table, rounded once (N entries)
@@ -41,7 +43,7 @@ __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const flo
     float2* zb = ex + R * F::EX;
     const int ntj = RAG ? (g.Jst + R - 1) / R : g.ny / R;
     const int nx = RAG ? g.nx : N;
-    int b = blockIdx.x;
+    int b = tile;
     const int jt = b % ntj;
     b /= ntj;
     const int k = b % g.nz;
@@ -58,7 +60,8 @@ __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const flo
 
     const int grp = threadIdx.x / G, t = threadIdx.x % G;
     const int p = grp >> 1, h = grp & 1;
-    if (t < Q) {
+    const bool act = T == R * G || grp < R;
+    if (act && t < Q) {
         const float* ra = M + (size_t)c * g.N + ((size_t)k * g.ny + j0 + 2 * p) * nx;
         const float* rb = ra + nx;
         const int na = !RAG || j0 + 2 * p < g.ny ? nx : 0, nb = !RAG || j0 + 2 * p + 1 < g.ny ? nx : 0;
@@ -89,7 +92,7 @@ __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const flo
         }
     }
     __syncthreads();
-    if (t < P) {
+    if (act && t < P) {
         float2 w[Q];
         F::stepB(w, t, ex + grp * F::EX, false);
 #pragma unroll
@@ -110,6 +113,12 @@ __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const flo
         else o = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
         S[(((size_t)kx * 3 + c) * g.nz + k) * g.Jst + j0 + r] = o;
     }
+}
+
+template <int N, int R, bool RAG = false>
+__global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const float* __restrict__ M,
+                                                                float2* __restrict__ S, float* __restrict__ Mcopy) {
+    pass1_rows<N, R, R * Fft2<N>::G, RAG>(g, blockIdx.x, M, S, Mcopy);
 }
 
 // ---------------------------------------------------------------- pass 2 --

@@ -387,6 +387,21 @@ struct XTma {
     uint32_t bar = 0;
 };
 
+// Eq. (6) with its contractions written out, so that every kernel that
+// inlines it rounds alike: f = c1 M x H + c2 M x (M x H).
+__device__ __forceinline__ void llg_rhs_fixed(const LlgCoef& cf, const float (&m)[3], const float (&h)[3],
+                                              float (&f)[3]) {
+    const float p0 = fmaf(m[1], h[2], -__fmul_rn(m[2], h[1]));
+    const float p1 = fmaf(m[2], h[0], -__fmul_rn(m[0], h[2]));
+    const float p2 = fmaf(m[0], h[1], -__fmul_rn(m[1], h[0]));
+    const float q0 = fmaf(m[1], p2, -__fmul_rn(m[2], p1));
+    const float q1 = fmaf(m[2], p0, -__fmul_rn(m[0], p2));
+    const float q2 = fmaf(m[0], p1, -__fmul_rn(m[1], p0));
+    f[0] = fmaf(cf.c1, p0, __fmul_rn(cf.c2, q0));
+    f[1] = fmaf(cf.c1, p1, __fmul_rn(cf.c2, q1));
+    f[2] = fmaf(cf.c1, p2, __fmul_rn(cf.c2, q2));
+}
+
 // A thread's cells of a ragged x-step tile (its trips of the field loop):
 // M and the exchange field of Eq. (4), formed before the spectrum arrives.
 template <int CPT> struct RagCells {
@@ -571,25 +586,42 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
             }
         }
         hh[0] += cf.hx;
-        hh[1] += cf.panis * m[1] + cf.hy;
-        hh[2] += cf.panis * m[2] + cf.hz;
+        if constexpr (RAG) {
+            hh[1] += fmaf(cf.panis, m[1], cf.hy);
+            hh[2] += fmaf(cf.panis, m[2], cf.hz);
+        } else {
+            hh[1] += cf.panis * m[1] + cf.hy;
+            hh[2] += cf.panis * m[2] + cf.hz;
+        }
         if constexpr (MODE == kModeHeff) {
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc) Mout[cc * Nc + cell] = hh[cc];
             continue;
         }
-        const float p0 = m[1] * hh[2] - m[2] * hh[1];
-        const float p1 = m[2] * hh[0] - m[0] * hh[2];
-        const float p2 = m[0] * hh[1] - m[1] * hh[0];
-        const float q0 = m[1] * p2 - m[2] * p1;
-        const float q1 = m[2] * p0 - m[0] * p2;
-        const float q2 = m[0] * p1 - m[1] * p0;
-        const float n0 = m[0] + cf.dt * (cf.c1 * p0 + cf.c2 * q0);
-        const float n1 = m[1] + cf.dt * (cf.c1 * p1 + cf.c2 * q1);
-        const float n2 = m[2] + cf.dt * (cf.c1 * p2 + cf.c2 * q2);
-        const float s = RAG ? cf.Ms / sqrtf(n0 * n0 + n1 * n1 + n2 * n2)
-                            : cf.Ms * rsqrtf(n0 * n0 + n1 * n1 + n2 * n2);
-        const float o0 = n0 * s, o1 = n1 * s, o2 = n2 * s;
+        float o0, o1, o2;
+        if constexpr (RAG) {
+            float f[3];
+            llg_rhs_fixed(cf, m, hh, f);
+            const float n0 = fmaf(cf.dt, f[0], m[0]), n1 = fmaf(cf.dt, f[1], m[1]), n2 = fmaf(cf.dt, f[2], m[2]);
+            const float s = cf.Ms / sqrtf(fmaf(n2, n2, fmaf(n1, n1, __fmul_rn(n0, n0))));
+            o0 = __fmul_rn(n0, s);
+            o1 = __fmul_rn(n1, s);
+            o2 = __fmul_rn(n2, s);
+        } else {
+            const float p0 = m[1] * hh[2] - m[2] * hh[1];
+            const float p1 = m[2] * hh[0] - m[0] * hh[2];
+            const float p2 = m[0] * hh[1] - m[1] * hh[0];
+            const float q0 = m[1] * p2 - m[2] * p1;
+            const float q1 = m[2] * p0 - m[0] * p2;
+            const float q2 = m[0] * p1 - m[1] * p0;
+            const float n0 = m[0] + cf.dt * (cf.c1 * p0 + cf.c2 * q0);
+            const float n1 = m[1] + cf.dt * (cf.c1 * p1 + cf.c2 * q1);
+            const float n2 = m[2] + cf.dt * (cf.c1 * p2 + cf.c2 * q2);
+            const float s = cf.Ms * rsqrtf(n0 * n0 + n1 * n1 + n2 * n2);
+            o0 = n0 * s;
+            o1 = n1 * s;
+            o2 = n2 * s;
+        }
         if (!isfinite(o0 + o1 + o2)) atomicOr(flag, kFlagNonFinite);   // |o| <= Ms when finite
         if (Mout) {
             Mout[cell] = o0;
@@ -688,11 +720,13 @@ __device__ __forceinline__ void load_rag_cells(const Geom& g, const LlgCoef& cf,
         for (int c = 0; c < 3; ++c) {
             const float* Mc = M + (size_t)c * Nc;
             const float m0 = __ldg(Mc + cell);
-            float lap = (__ldg(Mc + xp) - 2.f * m0 + __ldg(Mc + xm)) * cf.idx2 +
-                        (__ldg(Mc + yp) - 2.f * m0 + __ldg(Mc + ym)) * cf.idy2;
-            if (g.nz > 1) lap += (__ldg(Mc + zp) - 2.f * m0 + __ldg(Mc + zm)) * cf.idz2;
+            // contractions written out: the single and the batched kernel
+            // round alike
+            float lap = __fmul_rn(fmaf(-2.f, m0, __ldg(Mc + xp)) + __ldg(Mc + xm), cf.idx2);
+            lap = fmaf(fmaf(-2.f, m0, __ldg(Mc + yp)) + __ldg(Mc + ym), cf.idy2, lap);
+            if (g.nz > 1) lap = fmaf(fmaf(-2.f, m0, __ldg(Mc + zp)) + __ldg(Mc + zm), cf.idz2, lap);
             rc.m[u][c] = m0;
-            rc.ex[u][c] = cf.pexch * lap;
+            rc.ex[u][c] = __fmul_rn(cf.pexch, lap);
         }
     }
 }

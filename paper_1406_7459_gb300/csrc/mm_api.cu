@@ -191,7 +191,9 @@ static int build_plan(mm_ctx* c) {
         c->has_persist = ok && persist_lookup(g.nx, g.ny, g.nz, s.rb, &c->pf);
     }
     c->gf = g;
-    c->rag = allow_fast && !c->has_fs && !c->has_ss && plan_ragged(c);
+    // without the compile-time power-of-two kernels (MM_NO_FAST=1) a context
+    // takes the kernels that a batch takes for the same sample
+    c->rag = !c->has_fs && !c->has_ss && (allow_fast || ragged_batchable(g.nx, g.ny, g.nz)) && plan_ragged(c);
     if (c->rag) {
         c->has_fs = true;
         c->has_persist = false;

@@ -98,6 +98,7 @@ enum Pass3Mode { kModeDemag = 0, kModeHeff = 1, kModeStep = 2, kModeStepX = 3 };
 
 // Planning helpers (mm_api.cu), shared with the batched driver.
 int plan_padded_length(int n);
+int plan_ragged_len(int n);        // carrier length of a ragged side, or 0 (ragged_select.cu)
 bool plan_axis(int L, AxisPlan* p);
 void plan_twiddles(int L, float2* out);
 int set_error(int code, const char* msg);
@@ -190,6 +191,8 @@ bool fast_step_lookup_plane_b(int ny, int nz, FastStepFns* f);
 // Ragged films (ragged.cuh): the kernels and the carrier lengths NX >= nx,
 // NY >= ny; whether the plane kernel triggers the x-step early.
 bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY);
+// Films that a batch takes on the ragged kernels (ragged_batch.cuh).
+bool ragged_batchable(int nx, int ny, int nz);
 int ragged_early_trigger(const Geom& g, const FastStepFns& f, int sms);
 cudaError_t launch_ragged_pass1(const Geom& g, const FastStepFns& f, const float* M, float2* S, cudaStream_t s,
                                 float* Mcopy = nullptr);

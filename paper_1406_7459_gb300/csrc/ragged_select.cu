@@ -1,6 +1,6 @@
 // ragged_select.cu -- picks the kernels and carrier lengths of a ragged film
 // (ragged.cuh) and launches its row transform.
-#include "ragged.cuh"
+#include "ragged_batch.cuh"
 
 namespace mmk {
 
@@ -35,6 +35,12 @@ bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY) {
     }
     return ok && (ragged_lookup_x_a(*NX, f) || ragged_lookup_x_b(*NX, f) ||
                   ragged_lookup_x_c(*NX, f) || ragged_lookup_x_d(*NX, f));
+}
+
+int plan_ragged_len(int n) { return ragged_len(n); }
+
+bool ragged_batchable(int nx, int ny, int nz) {
+    return rag_x_class(ragged_len(nx)) >= 0 && rag_plane_class(ragged_len(ny), nz) >= 0;
 }
 
 // The plane kernel's trigger (fast_step.cuh), per L2-resident step, early

@@ -10,7 +10,7 @@ namespace mmk {
 // 36.8 us with two, 500x500x2 51.0 against 63.0: two rows leave 32-thread
 // transform groups too few per block and read 16-byte runs of the spectrum)
 // where their shared memory fits.
-template <int N> constexpr int rag_rows() {
+template <int N> __host__ __device__ constexpr int rag_rows() {
     return N <= 256 || XstepLayout<N, 4>::BYTES > 200 * 1024 ? 2 : 4;
 }
 
