@@ -38,6 +38,71 @@ static DpWeights dp_row(const double* w, int n) {
     return r;
 }
 
+// The kernels of one trial step where a stage is the plane pass and one
+// kernel: the row transform of the stage-2 state M + h a21 k1 (on the first
+// step stage 1 forms it), stages 2..6, and the seventh slope with the error
+// estimate.  The stage states alternate between two buffers (H is free here).
+static int dp_step_fused(mm_ctx* c, const DpPtrs& kp, const LlgCoef& cf, const float* M, float* cand, bool k1_valid,
+                         cudaStream_t s) {
+    float* Y[2] = {c->Mst, c->H};
+    auto args = [&](const double* w, int stage, float* out) {
+        StageArgs st{};
+        st.base = M;
+        st.kout = kp.k[stage - 1];
+        for (int j = 0; j < stage - 1; ++j)
+            if (w[j] != 0.0) {
+                st.k[st.nk] = kp.k[j];
+                st.w[st.nk++] = (float)w[j];
+            }
+        st.wf = (float)w[stage - 1];
+        st.out = out;
+        st.err = c->dperr;
+        return st;
+    };
+    if (!k1_valid) {
+        CU(cudaMemsetAsync(c->dperr, 0, sizeof(unsigned), s));
+        CU(form_spectrum(c, M, s));
+        int rc = fused_stage(c, kModeStage, M, args(kDpA[1], 1, Y[0]), cf, s);
+        if (rc != MM_OK) return rc;
+    } else {
+        CU(form_spectrum(c, M, s, Y[0], XComb{kp.k[0], (float)kDpA[1][0], cf.dt, c->dperr}));
+    }
+    for (int stage = 2; stage <= 6; ++stage) {
+        const bool last = stage == 6;
+        StageArgs st = args(last ? kDpB : kDpA[stage], stage, last ? cand : Y[(stage - 1) & 1]);
+        st.last = last;
+        int rc = fused_stage(c, kModeStage, Y[stage & 1], st, cf, s);
+        if (rc != MM_OK) return rc;
+    }
+    return fused_stage(c, kModeErr, cand, args(kDpE, 7, nullptr), cf, s);
+}
+
+// The same with a field evaluation and a stage update per stage (the general
+// kernels).
+static int dp_step_plain(mm_ctx* c, const DpPtrs& kp, const LlgCoef& cf, const float* M, float* cand, bool k1_valid,
+                         cudaStream_t s) {
+    int rc;
+    if (!k1_valid) {
+        rc = run_passes(c, kModeHeff, M, c->H, 0.0, s);
+        if (rc != MM_OK) return rc;
+        CU(launch_dp_stage(c->g.N, cf, kp, 1, dp_row(kDpA[1], 1), 0, M, c->H, M, c->Mst, nullptr, s));
+    } else {
+        CU(launch_dp_combine(c->g.N, kp, dp_row(kDpA[1], 1), 1, cf.dt, M, c->Mst, s));
+    }
+    for (int st = 2; st <= 6; ++st) {
+        rc = run_passes(c, kModeHeff, c->Mst, c->H, 0.0, s);
+        if (rc != MM_OK) return rc;
+        const bool last = st == 6;
+        const DpWeights w = last ? dp_row(kDpB, 6) : dp_row(kDpA[st], st);
+        CU(launch_dp_stage(c->g.N, cf, kp, st, w, last ? 1 : 0, c->Mst, c->H, M, last ? cand : c->Mst, nullptr, s));
+    }
+    rc = run_passes(c, kModeHeff, cand, c->H, 0.0, s);
+    if (rc != MM_OK) return rc;
+    CU(cudaMemsetAsync(c->dperr, 0, sizeof(unsigned), s));
+    CU(launch_dp_error(c->g.N, cf, kp, dp_row(kDpE, 7), cand, c->H, kp.k[6], c->dperr, s));
+    return MM_OK;
+}
+
 extern "C" int mm_run_adaptive(mm_ctx* c, double t_span, double* dt_io, double tol, int max_steps,
                                double stats[4]) {
     if (!c || !dt_io) return fail(MM_EINVAL, "null argument");
@@ -50,10 +115,10 @@ extern "C" int mm_run_adaptive(mm_ctx* c, double t_span, double* dt_io, double t
     for (int q = 0; q < 7; ++q)
         if (!c->dpk[q]) CU(cudaMalloc(&c->dpk[q], sizeof(float) * n3));
     if (!c->dperr) CU(cudaMalloc(&c->dperr, sizeof(unsigned)));
+    if (!c->hperr) CU(cudaMallocHost(&c->hperr, sizeof(unsigned)));
     cudaStream_t s = c->stream;
     DpPtrs kp;
     for (int q = 0; q < 7; ++q) kp.k[q] = c->dpk[q];
-    const DpWeights we = dp_row(kDpE, 7);
     double t = 0.0, dt = *dt_io;
     long long acc = 0, rej = 0, nev = 0;
     bool after_reject = false, k1_valid = false;
@@ -65,35 +130,16 @@ extern "C" int mm_run_adaptive(mm_ctx* c, double t_span, double* dt_io, double t
         const LlgCoef cf = make_coef(c, h);
         const float* M = c->Mbuf[p];
         float* cand = c->Mbuf[1 - p];
-        // stage 2 state (and k1 = f(M) on the first step; later k1 is the
-        // previous step's seventh stage)
-        if (!k1_valid) {
-            rc = run_passes(c, kModeHeff, M, c->H, 0.0, s);
-            if (rc != MM_OK) return rc;
-            CU(launch_dp_stage(c->g.N, cf, kp, 1, dp_row(kDpA[1], 1), 0, M, c->H, M, c->Mst, nullptr, s));
-            nev += 1;
-            k1_valid = true;
-        } else {
-            CU(launch_dp_combine(c->g.N, kp, dp_row(kDpA[1], 1), 1, (float)h, M, c->Mst, s));
-        }
-        for (int st = 2; st <= 6; ++st) {
-            rc = run_passes(c, kModeHeff, c->Mst, c->H, 0.0, s);
-            if (rc != MM_OK) return rc;
-            const bool last = st == 6;
-            const DpWeights w = last ? dp_row(kDpB, 6) : dp_row(kDpA[st], st);
-            CU(launch_dp_stage(c->g.N, cf, kp, st, w, last ? 1 : 0, c->Mst, c->H, M, last ? cand : c->Mst, nullptr,
-                               s));
-        }
-        rc = run_passes(c, kModeHeff, cand, c->H, 0.0, s);
+        rc = fused_stages(c) ? dp_step_fused(c, kp, cf, M, cand, k1_valid, s)
+                             : dp_step_plain(c, kp, cf, M, cand, k1_valid, s);
         if (rc != MM_OK) return rc;
-        CU(cudaMemsetAsync(c->dperr, 0, sizeof(unsigned), s));
-        CU(launch_dp_error(c->g.N, cf, kp, we, cand, c->H, kp.k[6], c->dperr, s));
-        unsigned bits = 0;
-        CU(cudaMemcpyAsync(&bits, c->dperr, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+        nev += k1_valid ? 0 : 1;
+        k1_valid = true;
+        CU(cudaMemcpyAsync(c->hperr, c->dperr, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
         CU(cudaStreamSynchronize(s));
         nev += 6;
         float errf;
-        std::memcpy(&errf, &bits, sizeof(float));
+        std::memcpy(&errf, c->hperr, sizeof(float));
         const double err = (double)errf;
         if (err <= tol) {
             t += h;

@@ -71,6 +71,7 @@ struct mm_ctx {
     bool spec_valid = false;   // S holds the x half-spectrum of M[cur] (two-kernel step)
     float* dpk[7] = {};        // Dormand-Prince stage slopes (adaptive runs), 3*N each
     unsigned* dperr = nullptr; // error estimate of the last trial step (float bits)
+    unsigned* hperr = nullptr; // its page-locked host copy
     PersistFns pf;             // persistent step (square power-of-two films it is built for)
     bool has_persist = false;  // the persistent step fits this grid and device
     int step_path = MM_STEP_AUTO;
@@ -84,6 +85,18 @@ namespace mmk {
 LlgCoef make_coef(const mm_ctx* c, double dt);
 // x R2C, plane, x C2R (+ field / step per mode) of M into out on stream s;
 // invalidates a pending step spectrum.
+cudaError_t form_spectrum(mm_ctx* c, const float* M, cudaStream_t s, float* Mcopy = nullptr,
+                          const XComb& comb = XComb{});
+// Whether a Runge-Kutta stage of this context is the plane pass and one
+// kernel (fused_stage) instead of a field evaluation and a stage update.
+// Not where the plane kernel runs more than 512 threads (512x512x4: 472 us per
+// RK4 step fused, 440 with the three-pass field evaluations).
+inline bool fused_stages(const mm_ctx* c) {
+    return c->has_fs ? c->rag || c->fs.ta <= 512 : c->has_ss && c->l.fx;
+}
+// One stage at the state Y whose x spectrum is in S: the slope's use per st
+// (mode kModeStage, which leaves the next state's spectrum in S, or kModeErr).
+int fused_stage(mm_ctx* c, int mode, const float* Y, const StageArgs& st, const LlgCoef& cf, cudaStream_t s);
 int run_passes(mm_ctx* c, int mode, const float* M, float* out, double dt, cudaStream_t s);
 
 }  // namespace mmk

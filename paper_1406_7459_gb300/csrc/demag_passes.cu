@@ -48,6 +48,8 @@ cudaError_t configure_pass_kernels(const Geom& g, const Launch& l) {
     cudaError_t e;
     if (l.fx) {
         e = cudaFuncSetAttribute(l.fx->p1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.fx->s1);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(l.fx->p1c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.fx->s1);
         for (int m = 0; m < 3 && e == cudaSuccess; ++m)
             e = cudaFuncSetAttribute(l.fx->p3[m], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.fx->s3);
         if (e != cudaSuccess) return e;
@@ -69,13 +71,15 @@ cudaError_t configure_pass_kernels(const Geom& g, const Launch& l) {
     if (!pf) return cudaErrorInvalidValue;
     return cudaFuncSetAttribute(pf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem2);
 }
-cudaError_t launch_pass1(const Geom& g, const Launch& l, const float* M, float2* S, cudaStream_t s, float* Mcopy) {
+cudaError_t launch_pass1(const Geom& g, const Launch& l, const float* M, float2* S, cudaStream_t s, float* Mcopy,
+                         const XComb& comb) {
     if (l.fx) {
         cudaLaunchAttribute attr[1];
         cudaLaunchConfig_t cfg = launch_config(dim3(3 * g.nz * (g.ny / l.fx->r1)), l.fx->t1, l.fx->s1, s, attr);
+        if (comb.K) return cudaLaunchKernelEx(&cfg, l.fx->p1c, g, M, S, Mcopy, comb);
         return cudaLaunchKernelEx(&cfg, l.fx->p1, g, M, S, Mcopy);
     }
-    if (Mcopy) return cudaErrorInvalidValue;      // the generic pass keeps no copy
+    if (Mcopy || comb.K) return cudaErrorInvalidValue;      // the generic pass keeps no copy and adds nothing
     const int ntj = (g.ny + l.r1 - 1) / l.r1;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = launch_config(dim3(3 * g.nz * ntj), l.t1, l.smem1, s, attr);

@@ -25,14 +25,83 @@ __host__ __device__ constexpr int pzlen(int L) { return L + L / 16 + 1; }
 // one complex line).  Groups of G threads: (pair, half).
 // Mcopy (may be null): a second copy of the rows read, e.g. the device copy
 // of a state that M points to in host memory.
-// RAG: a ragged sample, g.nx <= N cells per row and g.ny rows of a spectrum
+template <int N, int R>
+__global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const float* __restrict__ M,
+                                                                float2* __restrict__ S, float* __restrict__ Mcopy) {
+    using F = Fft2<N>;
+    constexpr int P = F::P, Q = F::Q, G = F::G, L = 2 * N, ZS = pzlen(2 * N);
+    constexpr int T = R * G;                              // the launch's block size
+    extern __shared__ float2 sm[];
+    float2* tw = sm;
+    float2* ex = tw + L;
+    float2* zb = ex + R * F::EX;
+    const int ntj = g.ny / R;
+    int b = blockIdx.x;
+    const int jt = b % ntj;
+    b /= ntj;
+    const int k = b % g.nz;
+    const int c = b / g.nz;
+    const int j0 = jt * R;
+#pragma unroll
+    for (int i = threadIdx.x; i < L; i += T) tw[i] = __ldg(g.twx + i);
+    pdl_wait();                           // M and S may belong to the previous kernel
+    __syncthreads();
+
+    const int grp = threadIdx.x / G, t = threadIdx.x % G;
+    const int p = grp >> 1, h = grp & 1;
+    if (t < Q) {
+        const float* ra = M + (size_t)c * g.N + ((size_t)k * g.ny + j0 + 2 * p) * N;
+        const float* rb = ra + N;
+        float2 v[P];
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            const int j = t + Q * q;
+            v[q] = make_float2(__ldg(ra + j), __ldg(rb + j));
+        }
+        if (Mcopy && h == 0) {
+            float* ca = Mcopy + (ra - M);
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const int j = t + Q * q;
+                ca[j] = v[q].x;
+                ca[N + j] = v[q].y;
+            }
+        }
+        if (h) F::odd_input(v, t, tw);
+        F::stepA(v, t, tw, ex + grp * F::EX, false);
+    }
+    __syncthreads();
+    if (t < P) {
+        float2 w[Q];
+        F::stepB(w, t, ex + grp * F::EX, false);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) zb[p * ZS + pz(2 * (t + P * q) + h)] = w[q];
+    }
+    __syncthreads();
+    // A[k] = (Z[k] + conj Z[L-k]) / 2 (even row), B[k] = -i (Z[k] - conj Z[L-k]) / 2
+#pragma unroll
+    for (int idx = threadIdx.x; idx < (N + 1) * R; idx += T) {
+        const int r = idx % R;
+        const int kx = idx / R;
+        const float2* line = zb + (r >> 1) * ZS;
+        const float2 zk = line[pz(kx)];
+        const float2 zm = line[pz((L - kx) & (L - 1))];
+        float2 o;
+        if ((r & 1) == 0) o = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+        else o = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+        S[(((size_t)kx * 3 + c) * g.nz + k) * g.Jst + j0 + r] = o;
+    }
+}
+
+// The same as a body with options.  RAG: a ragged sample, g.nx <= N cells per row and g.ny rows of a spectrum
 // row stride g.Jst (ny rounded up): cells past nx and rows past ny are zeros,
 // and the zero rows' spectra (up to Jst) are written like the others.
 // T: the block size (threads past the R G of the transforms only help with
 // the copies and the split).
-template <int N, int R, int T, bool RAG>
+template <int N, int R, int T, bool RAG, bool COMB = false>
 __device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float* __restrict__ M,
-                                           float2* __restrict__ S, float* __restrict__ Mcopy) {
+                                           float2* __restrict__ S, float* __restrict__ Mcopy,
+                                           const XComb& xc = XComb{}) {
     using F = Fft2<N>;
     constexpr int P = F::P, Q = F::Q, G = F::G, L = 2 * N, ZS = pzlen(2 * N);
     static_assert(T >= R * G, "block smaller than the tile's transform groups");
@@ -49,23 +118,26 @@ __device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float*
     const int k = b % g.nz;
     const int c = b / g.nz;
     const int j0 = jt * R;
+    if constexpr (RAG) {                  // the tables arrive while the rows are loaded
 #pragma unroll
-    for (int i = threadIdx.x; i < L; i += T) tw[i] = __ldg(g.twx + i);
-    if constexpr (RAG) {
+        for (int i = threadIdx.x; i < L; i += T) __pipeline_memcpy_async(tw + i, g.twx + i, sizeof(float2));
+        F::template load_ta<T>(ta, g.twx);
+        __pipeline_commit();
+    } else {
 #pragma unroll
-        for (int i = threadIdx.x; i < N; i += T) ta[i] = __ldg(g.twx + 2 * (i / Q) * (i % Q));
+        for (int i = threadIdx.x; i < L; i += T) tw[i] = __ldg(g.twx + i);
     }
     pdl_wait();                           // M and S may belong to the previous kernel
-    __syncthreads();
+    if constexpr (!RAG) __syncthreads();
 
     const int grp = threadIdx.x / G, t = threadIdx.x % G;
     const int p = grp >> 1, h = grp & 1;
     const bool act = T == R * G || grp < R;
-    if (act && t < Q) {
+    // the row pair's inputs, q = 0 .. P-1 at j = t + Q q (and the second copy)
+    auto load = [&](float2 (&v)[P]) {
         const float* ra = M + (size_t)c * g.N + ((size_t)k * g.ny + j0 + 2 * p) * nx;
         const float* rb = ra + nx;
         const int na = !RAG || j0 + 2 * p < g.ny ? nx : 0, nb = !RAG || j0 + 2 * p + 1 < g.ny ? nx : 0;
-        float2 v[P];
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             const int j = t + Q * q;
@@ -73,6 +145,15 @@ __device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float*
                 v[q] = make_float2(j < na ? __ldg(ra + j) : 0.f, j < nb ? __ldg(rb + j) : 0.f);
             else
                 v[q] = make_float2(__ldg(ra + j), __ldg(rb + j));
+        }
+        if constexpr (COMB) {                              // M + dt (w K), e.g. a stage state
+            const float* ka = xc.K + (ra - M);
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const int j = t + Q * q;
+                if (!RAG || j < na) v[q].x += xc.dt * (xc.w * __ldg(ka + j));
+                if (!RAG || j < nb) v[q].y += xc.dt * (xc.w * __ldg(ka + nx + j));
+            }
         }
         if (Mcopy && h == 0) {
             float* ca = Mcopy + (ra - M);
@@ -83,13 +164,21 @@ __device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float*
                 if (!RAG || j < nb) ca[nx + j] = v[q].y;
             }
         }
-        if constexpr (RAG) {
+    };
+    if constexpr (RAG) {
+        float2 v[P];
+        if (act && t < Q) load(v);
+        __pipeline_wait_prior(0);
+        __syncthreads();
+        if (act && t < Q) {
             if (h) F::odd_input_tab(v, t, tw);
             F::stepA_tab(v, t, ta, ex + grp * F::EX, false);
-        } else {
-            if (h) F::odd_input(v, t, tw);
-            F::stepA(v, t, tw, ex + grp * F::EX, false);
         }
+    } else if (act && t < Q) {
+        float2 v[P];
+        load(v);
+        if (h) F::odd_input(v, t, tw);
+        F::stepA(v, t, tw, ex + grp * F::EX, false);
     }
     __syncthreads();
     if (act && t < P) {
@@ -107,7 +196,7 @@ __device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float*
         if (RAG && j0 + r >= g.Jst) continue;
         const float2* line = zb + (r >> 1) * ZS;
         const float2 zk = line[pz(kx)];
-        const float2 zm = line[pz(kx == 0 ? 0 : L - kx)];
+        const float2 zm = line[pz(RAG ? (kx == 0 ? 0 : L - kx) : (L - kx) & (L - 1))];
         float2 o;
         if ((r & 1) == 0) o = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
         else o = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
@@ -115,10 +204,19 @@ __device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float*
     }
 }
 
+template <int N, int R>
+__global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_rag(Geom g, const float* __restrict__ M,
+                                                               float2* __restrict__ S, float* __restrict__ Mcopy) {
+    pass1_rows<N, R, R * Fft2<N>::G, true>(g, blockIdx.x, M, S, Mcopy);
+}
+
+// The same for M + dt (w K) (XComb), clearing *xc.zero.
 template <int N, int R, bool RAG = false>
-__global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const float* __restrict__ M,
-                                                                float2* __restrict__ S, float* __restrict__ Mcopy) {
-    pass1_rows<N, R, R * Fft2<N>::G, RAG>(g, blockIdx.x, M, S, Mcopy);
+__global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_comb(Geom g, const float* __restrict__ M,
+                                                                float2* __restrict__ S, float* __restrict__ Mcopy,
+                                                                XComb xc) {
+    pass1_rows<N, R, R * Fft2<N>::G, RAG, true>(g, blockIdx.x, M, S, Mcopy, xc);
+    if (xc.zero && blockIdx.x == 0 && threadIdx.x == 0) *xc.zero = 0;    // after the wait in pass1_rows
 }
 
 // ---------------------------------------------------------------- pass 2 --

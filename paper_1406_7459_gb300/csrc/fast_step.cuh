@@ -402,10 +402,35 @@ __device__ __forceinline__ void llg_rhs_fixed(const LlgCoef& cf, const float (&m
     f[2] = fmaf(cf.c1, p2, __fmul_rn(cf.c2, q2));
 }
 
+// a += sum_j w_j k_j of one cell.
+__device__ __forceinline__ void add_slopes(const StageArgs& st, size_t cell, size_t n, float (&a)[3]) {
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+        if (q < st.nk)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) a[c] = fmaf(st.w[q], __ldg(st.k[q] + c * n + cell), a[c]);
+}
+
+// Fold the block's largest e into *err: non-negative floats order like their
+// bit patterns; a NaN counts as infinite.
+template <int T> __device__ __forceinline__ void block_err_max(float e, unsigned* err) {
+    unsigned b = __float_as_uint(e != e ? __int_as_float(0x7f800000) : e);
+    const unsigned lanes = warp_lanes<T>();
+    b = __reduce_max_sync(lanes, b);
+    // most warps find a larger one there already and add no traffic
+    if ((threadIdx.x & 31) == 0 && b > *(volatile unsigned*)err) atomicMax(err, b);
+}
+
 // A thread's cells of a ragged x-step tile (its trips of the field loop):
 // M and the exchange field of Eq. (4), formed before the spectrum arrives.
 template <int CPT> struct RagCells {
     float m[CPT][3], ex[CPT][3];
+};
+
+// The same for a Heun or RK4 stage: the step's base state and the weighted
+// sum of the earlier slopes.
+template <int CPT> struct StageCells {
+    float p[CPT][3], a[CPT][3];
 };
 
 // MODE kModeStep: the Euler step (M^{n+1} replaces M^n in Mt and goes to
@@ -434,7 +459,9 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
                                            const float2* __restrict__ Sh, float2* __restrict__ Snext,
                                            float* __restrict__ Mout, int* __restrict__ flag,
                                            float* __restrict__ Mcopy = nullptr, const XTma& xt = XTma{},
-                                           const RagCells<(R * N + T - 1) / T>* rc = nullptr) {
+                                           const RagCells<(R * N + T - 1) / T>* rc = nullptr,
+                                           const StageArgs* st = nullptr,
+                                           const StageCells<(R * N + T - 1) / T>* sc = nullptr) {
     using Lay = XstepLayout<N, R>;
     using F = Fft2<N>;
     constexpr int P = F::P, Q = F::Q, G = F::G, L = Lay::L, H = Lay::H, NL = Lay::NL, ZS = Lay::ZS;
@@ -547,11 +574,11 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
     // The spectrum carries the zero-padded exchange stencil; a cell on a
     // free face lacks that neighbour, whose term in Eq. (4) is M(i) itself
     // (zero change), so each missing neighbour adds pexch M(i) / delta^2.
+    float emax = 0.f;                                      // kModeErr
     const float bz = cf.pexch * (float)((g.nz > 1) * ((k == 0) + (k == g.nz - 1))) * cf.idz2;
+    int u = 0;                                             // trip: the index into rc and sc
 #pragma unroll
-    for (int u = 0; u < (R * N + T - 1) / T; ++u) {
-        const int idx = u * T + threadIdx.x;
-        if (R * N % T != 0 && idx >= R * N) break;
+    for (int idx = threadIdx.x; idx < R * N; idx += T, ++u) {
         const int r = idx / N;
         const int i = idx % N;
         const int j = j0 + r;
@@ -599,7 +626,47 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
             continue;
         }
         float o0, o1, o2;
-        if constexpr (RAG) {
+        if constexpr (MODE == kModeErr) {
+            float f[3];
+            llg_rhs_fixed(cf, m, hh, f);
+            float d[3];
+#pragma unroll
+            for (int cc = 0; cc < 3; ++cc) {
+                st->kout[cc * Nc + cell] = f[cc];
+                d[cc] = __fmul_rn(st->wf, f[cc]);
+            }
+            add_slopes(*st, (size_t)cell, (size_t)Nc, d);
+            const float e = fabsf(cf.dt) * sqrtf(fmaf(d[2], d[2], fmaf(d[1], d[1], __fmul_rn(d[0], d[0])))) / cf.Ms;
+            emax = (e > emax || e != e) ? e : emax;        // a NaN wins (it fails the step)
+            continue;
+        } else if constexpr (MODE == kModeStage) {
+            float f[3], n[3];
+            llg_rhs_fixed(cf, m, hh, f);
+            if (st->acc) {
+#pragma unroll
+                for (int cc = 0; cc < 3; ++cc) {
+                    const float a = fmaf(st->wf, f[cc], sc->a[u][cc]);
+                    if (!st->last) st->acc[cc * Nc + cell] = a;
+                    n[cc] = st->last ? fmaf(cf.dt, a, sc->p[u][cc]) : fmaf(st->s, f[cc], sc->p[u][cc]);
+                }
+            } else {
+                float a[3];
+#pragma unroll
+                for (int cc = 0; cc < 3; ++cc) {
+                    st->kout[cc * Nc + cell] = f[cc];
+                    a[cc] = __fmul_rn(st->wf, f[cc]);
+                }
+                add_slopes(*st, (size_t)cell, (size_t)Nc, a);
+#pragma unroll
+                for (int cc = 0; cc < 3; ++cc) n[cc] = fmaf(cf.dt, a[cc], __ldg(st->base + cc * Nc + cell));
+            }
+            const float s =
+                st->last ? cf.Ms / sqrtf(fmaf(n[2], n[2], fmaf(n[1], n[1], __fmul_rn(n[0], n[0])))) : 1.f;
+            o0 = __fmul_rn(n[0], s);
+            o1 = __fmul_rn(n[1], s);
+            o2 = __fmul_rn(n[2], s);
+            if (st->last && st->flag && !isfinite(o0 + o1 + o2)) atomicOr(st->flag, kFlagNonFinite);
+        } else if constexpr (RAG) {
             float f[3];
             llg_rhs_fixed(cf, m, hh, f);
             const float n0 = fmaf(cf.dt, f[0], m[0]), n1 = fmaf(cf.dt, f[1], m[1]), n2 = fmaf(cf.dt, f[2], m[2]);
@@ -622,7 +689,7 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
             o1 = n1 * s;
             o2 = n2 * s;
         }
-        if (!isfinite(o0 + o1 + o2)) atomicOr(flag, kFlagNonFinite);   // |o| <= Ms when finite
+        if (MODE == kModeStep && !isfinite(o0 + o1 + o2)) atomicOr(flag, kFlagNonFinite);   // |o| <= Ms when finite
         if (Mout) {
             Mout[cell] = o0;
             Mout[Nc + cell] = o1;
@@ -638,8 +705,9 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
         Mt[(1 * R + r) * N + i] = o1;
         Mt[(2 * R + r) * N + i] = o2;
     }
+    if constexpr (MODE == kModeErr) block_err_max<T>(emax, st->err);
     __syncthreads();
-    if constexpr (MODE == kModeStep) {
+    if constexpr (MODE == kModeStep || MODE == kModeStage) {
         // ---- forward x of the new rows (first pass of the next step)
         if (fft_thread && t < Q) {
             const float* ra = Mt + (size_t)(lc * R + 2 * pr) * N;
@@ -731,6 +799,35 @@ __device__ __forceinline__ void load_rag_cells(const Geom& g, const LlgCoef& cf,
     }
 }
 
+// Heun and RK4: a thread's base states and slope sums of a stage tile, in
+// registers; both were written at least two launches ago, so the loads run
+// before the wait (256x256x4 per RK4 step: 70 us so, 83 with them in the
+// field loop).  Dormand-Prince stages read up to five slopes per cell and
+// load them in the field loop (128x128x4 adaptive run: 432 us so, 499 with
+// them here).
+template <int N, int R, int T, bool RAG>
+__device__ __forceinline__ void load_stage_cells(const Geom& g, const StageArgs& st, int tile,
+                                                 StageCells<(R * N + T - 1) / T>& sc) {
+    if (!st.acc) return;
+    const int ntj = (RAG ? g.Jst : g.ny) / R;
+    const int k = tile / ntj, j0 = (tile % ntj) * R;
+    const int nx = RAG ? g.nx : N, Nc = g.N;
+#pragma unroll
+    for (int u = 0; u < (R * N + T - 1) / T; ++u) {
+        const int idx = u * T + threadIdx.x;
+        if (R * N % T != 0 && idx >= R * N) break;
+        const int r = idx / N, i = idx % N, j = j0 + r;
+        if (RAG && (i >= nx || j >= g.ny)) continue;
+        const int cell = i + nx * (j + g.ny * k);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const size_t e = (size_t)c * Nc + cell;
+            sc.p[u][c] = __ldg(st.base + e);
+            sc.a[u][c] = st.first ? 0.f : st.acc[e];
+        }
+    }
+}
+
 // Fill the tile's M^n rows (floats [c][row][i]) with 16-byte asynchronous
 // copies (committed with the caller's next group).
 template <int N, int R, int T>
@@ -786,6 +883,40 @@ __global__ void __launch_bounds__(XstepLayout<N, R>::THREADS)
     __pipeline_commit();
     pdl_wait();
     xstep_body<N, R, MODE, T>(g, cf, blockIdx.x, tw, ta, Mt, sb, wk, Sh, Snext, Mout, flag, Mcopy);
+    __syncthreads();
+    pdl_trigger();
+}
+
+// K_B for a Runge-Kutta stage (StageArgs): the field at the stage state Y, its
+// slope, the next stage state and that state's x spectrum, so that a stage
+// is the plane kernel and this one.  The next state goes to another buffer
+// than Y (a ragged tile reads its neighbours' rows of Y).
+template <int N, int R, int MODE, bool RAG = false>
+__global__ void __launch_bounds__(XstepLayout<N, R>::THREADS)
+    k_xstep_stage(const __grid_constant__ Geom g, const __grid_constant__ LlgCoef cf, const float2* __restrict__ Sh,
+                  float2* __restrict__ Snext, const float* __restrict__ Y, const __grid_constant__ StageArgs st) {
+    using Lay = XstepLayout<N, R>;
+    using F = Fft2<N>;
+    constexpr int L = Lay::L;
+    constexpr int T = Lay::THREADS;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm + Lay::TW_OFF;
+    float2* ta = sm + Lay::TA_OFF;
+    float* Mt = reinterpret_cast<float*>(sm + Lay::MT_OFF);
+    float2* sb = sm + Lay::SB_OFF;
+    float2* wk = sm + Lay::W_OFF;
+#pragma unroll
+    for (int i = threadIdx.x; i < L / 2; i += T) copy16(tw + 2 * i, g.twx + 2 * i);
+    F::template load_ta<T>(ta, g.twx);
+    RagCells<(R * N + T - 1) / T> rc;
+    if constexpr (!RAG) load_mtile<N, R, T>(g, blockIdx.x, Y, Mt);
+    __pipeline_commit();
+    if constexpr (RAG) load_rag_cells<N, R, T>(g, cf, blockIdx.x, Y, Mt, rc);
+    StageCells<(R * N + T - 1) / T> sc;
+    if constexpr (MODE == kModeStage) load_stage_cells<N, R, T, RAG>(g, st, blockIdx.x, sc);
+    pdl_wait();
+    xstep_body<N, R, MODE, T, RAG>(g, cf, blockIdx.x, tw, ta, Mt, sb, wk, Sh, Snext, st.out, st.flag, nullptr, XTma{},
+                                   &rc, &st, &sc);
     __syncthreads();
     pdl_trigger();
 }

@@ -15,6 +15,8 @@ static void fill_xstep(FastStepFns* f) {
     f->kb[kModeDemag] = k_xstep_pdl<N, R, kModeDemag>;
     f->kb[kModeHeff] = k_xstep_pdl<N, R, kModeHeff>;
     f->kb[kModeStep] = k_xstep_pdl<N, R, kModeStep>;
+    f->kst[0] = k_xstep_stage<N, R, kModeStage>;
+    f->kst[1] = k_xstep_stage<N, R, kModeErr>;
     if constexpr (XstepLayout<N, R>::HM <= 256) {      // the box's kx / 2 extent
         f->kbt[kModeDemag] = k_xstep_tma<N, R, kModeDemag>;
         f->kbt[kModeHeff] = k_xstep_tma<N, R, kModeHeff>;
@@ -59,6 +61,10 @@ cudaError_t configure_step_kernels(const FastStepFns& f) {
                          : cudaSuccess;                   // x-step only (thick samples)
     if (e == cudaSuccess && f.p1)
         e = cudaFuncSetAttribute(f.p1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.s1);
+    if (e == cudaSuccess && f.p1c)
+        e = cudaFuncSetAttribute(f.p1c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.s1);
+    for (int m = 0; m < 2 && e == cudaSuccess; ++m)
+        e = cudaFuncSetAttribute(f.kst[m], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.sb);
     for (int m = 0; m < 3 && e == cudaSuccess; ++m) {
         e = cudaFuncSetAttribute(f.kb[m], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.sb);
         if (e == cudaSuccess && f.kbt[m])
@@ -134,6 +140,13 @@ cudaError_t launch_step_b(const Geom& g, const FastStepFns& f, const LlgCoef& c,
         return cudaLaunchKernelEx(&cfg, f.kbt[kModeStep], g, c, Sh, S, M, Mout, flag, Mcopy, f.tin, f.tout,
                                   f.tma_use);
     return cudaLaunchKernelEx(&cfg, f.kb[kModeStep], g, c, Sh, S, M, Mout, flag, Mcopy);
+}
+
+cudaError_t launch_stage_x(const Geom& g, int tiles, const FastStepFns& f, const LlgCoef& c, int mode,
+                           const float2* Sp, float2* S, const float* Y, const StageArgs& st, cudaStream_t s) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = launch_config(dim3(tiles), f.tb, f.sb, s, attr);
+    return cudaLaunchKernelEx(&cfg, f.kst[mode == kModeErr ? 1 : 0], g, c, Sp, S, Y, st);
 }
 
 cudaError_t launch_field_pdl(const Geom& g, const FastStepFns& f, const LlgCoef& c, int mode, const float* Kd,

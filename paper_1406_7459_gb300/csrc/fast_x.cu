@@ -8,6 +8,7 @@ template <int N>
 static void fill_x(FastFns* f) {
     constexpr int R1 = 8, R3 = 2;
     f->p1 = k_pass1_fast<N, R1>;
+    f->p1c = k_pass1_comb<N, R1>;
     f->r1 = R1;
     f->t1 = R1 * Fft2<N>::G;
     f->s1 = pass1_fast_smem<N, R1>();

@@ -253,6 +253,7 @@ static void release(mm_ctx* c) {
     cudaFree(c->Sh);
     for (int q = 0; q < 7; ++q) cudaFree(c->dpk[q]);
     cudaFree(c->dperr);
+    cudaFreeHost(c->hperr);
     cudaFree(c->Mbuf[0]);
     cudaFree(c->Mbuf[1]);
     cudaFree(c->H);
@@ -485,9 +486,21 @@ extern "C" int mm_get_m(mm_ctx* c, float* M) {
 
 // x R2C of M into the spectrum workspace S; Mcopy (has_fs, may be null): also
 // copy M there.
-static cudaError_t form_spectrum(mm_ctx* c, const float* M, cudaStream_t s, float* Mcopy = nullptr) {
-    if (c->rag) return launch_ragged_pass1(c->gf, c->fs, M, c->S, s, Mcopy);
-    return launch_pass1(c->g, c->l, M, c->S, s, Mcopy);
+cudaError_t mmk::form_spectrum(mm_ctx* c, const float* M, cudaStream_t s, float* Mcopy, const XComb& comb) {
+    if (c->rag) return launch_ragged_pass1(c->gf, c->fs, M, c->S, s, Mcopy, comb);
+    return launch_pass1(c->g, c->l, M, c->S, s, Mcopy, comb);
+}
+
+int mmk::fused_stage(mm_ctx* c, int mode, const float* Y, const StageArgs& st, const LlgCoef& cf, cudaStream_t s) {
+    if (c->has_fs) {
+        const Geom& g = c->gf;
+        CU(launch_step_a(g, c->fs, g.Kd, c->S, c->Sh, c->flag, s, true, c->fs.early));
+        CU(launch_stage_x(g, g.nz * (g.Jst / c->fs.rb), c->fs, cf, mode, c->Sh, c->S, Y, st, s));
+    } else {
+        CU(launch_fast_split(c->g, c->fsplit, c->Kt_ex, c->S, s));
+        CU(launch_stage_x(c->g, c->g.nz * (c->g.ny / c->fs.rb), c->fs, cf, mode, c->S, c->S, Y, st, s));
+    }
+    return MM_OK;
 }
 
 // The three-pass evaluation on the spectrum workspace S (which also holds
@@ -542,6 +555,26 @@ static int enqueue_rk_step(mm_ctx* c, int p, double dt, cudaStream_t s) {
     const float* av = ns == 2 ? heun_a : rk4_a;
     const float* bv = ns == 2 ? heun_b : rk4_b;
     const LlgCoef cf = make_coef(c, dt);
+    if (fused_stages(c)) {
+        // S holds the x spectrum of M[p]; every stage leaves the next
+        // state's, the last one M[1 - p]'s.  The stage states alternate
+        // between two buffers (H is free here).
+        for (int q = 0; q < ns; ++q) {
+            StageArgs st{};
+            st.base = c->Mbuf[p];
+            st.acc = c->acc;
+            st.wf = bv[q];
+            st.s = av[q] * cf.dt;
+            st.first = q == 0;
+            st.last = q == ns - 1;
+            st.out = st.last ? c->Mbuf[1 - p] : (q & 1 ? c->H : c->Mst);
+            st.flag = c->flag;
+            const float* Y = q == 0 ? c->Mbuf[p] : (q & 1 ? c->Mst : c->H);
+            int rc = fused_stage(c, kModeStage, Y, st, cf, s);
+            if (rc != MM_OK) return rc;
+        }
+        return MM_OK;
+    }
     for (int st = 0; st < ns; ++st) {
         const float* Min = st == 0 ? c->Mbuf[p] : c->Mst;
         int rc = run_passes(c, kModeHeff, Min, c->H, dt, s);
@@ -609,7 +642,8 @@ static int capture_step(mm_ctx* c, int kind, int p, double dt) {
 
 // Form S[cur] from M[cur] when the two-kernel step needs it.
 static int ensure_spectrum(mm_ctx* c) {
-    if (!(c->has_fs || c->has_ss || c->has_gx) || c->spec_valid || c->method != MM_INTEGRATOR_EULER) return MM_OK;
+    const bool reads = c->method == MM_INTEGRATOR_EULER ? c->has_fs || c->has_ss || c->has_gx : fused_stages(c);
+    if (c->spec_valid || !reads) return MM_OK;
     CU(form_spectrum(c, c->Mbuf[c->cur], c->stream));
     c->spec_valid = true;
     return MM_OK;

@@ -77,6 +77,14 @@ struct LlgCoef {
     float dt;
 };
 
+// Row transforms of M + dt (w K) instead of M (K null: M itself), clearing
+// the error estimate *zero.
+struct XComb {
+    const float* K = nullptr;
+    float w = 0.f, dt = 0.f;
+    unsigned* zero = nullptr;
+};
+
 struct FastFns;
 struct FastSplitFns;
 
@@ -94,7 +102,30 @@ struct Launch {
 
 // kModeStepX (generic kernels only): the Euler step followed by the forward
 // x R2C of the new rows into S, the first pass of the next step.
-enum Pass3Mode { kModeDemag = 0, kModeHeff = 1, kModeStep = 2, kModeStepX = 3 };
+// kModeStage, kModeErr (x-step kernels only): a Runge-Kutta stage's field,
+// slope and update followed by the forward x R2C of the next stage state;
+// the last slope of a Dormand-Prince step with its error estimate.
+enum Pass3Mode { kModeDemag = 0, kModeHeff = 1, kModeStep = 2, kModeStepX = 3, kModeStage = 4, kModeErr = 5 };
+
+// What a stage does with its slope f = f(Y) (each pointer 3 N floats).
+//   acc set (Heun, RK4): a = wf f (+ acc unless first); the next state is
+//     base + s f, or on the last stage base + dt a renormalised to Ms.
+//   else (Dormand-Prince): f -> kout; a = wf f + sum_j w_j k_j; the next
+//     state is base + dt a, renormalised when last; kModeErr: err = max over
+//     cells of |dt a| / Ms, folded into *err.
+struct StageArgs {
+    const float* base;
+    float* acc;
+    float* kout;
+    const float* k[6];
+    float w[6];
+    int nk;
+    float s, wf;
+    int first, last;
+    float* out;
+    int* flag;                 // non-finite new state (null: not reported)
+    unsigned* err;
+};
 
 // Planning helpers (mm_api.cu), shared with the batched driver.
 int plan_padded_length(int n);
@@ -106,7 +137,7 @@ int set_error(int code, const char* msg);
 // Launchers (demag_passes.cu).  All asynchronous on `s`.
 // Mcopy (compile-time x passes only, may be null): also copy M there.
 cudaError_t launch_pass1(const Geom& g, const Launch& l, const float* M, float2* S, cudaStream_t s,
-                         float* Mcopy = nullptr);
+                         float* Mcopy = nullptr, const XComb& comb = XComb{});
 cudaError_t launch_plane(const Geom& g, const Launch& l, float2* S, cudaStream_t s);
 cudaError_t launch_pass3(const Geom& g, const Launch& l, const LlgCoef& c, int mode, const float2* S,
                          const float* M, float* out, int* flag, cudaStream_t s);
@@ -119,6 +150,7 @@ PlaneFn plane_fn_mid(int Lz);     // plane_mid.cu
 // Compile-time specialised kernels for power-of-two grids (fast_*.cu).
 struct FastFns {
     void (*p1)(Geom, const float*, float2*, float*) = nullptr;
+    void (*p1c)(Geom, const float*, float2*, float*, XComb) = nullptr;
     int r1 = 0, t1 = 0;
     size_t s1 = 0;
     void (*pl)(Geom, float2*) = nullptr;
@@ -166,10 +198,13 @@ struct FastStepFns {
     // `tma_use` (mm_set_tiled_copies) are set
     void (*kbt[3])(Geom, LlgCoef, const float2*, float2*, const float*, float*, int*, float*, CUtensorMap,
                    CUtensorMap, int) = {nullptr, nullptr, nullptr};
+    // stage kernels: [0] kModeStage, [1] kModeErr
+    void (*kst[2])(Geom, LlgCoef, const float2*, float2*, const float*, StageArgs) = {nullptr, nullptr};
     int rb = 0, tb = 0;
     size_t sb = 0;
     // ragged films: their row transform (the exact sizes use FastFns::p1)
     void (*p1)(Geom, const float*, float2*, float*) = nullptr;
+    void (*p1c)(Geom, const float*, float2*, float*, XComb) = nullptr;
     int r1 = 0, t1 = 0;
     size_t s1 = 0;
     bool tma = false;
@@ -195,7 +230,11 @@ bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY);
 bool ragged_batchable(int nx, int ny, int nz);
 int ragged_early_trigger(const Geom& g, const FastStepFns& f, int sms);
 cudaError_t launch_ragged_pass1(const Geom& g, const FastStepFns& f, const float* M, float2* S, cudaStream_t s,
-                                float* Mcopy = nullptr);
+                                float* Mcopy = nullptr, const XComb& comb = XComb{});
+// The x-step kernel of stage mode `mode` after the plane pass (from Sp into S,
+// which may be the same buffer).
+cudaError_t launch_stage_x(const Geom& g, int tiles, const FastStepFns& f, const LlgCoef& c, int mode,
+                           const float2* Sp, float2* S, const float* Y, const StageArgs& st, cudaStream_t s);
 // K_A reads the x half-spectrum S and writes its output to Sh; K_B reads Sh
 // and writes the next step's S.
 cudaError_t launch_step_pdl(const Geom& g, const FastStepFns& f, const LlgCoef& c, float2* S, float2* Sh,

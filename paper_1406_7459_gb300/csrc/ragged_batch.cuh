@@ -135,7 +135,7 @@ __device__ __forceinline__ void rag_xstep_tile(const RagDesc& d, int tile, int p
 }
 
 // Row transform of 4 rows (tile) of M[par] into S, one row group per tile
-// as in k_pass1_fast<N, 4, true>.
+// as in k_pass1_rag<N, 4>.
 constexpr int kRagRows1 = 4;
 template <int N, int T>
 __device__ __forceinline__ void rag_pass1_tile(const RagDesc& d, int tile, int par) {

@@ -44,20 +44,23 @@ bool ragged_batchable(int nx, int ny, int nz) {
 }
 
 // The plane kernel's trigger (fast_step.cuh), per L2-resident step, early
-// against late: where the x tiles cover the SMs early wins (250x250x4 18.9
-// against 20.2 us, 600x400x1 28.5 against 30.6, 50x200x2 6.9 against 7.2), as
-// it does where planes and tiles together leave each SM one block (30x30x1
-// 4.4 against 4.9); in between the early tiles share a few SMs with planes
-// and hold those up (200x60x3 12.3 against 9.6, 100x100x1 7.1 against 6.7).
+// against late.  Early wins where the x tiles cover the SMs (250x250x4 18.9
+// against 20.2 us, 300x300x3 42.5 against 44.2), where the planes do so
+// evenly, several to each (600x400x1 28.5 against 30.7, 700x64x1 17.9 against
+// 19.5, 400x300x2 33.2 against 33.7), and where planes and tiles together
+// leave each SM one block (30x30x1 4.4 against 4.9).  In between the early
+// tiles crowd onto the SMs with fewer planes (200x60x3 12.3 against 9.6,
+// 100x100x1 7.1 against 6.7).
 int ragged_early_trigger(const Geom& g, const FastStepFns& f, int sms) {
     const int tiles = g.nz * (g.Jst / f.rb);
-    return tiles >= sms || tiles + g.Hx <= sms;
+    return tiles >= sms || g.Hx >= 3 * sms || tiles + g.Hx <= sms;
 }
 
 cudaError_t launch_ragged_pass1(const Geom& g, const FastStepFns& f, const float* M, float2* S, cudaStream_t s,
-                                float* Mcopy) {
+                                float* Mcopy, const XComb& comb) {
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = launch_config(dim3(3 * g.nz * ((g.Jst + f.r1 - 1) / f.r1)), f.t1, f.s1, s, attr);
+    if (comb.K) return cudaLaunchKernelEx(&cfg, f.p1c, g, M, S, Mcopy, comb);
     return cudaLaunchKernelEx(&cfg, f.p1, g, M, S, Mcopy);
 }
 

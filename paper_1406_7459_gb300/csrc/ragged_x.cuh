@@ -19,11 +19,14 @@ template <int N> void rag_fill_x(FastStepFns* f) {
     f->kb[kModeDemag] = k_xstep_pdl<N, R, kModeDemag, true>;
     f->kb[kModeHeff] = k_xstep_pdl<N, R, kModeHeff, true>;
     f->kb[kModeStep] = k_xstep_pdl<N, R, kModeStep, true>;
+    f->kst[0] = k_xstep_stage<N, R, kModeStage, true>;
+    f->kst[1] = k_xstep_stage<N, R, kModeErr, true>;
     f->rb = R;
     f->tb = XstepLayout<N, R>::THREADS;
     f->sb = XstepLayout<N, R>::BYTES;
     constexpr int R1 = 4;                     // small tiles: a run's first transform is one wave
-    f->p1 = k_pass1_fast<N, R1, true>;
+    f->p1 = k_pass1_rag<N, R1>;
+    f->p1c = k_pass1_comb<N, R1, true>;
     f->r1 = R1;
     f->t1 = R1 * Fft2<N>::G;
     f->s1 = pass1_fast_smem<N, R1, true>();
