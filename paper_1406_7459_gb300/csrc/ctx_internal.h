@@ -58,10 +58,11 @@ struct mm_ctx {
     FastStepFns fs;            // two-kernel step (power-of-two grids)
     FastSplitFns fsplit;       // compile-time split pass 2 (thick power-of-two samples)
     bool has_fs = false;
-    bool rag = false;          // has_fs through the ragged kernels; Kt is formed on demand
+    bool rag = false;          // has_fs or has_ss through the ragged kernels; Kt is formed on demand
     bool has_ss = false;       // thick power-of-two samples: split pass 2 + the x-step kernel
     bool has_gx = false;       // generic x passes: the step's pass 3 also forms the next x spectrum
-    float* Kt_ex = nullptr;    // tensor spectrum with the exchange stencil folded in (has_ss)
+    float* Kt_ex = nullptr;    // has_ss: tensor spectrum with the exchange stencil folded in (ragged: plain,
+                               // on the carrier lengths)
     float2* Sh = nullptr;      // plane-kernel output of the two-kernel step (layout of S)
     int method = MM_INTEGRATOR_EULER;
     float* Mst = nullptr;      // Runge-Kutta stage state
@@ -92,7 +93,7 @@ cudaError_t form_spectrum(mm_ctx* c, const float* M, cudaStream_t s, float* Mcop
 // Not where the plane kernel runs more than 512 threads (512x512x4: 472 us per
 // RK4 step fused, 440 with the three-pass field evaluations).
 inline bool fused_stages(const mm_ctx* c) {
-    return c->has_fs ? c->rag || c->fs.ta <= 512 : c->has_ss && c->l.fx;
+    return c->has_fs ? c->rag || c->fs.ta <= 512 : c->has_ss && (c->rag || c->l.fx);
 }
 // One stage at the state Y whose x spectrum is in S: the slope's use per st
 // (mode kModeStage, which leaves the next state's spectrum in S, or kModeErr).

@@ -122,6 +122,7 @@ template <> __device__ __forceinline__ void dftp<24>(float2* a) { dft_ab<8, 3>(a
 // the powers of two (ragged samples, film_ragged) keep P even and the group
 // of max(P, Q) threads within 8, 16 or 32 lanes (Fft2::G).
 template <int N> struct Split;
+template <> struct Split<24> { static constexpr int P = 8, Q = 3; };
 template <> struct Split<48> { static constexpr int P = 8, Q = 6; };
 template <> struct Split<96> { static constexpr int P = 16, Q = 6; };
 template <> struct Split<192> { static constexpr int P = 16, Q = 12; };

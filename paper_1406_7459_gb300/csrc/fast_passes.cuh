@@ -93,9 +93,9 @@ __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const flo
     }
 }
 
-// The same as a body with options.  RAG: a ragged sample, g.nx <= N cells per row and g.ny rows of a spectrum
-// row stride g.Jst (ny rounded up): cells past nx and rows past ny are zeros,
-// and the zero rows' spectra (up to Jst) are written like the others.
+// The same as a body with options.  RAG: a ragged sample, g.nx <= N cells per row and g.ny rows of the g.Jr of
+// the spectrum: cells past nx and rows past ny are zeros,
+// and the zero rows' spectra (up to Jr) are written like the others.
 // T: the block size (threads past the R G of the transforms only help with
 // the copies and the split).
 template <int N, int R, int T, bool RAG, bool COMB = false>
@@ -110,7 +110,7 @@ __device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float*
     float2* ta = tw + L;                  // RAG: every twiddle from a table, rounded once (N entries)
     float2* ex = tw + L + (RAG ? N : 0);
     float2* zb = ex + R * F::EX;
-    const int ntj = RAG ? (g.Jst + R - 1) / R : g.ny / R;
+    const int ntj = RAG ? (g.Jr + R - 1) / R : g.ny / R;
     const int nx = RAG ? g.nx : N;
     int b = tile;
     const int jt = b % ntj;
@@ -193,7 +193,7 @@ __device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float*
     for (int idx = threadIdx.x; idx < (N + 1) * R; idx += T) {
         const int r = idx % R;
         const int kx = idx / R;
-        if (RAG && j0 + r >= g.Jst) continue;
+        if (RAG && j0 + r >= g.Jr) continue;
         const float2* line = zb + (r >> 1) * ZS;
         const float2 zk = line[pz(kx)];
         const float2 zm = line[pz(RAG ? (kx == 0 ? 0 : L - kx) : (L - kx) & (L - 1))];

@@ -446,7 +446,7 @@ template <int CPT> struct StageCells {
 // 16-byte asynchronous copies of this thread (the gather below waits for
 // all of them).  sb stages the tile's rows of Sh, wk the transforms.
 //
-// RAG: a ragged sample of g.nx <= N cells per row and g.Jst (a multiple of
+// RAG: a ragged sample of g.nx <= N cells per row and g.Jr (a multiple of
 // R) rows of spectrum of which g.ny are the sample's; Mt is zero past both
 // and M^n itself comes in rc (load_rag_cells).
 // The exchange stays the stencil of Eq. (4), as on the general path (the
@@ -468,7 +468,7 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
     constexpr int HM = Lay::HM, HP = Lay::HP, HOFF = Lay::HOFF;
     constexpr int RP = R / 2;                             // row pairs of the tile
     static_assert(T >= 2 * NL * G, "block smaller than the tile's transform groups");
-    const int ntj = (RAG ? g.Jst : g.ny) / R;
+    const int ntj = (RAG ? g.Jr : g.ny) / R;
     const int nx = RAG ? g.nx : N;
     const int jt = tile % ntj;
     const int k = tile / ntj;
@@ -767,7 +767,7 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
 template <int N, int R, int T>
 __device__ __forceinline__ void load_rag_cells(const Geom& g, const LlgCoef& cf, int tile, const float* __restrict__ M,
                                                float* Mt, RagCells<(R * N + T - 1) / T>& rc) {
-    const int ntj = g.Jst / R;
+    const int ntj = g.Jr / R;
     const int k = tile / ntj, j0 = (tile % ntj) * R;
     const int nx = g.nx, Nc = g.N, plane_xy = nx * g.ny;
 #pragma unroll
@@ -809,7 +809,7 @@ template <int N, int R, int T, bool RAG>
 __device__ __forceinline__ void load_stage_cells(const Geom& g, const StageArgs& st, int tile,
                                                  StageCells<(R * N + T - 1) / T>& sc) {
     if (!st.acc) return;
-    const int ntj = (RAG ? g.Jst : g.ny) / R;
+    const int ntj = (RAG ? g.Jr : g.ny) / R;
     const int k = tile / ntj, j0 = (tile % ntj) * R;
     const int nx = RAG ? g.nx : N, Nc = g.N;
 #pragma unroll

@@ -135,7 +135,7 @@ cudaError_t launch_step_a(const Geom& g, const FastStepFns& f, const float* Kd, 
 cudaError_t launch_step_b(const Geom& g, const FastStepFns& f, const LlgCoef& c, const float2* Sh, float2* S,
                           const float* M, float* Mout, int* flag, cudaStream_t s, bool pdl, float* Mcopy) {
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = launch_config(dim3(g.nz * (g.Jst / f.rb)), f.tb, f.sb, s, attr, pdl);
+    cudaLaunchConfig_t cfg = launch_config(dim3(g.nz * (g.Jr / f.rb)), f.tb, f.sb, s, attr, pdl);
     if (f.tma && f.tma_use && Sh == f.tin_buf && S == f.tout_buf)
         return cudaLaunchKernelEx(&cfg, f.kbt[kModeStep], g, c, Sh, S, M, Mout, flag, Mcopy, f.tin, f.tout,
                                   f.tma_use);
@@ -154,7 +154,7 @@ cudaError_t launch_field_pdl(const Geom& g, const FastStepFns& f, const LlgCoef&
     cudaError_t e = launch_step_a(g, f, Kd, S, Sh, flag, s, true, 0);   // late: measured faster here
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = launch_config(dim3(g.nz * (g.Jst / f.rb)), f.tb, f.sb, s, attr, true);
+    cudaLaunchConfig_t cfg = launch_config(dim3(g.nz * (g.Jr / f.rb)), f.tb, f.sb, s, attr, true);
     if (f.tma && f.tma_use && Sh == f.tin_buf)
         return cudaLaunchKernelEx(&cfg, f.kbt[mode], g, c, (const float2*)Sh, (float2*)nullptr, M, out, flag,
                                   (float*)nullptr, f.tin, f.tout, f.tma_use);

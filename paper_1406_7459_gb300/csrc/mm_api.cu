@@ -83,9 +83,35 @@ static bool plan_ragged(mm_ctx* c) {
     f.Hy = NY + 1;
     f.Hz = 1;
     f.Jst = jst;
+    f.Jr = jst;
     // the x-step kernel indexes the spectrum and M with 32-bit offsets
     if (!(3.0 * f.Hx * f.nz * f.Jst < (double)INT_MAX && 3.0 * f.N < (double)INT_MAX)) return false;
     c->fs = fs;
+    return true;
+}
+
+// Ragged thick samples (or films whose planes exceed shared memory): the
+// split pass and the x-step kernel on carrier lengths, in place on S.
+static bool plan_ragged_split(mm_ctx* c) {
+    const Geom& g = c->g;
+    FastStepFns fs;
+    FastSplitFns sp;
+    int NX = 0, NY = 0, NZ = 0;
+    if (!ragged_split_lookup(g.ny, g.nz, &sp, &NY, &NZ) || !ragged_lookup_x(g.nx, &fs, &NX)) return false;
+    Geom f = g;
+    f.Lx = 2 * NX;
+    f.Ly = 2 * NY;
+    f.Lz = NZ == 1 ? 1 : 2 * NZ;
+    f.Hx = NX + 1;
+    f.Hy = NY + 1;
+    f.Hz = f.Lz / 2 + 1;
+    f.Jst = f.Ly;                             // a line holds its y spectrum
+    f.Jr = (g.ny + 3) & ~3;
+    if (!(3.0 * f.Hx * f.nz * f.Jst < (double)INT_MAX && 3.0 * f.N < (double)INT_MAX)) return false;
+    c->gf = f;
+    c->fs = fs;
+    c->fs.ka = nullptr;
+    c->fsplit = sp;
     return true;
 }
 
@@ -105,6 +131,7 @@ static int build_plan(mm_ctx* c) {
     g.Hy = g.Ly / 2 + 1;
     g.Hz = g.Lz / 2 + 1;
     g.Jst = g.ny;
+    g.Jr = g.ny;
     if (!make_axis_plan(g.Lx, &g.px) || !make_axis_plan(g.Ly, &g.py) || !make_axis_plan(g.Lz, &g.pz))
         return fail(MM_EUNSUPPORTED, "no radix plan for padded lengths %d %d %d", g.Lx, g.Ly, g.Lz);
 
@@ -197,6 +224,9 @@ static int build_plan(mm_ctx* c) {
     if (c->rag) {
         c->has_fs = true;
         c->has_persist = false;
+    } else if (allow_fast && !c->has_fs && !c->has_ss) {
+        c->gf = g;
+        c->rag = c->has_ss = plan_ragged_split(c);
     }
     if (!c->has_fs && !c->has_ss && !l.fx) {
         c->has_gx = true;
@@ -322,11 +352,11 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
             CU(cudaMalloc(&c->Sh, sizeof(float2) * nS));
             CU(cudaMemset(c->S + (size_t)gf.Hx * plane, 0, sizeof(float2) * plane));
             CU(cudaMemset(c->Sh + (size_t)gf.Hx * plane, 0, sizeof(float2) * plane));
-            // ragged films keep the exchange stencil: no folded spectrum
+            // ragged samples keep the exchange stencil: no folded spectrum
             if (!c->rag) CU(cudaMalloc(&c->Kd, sizeof(float) * 6 * (size_t)gf.Hx * kd_row(gf.Hy) * gf.nz));
             CU(cudaMalloc(&c->Kd0, sizeof(float) * 6 * (size_t)gf.Hx * kd_row(gf.Hy) * gf.nz));
         }
-        if (c->has_ss) CU(cudaMalloc(&c->Kt_ex, sizeof(float) * 6 * (size_t)g.Hx * g.Hy * g.Hz));
+        if (c->has_ss) CU(cudaMalloc(&c->Kt_ex, sizeof(float) * 6 * (size_t)gf.Hx * gf.Hy * gf.Hz));
         CU(cudaMalloc(&c->Mbuf[0], sizeof(float) * 3 * N));
         CU(cudaMalloc(&c->Mbuf[1], sizeof(float) * 3 * N));
         CU(cudaMalloc(&c->H, sizeof(float) * 3 * N));
@@ -349,11 +379,12 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
             q->twx = c->tw;
             q->twy = c->tw + gf.Lx;
             q->twz = c->tw + gf.Lx + gf.Ly;
-            q->Kt = c->Kt;
+            q->Kt = c->rag && c->has_ss ? c->Kt_ex : c->Kt;
             q->Kd = c->rag ? c->Kd0 : c->Kd;
             q->Kd0 = c->Kd0;
         }
         if (!c->rag) CU(configure_pass_kernels(g, c->l));
+        else if (c->has_ss) CU(configure_fast_split(c->fsplit));
         if (c->has_fs || c->has_ss) CU(configure_step_kernels(c->fs));
         if (c->has_fs) {
             int sms = 0;
@@ -386,11 +417,13 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
         exf.idx2 = 1.0 / (c->cell[0] * c->cell[0]);
         exf.idy2 = 1.0 / (c->cell[1] * c->cell[1]);
         exf.idz2 = 1.0 / (c->cell[2] * c->cell[2]);
-        if (e == cudaSuccess && c->rag)
+        if (e == cudaSuccess && c->rag && c->has_ss)
+            e = tensor_spectrum(c->grid, L, Nd, c->Kt_ex, w1, w2, c->stream);
+        else if (e == cudaSuccess && c->rag)
             e = tensor_spectrum(c->grid, L, Nd, nullptr, w1, w2, c->stream, c->Kd0);
         else if (e == cudaSuccess)
             e = tensor_spectrum(c->grid, L, Nd, c->Kt, w1, w2, c->stream, c->Kd, exf, c->Kd0);
-        if (e == cudaSuccess && c->has_ss) {
+        if (e == cudaSuccess && c->has_ss && !c->rag) {
             ExchangeFold ex3 = exf;
             ex3.on = 1;
             e = tensor_fold_exchange3(c->g, ex3, c->Kt, c->Kt_ex, c->stream);
@@ -495,10 +528,10 @@ int mmk::fused_stage(mm_ctx* c, int mode, const float* Y, const StageArgs& st, c
     if (c->has_fs) {
         const Geom& g = c->gf;
         CU(launch_step_a(g, c->fs, g.Kd, c->S, c->Sh, c->flag, s, true, c->fs.early));
-        CU(launch_stage_x(g, g.nz * (g.Jst / c->fs.rb), c->fs, cf, mode, c->Sh, c->S, Y, st, s));
+        CU(launch_stage_x(g, g.nz * (g.Jr / c->fs.rb), c->fs, cf, mode, c->Sh, c->S, Y, st, s));
     } else {
-        CU(launch_fast_split(c->g, c->fsplit, c->Kt_ex, c->S, s));
-        CU(launch_stage_x(c->g, c->g.nz * (c->g.ny / c->fs.rb), c->fs, cf, mode, c->S, c->S, Y, st, s));
+        CU(launch_fast_split(c->gf, c->fsplit, c->Kt_ex, c->S, s));
+        CU(launch_stage_x(c->gf, c->g.nz * (c->gf.Jr / c->fs.rb), c->fs, cf, mode, c->S, c->S, Y, st, s));
     }
     return MM_OK;
 }
@@ -519,7 +552,7 @@ int mmk::run_passes(mm_ctx* c, int mode, const float* M, float* out, double dt, 
         return MM_OK;
     }
     if (c->has_ss && (mode == kModeDemag || mode == kModeHeff)) {
-        CU(launch_split_xstep(c->g, c->fsplit, c->fs, cf, mode, mode == kModeDemag ? c->Kt : c->Kt_ex, c->S, M,
+        CU(launch_split_xstep(c->gf, c->fsplit, c->fs, cf, mode, mode == kModeDemag ? c->gf.Kt : c->Kt_ex, c->S, M,
                               out, nullptr, s));
         return MM_OK;
     }
@@ -594,7 +627,7 @@ static int enqueue_step(mm_ctx* c, int p, double dt, cudaStream_t s) {
         return MM_OK;
     }
     if (c->has_ss) {
-        CU(launch_split_xstep(c->g, c->fsplit, c->fs, make_coef(c, dt), kModeStep, c->Kt_ex, c->S, c->Mbuf[p],
+        CU(launch_split_xstep(c->gf, c->fsplit, c->fs, make_coef(c, dt), kModeStep, c->Kt_ex, c->S, c->Mbuf[p],
                               c->Mbuf[1 - p], c->flag, s));
         return MM_OK;
     }
@@ -933,6 +966,14 @@ extern "C" int mm_time_passes(mm_ctx* c, int reps, double dt, void* flush, unsig
                 CU(cudaEventRecord(ev[2], c->stream));
                 CU(launch_step_b(c->gf, c->fs, cf, c->Sh, c->S, c->Mbuf[p], c->Mbuf[1 - p], c->flag,
                                  c->stream, false));
+                c->spec_valid = true;
+            } else if (c->rag) {
+                // split pass and x-step on carrier lengths
+                CU(form_spectrum(c, c->Mbuf[p], c->stream));
+                CU(cudaEventRecord(ev[1], c->stream));
+                CU(launch_fast_split(c->gf, c->fsplit, c->Kt_ex, c->S, c->stream));
+                CU(cudaEventRecord(ev[2], c->stream));
+                CU(launch_xstep(c->gf, c->fs, cf, kModeStep, c->S, c->Mbuf[p], c->Mbuf[1 - p], c->flag, c->stream));
                 c->spec_valid = true;
             } else {
                 c->spec_valid = false;            // S no longer holds a step's x spectrum

@@ -21,7 +21,8 @@ struct Geom {
     int nx, ny, nz, N;
     int Lx, Ly, Lz;
     int Hx, Hy, Hz;            // L/2 + 1: stored half-spectrum / octant extents
-    int Jst;                   // stride of j in S (= ny)
+    int Jst;                   // stride of j in S
+    int Jr;                    // rows j of S that are read and written (ny, or ny rounded up)
     AxisPlan px, py, pz;
     const float2* twx;         // W_Lx^m, m < Lx (FP32, from FP64)
     const float2* twy;
@@ -225,6 +226,8 @@ bool fast_step_lookup_plane_a(int ny, int nz, FastStepFns* f);
 bool fast_step_lookup_plane_b(int ny, int nz, FastStepFns* f);
 // Ragged films (ragged.cuh): the kernels and the carrier lengths NX >= nx,
 // NY >= ny; whether the plane kernel triggers the x-step early.
+bool ragged_lookup_x(int nx, FastStepFns* f, int* NX);
+bool ragged_split_lookup(int ny, int nz, FastSplitFns* f, int* NY, int* NZ);   // split_ragged.cu
 bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY);
 // Films that a batch takes on the ragged kernels (ragged_batch.cuh).
 bool ragged_batchable(int nx, int ny, int nz);
@@ -271,6 +274,8 @@ cudaError_t launch_persist(const Geom& g, const PersistFns& f, const LlgCoef& c,
 // Default poll limit of a grid-barrier wait (of the order of a second).
 constexpr long long kGridWaitLimit = 1LL << 20;
 
+cudaError_t launch_xstep(const Geom& g, const FastStepFns& fs, const LlgCoef& c, int mode, float2* S, const float* M,
+                         float* out, int* flag, cudaStream_t s, float* Mcopy = nullptr);
 // Thick-sample step / field: launch_fast_split with Kt, then the x-step
 // kernel of mode `mode` in place on S (S -> S, M -> out).
 cudaError_t launch_split_xstep(const Geom& g, const FastSplitFns& f2, const FastStepFns& fs, const LlgCoef& c,

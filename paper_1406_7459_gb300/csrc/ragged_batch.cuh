@@ -43,6 +43,7 @@ __device__ __forceinline__ Geom rag_geom(const RagDesc& d) {
     g.nz = d.nz;
     g.N = d.N;
     g.Jst = d.Jst;
+    g.Jr = d.Jst;
     g.twx = d.twx;
     g.twy = d.twy;
     return g;

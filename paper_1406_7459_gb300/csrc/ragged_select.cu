@@ -17,10 +17,14 @@ bool ragged_lookup_plane_nz6(int NY, FastStepFns* f);
 bool ragged_lookup_plane_nz7(int NY, FastStepFns* f);
 bool ragged_lookup_plane_nz8(int NY, FastStepFns* f);
 
-bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY) {
+bool ragged_lookup_x(int nx, FastStepFns* f, int* NX) {
     *NX = ragged_len(nx);
+    return ragged_lookup_x_a(*NX, f) || ragged_lookup_x_b(*NX, f) || ragged_lookup_x_c(*NX, f) ||
+           ragged_lookup_x_d(*NX, f);
+}
+
+bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY) {
     *NY = ragged_len(ny);
-    if (!*NX || !*NY) return false;
     bool ok = false;
     switch (nz) {
         case 1: ok = ragged_lookup_plane_nz1(*NY, f); break;
@@ -33,8 +37,7 @@ bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY) {
         case 8: ok = ragged_lookup_plane_nz8(*NY, f); break;
         default: break;
     }
-    return ok && (ragged_lookup_x_a(*NX, f) || ragged_lookup_x_b(*NX, f) ||
-                  ragged_lookup_x_c(*NX, f) || ragged_lookup_x_d(*NX, f));
+    return ok && ragged_lookup_x(nx, f, NX);
 }
 
 int plan_ragged_len(int n) { return ragged_len(n); }
@@ -52,14 +55,14 @@ bool ragged_batchable(int nx, int ny, int nz) {
 // tiles crowd onto the SMs with fewer planes (200x60x3 12.3 against 9.6,
 // 100x100x1 7.1 against 6.7).
 int ragged_early_trigger(const Geom& g, const FastStepFns& f, int sms) {
-    const int tiles = g.nz * (g.Jst / f.rb);
+    const int tiles = g.nz * (g.Jr / f.rb);
     return tiles >= sms || g.Hx >= 3 * sms || tiles + g.Hx <= sms;
 }
 
 cudaError_t launch_ragged_pass1(const Geom& g, const FastStepFns& f, const float* M, float2* S, cudaStream_t s,
                                 float* Mcopy, const XComb& comb) {
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = launch_config(dim3(3 * g.nz * ((g.Jst + f.r1 - 1) / f.r1)), f.t1, f.s1, s, attr);
+    cudaLaunchConfig_t cfg = launch_config(dim3(3 * g.nz * ((g.Jr + f.r1 - 1) / f.r1)), f.t1, f.s1, s, attr);
     if (comb.K) return cudaLaunchKernelEx(&cfg, f.p1c, g, M, S, Mcopy, comb);
     return cudaLaunchKernelEx(&cfg, f.p1, g, M, S, Mcopy);
 }

@@ -1,5 +1,5 @@
-"""Ragged films: sides that are no powers of two, carried in the compile-time
-transform lengths of the two-kernel step.  Sizes sit just above and at the
+"""Ragged samples: sides that are no powers of two, carried in the compile-time
+transform lengths of the two-kernel step and of the split pass.  Sizes sit just above and at the
 carrier lengths (one row or cell into the next length, tiles with one valid
 row, a full carrier), for every layer count and carrier length of the plane
 and x kernels.  Tolerances are those of the other field and step tests: 1e-5
@@ -30,7 +30,14 @@ GRIDS = [(17, 33, 1), (33, 17, 2), (48, 50, 3), (49, 65, 4), (65, 97, 5), (97, 4
          (5, 129, 8), (9, 6, 1)]
 
 
-@pytest.mark.parametrize("grid", GRIDS)
+# thick samples and planes beyond shared memory: every z column length (first
+# and last layer count of it), one odd line, rows and lines past a tile
+THICK = [(17, 33, 9), (33, 18, 16), (20, 49, 17), (40, 17, 24), (65, 20, 25), (16, 30, 33), (18, 20, 48), (9, 34, 49),
+         (12, 17, 64), (17, 12, 65), (8, 10, 96), (10, 9, 97), (7, 18, 128), (100, 65, 10), (257, 20, 12),
+         (20, 1000, 3), (33, 700, 4), (18, 513, 7), (17, 641, 8), (5, 300, 15)]
+
+
+@pytest.mark.parametrize("grid", GRIDS + THICK)
 def test_ragged_film_fields_and_steps(grid):
     from paper_1406_7459_gb300 import mm
     nx, ny, nz = grid
@@ -38,7 +45,7 @@ def test_ragged_film_fields_and_steps(grid):
     Ku, alpha, dt, Hext = 2e4, 0.2, 2e-14, (1e4, -5e3, 2e3)
     M = inputs.random_unit_m(grid, MS, seed=sum(grid))
     ctx = mm.mm_create(grid, cell, MS, A_EX, Ku, alpha, GAMMA)
-    assert mm.mm_plan_info(ctx)[1] == 2
+    assert mm.mm_plan_info(ctx)[1] == (4 if grid in THICK else 2)
     mm.mm_set_field(ctx, Hext)
     Md = torch.from_numpy(M.reshape(-1)).cuda()
     out = torch.full_like(Md, float("nan"))
@@ -79,3 +86,34 @@ def test_ragged_spectrum_is_formed_on_demand():
     mm.mm_demag_field_noalloc(grid, Kt, M, b)
     torch.cuda.synchronize()
     assert rel_l2(a.cpu().numpy().astype(np.float64), b.cpu().numpy().astype(np.float64)) < 1e-5
+
+
+@pytest.mark.parametrize("method", ["heun", "rk4"])
+@pytest.mark.parametrize("grid", [(21, 37, 3), (257, 9, 2), (19, 22, 11)])
+def test_ragged_runge_kutta_and_pass_timing(method, grid):
+    """Fused stages on ragged films and blocks, in runs that end inside and
+    after a captured graph, with a field evaluation in between; then one step
+    advanced by the timing entry point."""
+    from paper_1406_7459_gb300 import mm
+    cell, Hext, dt = (4e-9, 3e-9, 5e-9), (1e4, -5e3, 2e3), 5e-14
+    M = inputs.random_unit_m(grid, MS, seed=5)
+    ctx = mm.mm_create(grid, cell, MS, A_EX, 1e4, 0.2, GAMMA)
+    mm.mm_set_integrator(ctx, method)
+    mm.mm_set_field(ctx, Hext)
+    Md = torch.from_numpy(M.reshape(-1)).cuda()
+    out = torch.empty_like(Md)
+    mm.mm_set_m(ctx, Md)
+    mm.mm_step(ctx, 17, dt)
+    mm.mm_effective_field(ctx, Md, out)
+    mm.mm_step(ctx, 2, dt)
+    mm.mm_set_integrator(ctx, "euler")
+    mm.mm_time_passes(ctx, 1, dt)
+    mm.mm_step(ctx, 1, dt)
+    mm.mm_get_m(ctx, out)
+    mm.mm_sync(ctx)
+    Kt, Lp = oracle_spectrum(grid, cell)
+    args = (dt, method, cell, MS, A_EX, 1e4, 0.2, GAMMA, Hext, Kt, Lp)
+    ref = L.run_rk(M.astype(np.float64), 19, *args)
+    ref = L.run_rk(ref, 2, dt, "euler", *args[2:])
+    got = out.cpu().numpy().reshape(ref.shape)
+    assert rel_l2(got - M, ref - M) < 1e-4
