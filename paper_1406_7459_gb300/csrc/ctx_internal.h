@@ -47,6 +47,7 @@ struct mm_ctx {
     int* flag = nullptr;
     double* partials = nullptr;
     double* Edev = nullptr;
+    double* Ehost = nullptr;   // page-locked copy
     float2* tw = nullptr;      // twiddles of x, y, z back to back
     // step graphs [kind][parity]: kind 0 one step, kind 1 kGraphSteps steps
     cudaGraphExec_t step_exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};

@@ -294,6 +294,7 @@ static void release(mm_ctx* c) {
     cudaFree(c->flag);
     cudaFree(c->partials);
     cudaFree(c->Edev);
+    cudaFreeHost(c->Ehost);
     cudaFree(c->tw);
     cudaFree(c->gbar);
     if (c->cap) cudaStreamDestroy(c->cap);
@@ -362,7 +363,9 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
         CU(cudaMalloc(&c->H, sizeof(float) * 3 * N));
         CU(cudaMalloc(&c->flag, sizeof(int)));
         CU(cudaMalloc(&c->partials, sizeof(double) * energy_partials_elems(g.N)));
-        CU(cudaMalloc(&c->Edev, sizeof(double) * 5));
+        CU(cudaMemset(c->partials, 0, sizeof(double) * energy_partials_elems(g.N)));
+        CU(cudaMalloc(&c->Edev, sizeof(double) * 6));
+        CU(cudaMallocHost(&c->Ehost, sizeof(double) * 6));
         const size_t ntw = (size_t)gf.Lx + gf.Ly + gf.Lz;
         CU(cudaMalloc(&c->tw, sizeof(float2) * ntw));
         {
@@ -854,12 +857,16 @@ extern "C" int mm_step_host(mm_ctx* c, const float* M_in, int n, double dt, floa
     return MM_OK;
 }
 
-static int read_flag(mm_ctx* c) {
-    int f = 0;
-    CU(cudaMemcpy(&f, c->flag, sizeof(int), cudaMemcpyDeviceToHost));
+static int flag_status(int f) {
     if (f & kFlagTimeout) return fail(MM_ETIMEOUT, "a device-side wait gave up; the state is incomplete");
     if (f) return fail(MM_ENONFINITE, "a step produced a non-finite magnetisation");
     return MM_OK;
+}
+
+static int read_flag(mm_ctx* c) {
+    int f = 0;
+    CU(cudaMemcpy(&f, c->flag, sizeof(int), cudaMemcpyDeviceToHost));
+    return flag_status(f);
 }
 
 extern "C" int mm_sync(mm_ctx* c) {
@@ -872,14 +879,14 @@ extern "C" int mm_energy(mm_ctx* c, double E[5]) {
     if (!c || !E) return fail(MM_EINVAL, "null argument");
     int rc = run_passes(c, kModeDemag, c->Mbuf[c->cur], c->H, 0.0, c->stream);
     if (rc != MM_OK) return rc;
-    CU(energy_reduce_full(c->g, c->Ms, c->Hext, c->cell, c->A, c->Ku, c->Mbuf[c->cur], c->H, c->partials,
+    CU(energy_reduce_full(c->g, c->Ms, c->Hext, c->cell, c->A, c->Ku, c->Mbuf[c->cur], c->H, c->flag, c->partials,
                           c->Edev, c->stream));
-    double h[5];
-    CU(cudaMemcpyAsync(h, c->Edev, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    // one copy brings the terms and the status word
+    CU(cudaMemcpyAsync(c->Ehost, c->Edev, sizeof(double) * 6, cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
-    rc = read_flag(c);
+    rc = flag_status((int)c->Ehost[5]);
     if (rc != MM_OK) return rc;
-    for (int q = 0; q < 5; ++q) E[q] = h[q];
+    for (int q = 0; q < 5; ++q) E[q] = c->Ehost[q];
     return MM_OK;
 }
 

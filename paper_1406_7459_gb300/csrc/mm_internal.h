@@ -343,11 +343,12 @@ cudaError_t tensor_spectrum(const int grid[3], const int L[3], const double* N_d
 cudaError_t tensor_fold_exchange3(const Geom& g, ExchangeFold ex, const float* Kt, float* Kt_ex, cudaStream_t s);
 size_t tensor_work_elems(const int grid[3], const int L[3]);
 
-// Energy (energy.cu): E[0..4] into out_dev (5 doubles, device); partials is
-// device scratch of energy_partials_elems(N) doubles.
+// Energy (energy.cu): E[0..4] and the status word *flag (as a double) into
+// out_dev (6 doubles, device); partials is device scratch of
+// energy_partials_elems(N) doubles, zeroed once before the first call.
 size_t energy_partials_elems(int N);
 cudaError_t energy_reduce_full(const Geom& g, double Ms, const double Hext[3], const double cell[3], double A,
-                               double Ku, const float* M, const float* Hd, double* partials, double* out_dev,
-                               cudaStream_t s);
+                               double Ku, const float* M, const float* Hd, const int* flag, double* partials,
+                               double* out_dev, cudaStream_t s);
 
 }  // namespace mmk
