@@ -22,10 +22,12 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/mm.h"
 #include "mm_internal.h"
+#include "fno_back.cuh"
 #include "gemm_tc.cuh"
 
 using namespace mmk;
@@ -204,6 +206,35 @@ __global__ void __launch_bounds__(kYdftThreads)
         const float* fr = Fre + (size_t)iy * H;
         const float* fi = Fim + (size_t)iy * H;
         float sr[4] = {0.f, 0.f, 0.f, 0.f}, si[4] = {0.f, 0.f, 0.f, 0.f};
+        // one row's four kx: a 16-byte read each of its real and imaginary
+        // parts where a row holds whole quads of modes
+        auto row4 = [&](const float* row, float cr, float ci) {
+            float ar[4], ai[4];
+            if ((m & 3) == 0) {
+                const float4 r4 = *reinterpret_cast<const float4*>(row + k0);
+                const float4 i4 = *reinterpret_cast<const float4*>(row + m + k0);
+                ar[0] = r4.x;
+                ar[1] = r4.y;
+                ar[2] = r4.z;
+                ar[3] = r4.w;
+                ai[0] = i4.x;
+                ai[1] = i4.y;
+                ai[2] = i4.z;
+                ai[3] = i4.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int kx = min(k0 + j, m - 1);      // lanes past m are dropped below
+                    ar[j] = row[kx];
+                    ai[j] = row[m + kx];
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                sr[j] += cr * ar[j] - ci * ai[j];
+                si[j] += cr * ai[j] + ci * ar[j];
+            }
+        };
         int y = y0;
         if (((H | yl) & 3) == 0) {                          // four y per F load
             for (; y + 3 < y1; y += 4) {
@@ -211,29 +242,10 @@ __global__ void __launch_bounds__(kYdftThreads)
                 const float4 d4 = __ldg(reinterpret_cast<const float4*>(fi + y));
                 const float crv[4] = {c4.x, c4.y, c4.z, c4.w}, civ[4] = {d4.x, d4.y, d4.z, d4.w};
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float* row = sa + (y + u) * m2;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int kx = min(k0 + j, m - 1);  // lanes past m are dropped below
-                        const float ar = row[kx], ai = row[m + kx];
-                        sr[j] += crv[u] * ar - civ[u] * ai;
-                        si[j] += crv[u] * ai + civ[u] * ar;
-                    }
-                }
+                for (int u = 0; u < 4; ++u) row4(sa + (y + u) * m2, crv[u], civ[u]);
             }
         }
-        for (; y < y1; ++y) {
-            const float cr = __ldg(fr + y), ci = __ldg(fi + y);
-            const float* row = sa + y * m2;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int kx = min(k0 + j, m - 1);
-                const float ar = row[kx], ai = row[m + kx];
-                sr[j] += cr * ar - ci * ai;
-                si[j] += cr * ai + ci * ar;
-            }
-        }
+        for (; y < y1; ++y) row4(sa + y * m2, __ldg(fr + y), __ldg(fi + y));
         float* p = part + ((size_t)sh * NT + q) * 8;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -367,6 +379,33 @@ __global__ void __launch_bounds__(256)
         const float* gr = Gre + (size_t)y * nky;
         const float* gi = Gim + (size_t)y * nky;
         float sr[4] = {0.f, 0.f, 0.f, 0.f}, si[4] = {0.f, 0.f, 0.f, 0.f};
+        auto mode4 = [&](int iy, float a, float c) {
+            float xr[4], xi[4];
+            if ((m & 3) == 0) {
+                const float4 r4 = *reinterpret_cast<const float4*>(wr + iy * m + k0);
+                const float4 i4 = *reinterpret_cast<const float4*>(wi + iy * m + k0);
+                xr[0] = r4.x;
+                xr[1] = r4.y;
+                xr[2] = r4.z;
+                xr[3] = r4.w;
+                xi[0] = i4.x;
+                xi[1] = i4.y;
+                xi[2] = i4.z;
+                xi[3] = i4.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int kx = min(k0 + j, m - 1);     // lanes past m are not stored
+                    xr[j] = wr[iy * m + kx];
+                    xi[j] = wi[iy * m + kx];
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                sr[j] += a * xr[j] - c * xi[j];
+                si[j] += a * xi[j] + c * xr[j];
+            }
+        };
         // four iy per G load (a warp's lanes span several rows y); rows of
         // 2m floats start on 16 bytes for even m
         for (int i4 = 0; (nky & 3) == 0 && i4 < nky; i4 += 4) {
@@ -374,27 +413,9 @@ __global__ void __launch_bounds__(256)
             const float4 c4 = __ldg(reinterpret_cast<const float4*>(gi + i4));
             const float av[4] = {a4.x, a4.y, a4.z, a4.w}, cv[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int iy = i4 + u;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int kx = min(k0 + j, m - 1);     // lanes past m are not stored
-                    const float xr = wr[iy * m + kx], xi = wi[iy * m + kx];
-                    sr[j] += av[u] * xr - cv[u] * xi;
-                    si[j] += av[u] * xi + cv[u] * xr;
-                }
-            }
+            for (int u = 0; u < 4; ++u) mode4(i4 + u, av[u], cv[u]);
         }
-        for (int iy = 0; (nky & 3) != 0 && iy < nky; ++iy) {
-            const float a = __ldg(gr + iy), c = __ldg(gi + iy);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int kx = min(k0 + j, m - 1);
-                const float xr = wr[iy * m + kx], xi = wi[iy * m + kx];
-                sr[j] += a * xr - c * xi;
-                si[j] += a * xi + c * xr;
-            }
-        }
+        for (int iy = 0; (nky & 3) != 0 && iy < nky; ++iy) mode4(iy, __ldg(gr + iy), __ldg(gi + iy));
         __nv_bfloat16* z = Zb + ((size_t)bo * H + y) * nky;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -680,175 +701,6 @@ __global__ void k_outer(const float* __restrict__ a, int Ca, const float* __rest
     if ((threadIdx.x & 31) == 0) atomicAdd(g + o * Cx + c, acc);
 }
 
-// Weight gradients of a per-pixel channel map: g[o][c] += sum_{b,p}
-// a[b][o][p] f_c(b, p) for o < CA, c < CB, and, when gb, gb[o] += sum_{b,p}
-// a[b][o][p].  f_c is xm[b][c][p], or with LIFT the lift's features (x[b][c][p]
-// for c < 3, then y / H and x / W of pixel p).  A block reduces PCH pixels of
-// one sample: 64-pixel tiles of a and f staged in shared memory with
-// 16-byte loads, thread (pixel group, RO x RC output tile) accumulating in
-// registers, the pixel groups summed through shared memory at the end, one
-// atomic add per output and block.
-template <int CA, int CB, bool LIFT>
-__global__ void __launch_bounds__(256) k_wgrad(const float* __restrict__ a, const float* __restrict__ xm, int H, int W,
-                                               long long np, int B, float* __restrict__ g, float* __restrict__ gb) {
-    constexpr int T = 256, PCH = 2048;
-    constexpr int RO = CA < 4 ? CA : 4, RC = CB == 5 ? 5 : 4;
-    static_assert(CA % RO == 0 && CB % RC == 0, "output tiles");
-    constexpr int NGO = CA / RO, NGC = CB / RC, GS = NGO * NGC, PG = T / GS;
-    constexpr int TP = PG > 64 ? PG : 64;                  // pixels per staged tile
-    static_assert(T % GS == 0 && TP % PG == 0 && PCH % TP == 0, "pixel groups");
-    constexpr int NV = RO * RC + RO;                       // per-thread sums (outputs, then biases)
-    constexpr int TS = TP + 1;                             // padded tile row: rows 4 apart in banks differ
-    constexpr int SU = (CA + CB) * TS > T * NV ? (CA + CB) * TS : T * NV;
-    __shared__ __align__(16) float su[SU];                 // tiles, then the group reduction
-    float* as = su;
-    float* fs = su + CA * TS;
-    float* red = su;
-    const long long cpb = (np + PCH - 1) / PCH;
-    const int b = (int)(blockIdx.x / cpb);
-    const long long c0 = (blockIdx.x - (long long)b * cpb) * PCH;
-    const long long c1 = np - c0 < PCH ? np : c0 + PCH;
-    const int gi = threadIdx.x % GS, pg = threadIdx.x / GS;
-    const int o0 = (gi / NGC) * RO, k0 = (gi % NGC) * RC;
-    float acc[RO][RC], bacc[RO];
-#pragma unroll
-    for (int i = 0; i < RO; ++i) {
-        bacc[i] = 0.f;
-#pragma unroll
-        for (int j = 0; j < RC; ++j) acc[i][j] = 0.f;
-    }
-    const float* ab = a + (long long)b * CA * np;
-    const bool vec = (np & 3) == 0;
-    for (long long p0 = c0; p0 < c1; p0 += TP) {
-        const int tw = (int)(c1 - p0 < TP ? c1 - p0 : TP);
-        __syncthreads();
-        if (vec && tw == TP) {
-            for (int e = threadIdx.x; e < CA * TP / 4; e += T) {
-                const int r = e / (TP / 4), q = e - r * (TP / 4);
-                const float4 v4 = *reinterpret_cast<const float4*>(ab + r * np + p0 + 4 * q);
-                float* d = as + r * TS + 4 * q;
-                d[0] = v4.x;
-                d[1] = v4.y;
-                d[2] = v4.z;
-                d[3] = v4.w;
-            }
-        } else {
-            for (int e = threadIdx.x; e < CA * TP; e += T) {
-                const int r = e / TP, q = e - r * TP;
-                as[r * TS + q] = q < tw ? ab[r * np + p0 + q] : 0.f;
-            }
-        }
-        for (int e = threadIdx.x; e < CB * TP; e += T) {
-            const int r = e / TP, q = e - r * TP;
-            const long long pp = p0 + q;
-            float v = 0.f;
-            if (q < tw) {
-                if (LIFT && r >= 3)
-                    v = r == 3 ? (float)(pp / W) / (float)H : (float)(pp % W) / (float)W;
-                else
-                    v = xm[((long long)b * (LIFT ? 3 : CB) + r) * np + pp];
-            }
-            fs[r * TS + q] = v;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int q = pg; q < TP; q += PG) {
-            float av[RO], fv[RC];
-#pragma unroll
-            for (int i = 0; i < RO; ++i) av[i] = as[(o0 + i) * TS + q];
-#pragma unroll
-            for (int j = 0; j < RC; ++j) fv[j] = fs[(k0 + j) * TS + q];
-#pragma unroll
-            for (int i = 0; i < RO; ++i) {
-                bacc[i] += av[i];
-#pragma unroll
-                for (int j = 0; j < RC; ++j) acc[i][j] = fmaf(av[i], fv[j], acc[i][j]);
-            }
-        }
-    }
-    // sum the pixel groups: red[pg][gi][..] over the tiles' space
-    __syncthreads();
-    float* mine = red + (size_t)threadIdx.x * NV;
-#pragma unroll
-    for (int i = 0; i < RO; ++i) {
-        mine[RO * RC + i] = bacc[i];
-#pragma unroll
-        for (int j = 0; j < RC; ++j) mine[i * RC + j] = acc[i][j];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < GS * NV; e += T) {
-        const int gg = e / NV, k = e - gg * NV;
-        float sum = 0.f;
-        for (int q = 0; q < PG; ++q) sum += red[((size_t)q * GS + gg) * NV + k];
-        const int oo = (gg / NGC) * RO, kk = (gg % NGC) * RC;
-        if (k < RO * RC)
-            atomicAdd(g + (oo + k / RC) * CB + kk + k % RC, sum);
-        else if (gb && gg % NGC == 0)
-            atomicAdd(gb + oo + (k - RO * RC), sum);
-    }
-}
-
-// Per-pixel channel map through a transposed matrix:
-// out[b][j][p] = sum_i M[i][j] in[b][i][p] (M stored CI x CO), FP32.  Tiles
-// of 64 pixels x CI channels staged in shared memory with 16-byte loads;
-// thread (p, og) forms CO / OG outputs and stores them (consecutive
-// threads, consecutive pixels).
-template <int CI, int CO>
-__global__ void __launch_bounds__(256) k_chanmap_t(const float* __restrict__ in, const float* __restrict__ M,
-                                                   long long np, int B, float* __restrict__ out) {
-    constexpr int T = 256, TP = 64, OG = T / TP, OPG = CO / OG;
-    static_assert(CO % OG == 0, "output groups");
-    constexpr int CP = (CI + 3) & ~3;                      // row of the transposed matrix, padded to 4
-    __shared__ __align__(16) float Ms[CO * CP];            // Ms[j][i] = M[i][j]
-    __shared__ __align__(16) float is[CI * TP];
-    for (int e = threadIdx.x; e < CO * CP; e += T) {
-        const int j = e / CP, i = e - j * CP;
-        Ms[e] = i < CI ? M[i * CO + j] : 0.f;
-    }
-    const long long tpb = (np + TP - 1) / TP, ntiles = (long long)B * tpb;
-    const bool vec = (np & 3) == 0;
-    const int p = threadIdx.x % TP, og = threadIdx.x / TP;
-    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int b = (int)(tile / tpb);
-        const long long p0 = (tile - (long long)b * tpb) * TP;
-        const int tw = (int)(np - p0 < TP ? np - p0 : TP);
-        const float* ib = in + (long long)b * CI * np + p0;
-        __syncthreads();
-        if (vec && tw == TP) {
-            for (int e = threadIdx.x; e < CI * TP / 4; e += T) {
-                const int r = e / (TP / 4), q = e - r * (TP / 4);
-                reinterpret_cast<float4*>(is)[e] = *reinterpret_cast<const float4*>(ib + r * np + 4 * q);
-            }
-        } else {
-            for (int e = threadIdx.x; e < CI * TP; e += T) {
-                const int r = e / TP, q = e - r * TP;
-                is[e] = q < tw ? ib[r * np + q] : 0.f;
-            }
-        }
-        __syncthreads();
-        if (p >= tw) continue;
-        float xv[CP];
-#pragma unroll
-        for (int i = 0; i < CP; ++i) xv[i] = i < CI ? is[i * TP + p] : 0.f;
-        float* ob = out + (long long)b * CO * np + p0 + p;
-#pragma unroll 4
-        for (int jj = 0; jj < OPG; ++jj) {
-            const int j = og * OPG + jj;
-            const float4* m4 = reinterpret_cast<const float4*>(Ms + j * CP);
-            float acc = 0.f;
-#pragma unroll
-            for (int i4 = 0; i4 < CP / 4; ++i4) {
-                const float4 w = m4[i4];
-                acc = fmaf(w.x, xv[4 * i4], acc);
-                acc = fmaf(w.y, xv[4 * i4 + 1], acc);
-                acc = fmaf(w.z, xv[4 * i4 + 2], acc);
-                acc = fmaf(w.w, xv[4 * i4 + 3], acc);
-            }
-            ob[(long long)j * np] = acc;
-        }
-    }
-}
-
 __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m1,
                        float* __restrict__ m2, long long n, float lr, float b1, float b2, float c1, float c2,
                        float eps) {
@@ -946,6 +798,8 @@ static void fno_free(mm_fno* f) {
     cudaFree(f->zb); cudaFree(f->db16); cudaFree(f->dloss); cudaFree(f->err);
 }
 
+static cudaError_t back_part(mm_fno* f, int which, int B, int l, const float* p);
+
 extern "C" int mm_fno_create(mm_fno** out, int H, int W, int width, int modes, int layers, int max_batch,
                              unsigned long long seed, void* stream) {
     if (!out) return fno_fail(MM_EINVAL, "out is NULL");
@@ -1033,6 +887,7 @@ extern "C" int mm_fno_create(mm_fno** out, int H, int W, int width, int modes, i
         FCU(cudaStreamCreateWithFlags(&f->cap, cudaStreamNonBlocking));
         FCU(cudaMemset(f->err, 0, sizeof(int)));
         FCU(gemm_configure());
+        FCU(back_part(f, 3, 0, 0, nullptr));
         return MM_OK;
     }();
     if (rc != MM_OK) {
@@ -1218,69 +1073,96 @@ static int fno_forward(mm_fno* f, int B, const float* x, bool train, float* y = 
     return MM_OK;
 }
 
+// The activation-sized parts of the backward pass for the widths that
+// fno_back.cuh is instantiated for.
+template <int CW> static cudaError_t back_head(mm_fno* f, int B, const float* t) {
+    const unsigned blocks = (unsigned)(B * ((f->np + kHeadPx - 1) / kHeadPx));
+    k_head_back<CW><<<blocks, 256, 0, f->s>>>(f->y, t, f->vf[f->L], f->np, (long long)B * 3 * f->np, f->dy, f->dloss,
+                                              f->g + f->oQ, f->g + f->oq);
+    return cudaGetLastError();
+}
+template <int CW> static cudaError_t back_layer(mm_fno* f, int B, int l) {
+    using Cfg = LayerBackCfg<CW>;
+    const long long CC = (long long)f->C * f->C, tiles = (long long)B * ((f->np + Cfg::TP - 1) / Cfg::TP);
+    const unsigned most = 152 * (CW <= 32 ? 3 : 2);
+    const unsigned blocks = (unsigned)(tiles < most ? tiles : most);
+    const float* Wl = f->w + f->oW + l * CC;
+    float *gW = f->g + f->oW + l * CC, *gb = f->g + f->ob + (long long)l * f->C;
+    if (l == f->L - 1)
+        k_layer_back<CW, kBackHead><<<blocks, Cfg::T, Cfg::BYTES, f->s>>>(f->dy, nullptr, f->vf[l], Wl, f->w + f->oQ,
+                                                                          f->np, B, f->db16, f->tmp, gW, gb);
+    else
+        k_layer_back<CW, kBackAct><<<blocks, Cfg::T, Cfg::BYTES, f->s>>>(f->dv, f->u[l], f->vf[l], Wl, nullptr, f->np,
+                                                                         B, f->db16, f->tmp, gW, gb);
+    return cudaGetLastError();
+}
+template <int CW> static cudaError_t back_lift(mm_fno* f, int B, const float* x) {
+    const unsigned blocks = (unsigned)(B * ((f->np + kHeadPx - 1) / kHeadPx));
+    k_lift_back<CW><<<blocks, 256, 0, f->s>>>(f->dv, x, f->H, f->W, f->g + f->oP, f->g + f->op);
+    return cudaGetLastError();
+}
+template <int CW> static cudaError_t back_configure() {
+    cudaError_t e = cudaFuncSetAttribute(k_layer_back<CW, kBackAct>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)LayerBackCfg<CW>::BYTES);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_layer_back<CW, kBackHead>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)LayerBackCfg<CW>::BYTES);
+    return e;
+}
+
+static bool back_fused(const mm_fno* f) { return f->C == 8 || f->C == 16 || f->C == 32 || f->C == 64; }
+
+// which: 0 head, 1 layer l, 2 lift, 3 shared-memory limits
+static cudaError_t back_part(mm_fno* f, int which, int B, int l, const float* p) {
+    auto run = [&](auto cw) {
+        constexpr int CW = decltype(cw)::value;
+        return which == 0   ? back_head<CW>(f, B, p)
+               : which == 1 ? back_layer<CW>(f, B, l)
+               : which == 2 ? back_lift<CW>(f, B, p)
+                            : back_configure<CW>();
+    };
+    switch (f->C) {
+        case 8: return run(std::integral_constant<int, 8>{});
+        case 16: return run(std::integral_constant<int, 16>{});
+        case 32: return run(std::integral_constant<int, 32>{});
+        case 64: return run(std::integral_constant<int, 64>{});
+        default: return cudaSuccess;
+    }
+}
+
 // backward pass for the batch whose forward pass is in f; t (B, 3, H, W)
 // FP32 device; gradients into f->g, loss (FP64) into f->dloss.
-// Tiled backward helpers for the widths they are instantiated for.
-template <int CW>
-static void bw_launch(mm_fno* f, int B, int which, int l, const float* a, const float* xm, const float* xin) {
-    const long long np = f->np;
-    const int C = f->C;
-    const unsigned blocks = (unsigned)(B * ((np + 2047) / 2048));
-    const long long tiles = (long long)B * ((np + 63) / 64);
-    const unsigned cgrid = (unsigned)(tiles < 152 * 8 ? tiles : 152 * 8);
-    cudaStream_t s = f->s;
-    switch (which) {
-        case 0:   // Q, q from dy and the last activations; dv = Q^T dy
-            k_wgrad<3, CW, false><<<blocks, 256, 0, s>>>(a, xm, f->H, f->W, np, B, f->g + f->oQ, f->g + f->oq);
-            k_chanmap_t<3, CW><<<cgrid, 256, 0, s>>>(a, f->w + f->oQ, np, B, f->dv);
-            break;
-        case 1:   // W_l, b_l from du and v_l; tmp = W_l^T du
-            k_wgrad<CW, CW, false><<<blocks, 256, 0, s>>>(a, xm, f->H, f->W, np, B, f->g + f->oW + (long long)l * C * C,
-                                                          f->g + f->ob + (long long)l * C);
-            k_chanmap_t<CW, CW><<<cgrid, 256, 0, s>>>(a, f->w + f->oW + (long long)l * C * C, np, B, f->tmp);
-            break;
-        default:  // P, p from dv_0 and the lift's features
-            k_wgrad<CW, 5, true><<<blocks, 256, 0, s>>>(a, xin, f->H, f->W, np, B, f->g + f->oP, f->g + f->op);
-            break;
-    }
-}
-
-static bool bw_tiled(mm_fno* f, int B, int which, int l, const float* a, const float* xm, const float* xin) {
-    switch (f->C) {
-        case 8: bw_launch<8>(f, B, which, l, a, xm, xin); return true;
-        case 16: bw_launch<16>(f, B, which, l, a, xm, xin); return true;
-        case 32: bw_launch<32>(f, B, which, l, a, xm, xin); return true;
-        case 64: bw_launch<64>(f, B, which, l, a, xm, xin); return true;
-        default: return false;
-    }
-}
-
 static int fno_backward(mm_fno* f, int B, const float* x, const float* t) {
     const int C = f->C, m = f->m, L = f->L, H = f->H, W = f->W;
     const long long np = f->np, act = (long long)B * C * np, ny = (long long)B * 3 * np;
     const int nmode = 2 * m * m;
+    const bool fused = back_fused(f);
     cudaStream_t s = f->s;
     FCU(cudaMemsetAsync(f->g, 0, 4 * f->n_params, s));
     FCU(cudaMemsetAsync(f->dloss, 0, 8, s));
-    k_loss<<<grid1(ny), 256, 0, s>>>(f->y, t, ny, f->dy, f->dloss);
     const int gx = 64;
-    if (!bw_tiled(f, B, 0, 0, f->dy, f->vf[L], x)) {
+    if (fused) {
+        FCU(back_part(f, 0, B, 0, t));
+    } else {
+        k_loss<<<grid1(ny), 256, 0, s>>>(f->y, t, ny, f->dy, f->dloss);
         k_outer<<<dim3(gx, 3 * C), 256, 0, s>>>(f->dy, 3, f->vf[L], C, np, B, f->g + f->oQ);
         k_colsum<<<dim3(gx, 3), 256, 0, s>>>(f->dy, 3, np, B, f->g + f->oq);
         k_pointwise<<<grid1(B * np), 256, 0, s>>>(f->dy, 3, f->w + f->oQ, nullptr, C, np, B, 1, f->dv);
     }
     for (int l = L - 1; l >= 0; --l) {
-        if (l < L - 1) k_act_back<<<grid1(act), 256, 0, s>>>(f->u[l], f->dv, act);
-        // dv now holds du for layer l
-        if (!bw_tiled(f, B, 1, l, f->dv, f->vf[l], x)) {
+        if (fused) {
+            FCU(back_part(f, 1, B, l, nullptr));
+        } else {
+            if (l < L - 1) k_act_back<<<grid1(act), 256, 0, s>>>(f->u[l], f->dv, act);
+            // dv now holds du for layer l
             k_colsum<<<dim3(gx, C), 256, 0, s>>>(f->dv, C, np, B, f->g + f->ob + (long long)l * C);
             k_outer<<<dim3(gx, C * C), 256, 0, s>>>(f->dv, C, f->vf[l], C, np, B,
                                                      f->g + f->oW + (long long)l * C * C);
             k_pointwise<<<grid1(B * np), 256, 0, s>>>(f->dv, C, f->w + f->oW + (long long)l * C * C, nullptr, C, np, B,
                                                        1, f->tmp);
+            k_to_bf16<<<grid1(act), 256, 0, s>>>(f->dv, f->db16, act, 1.f);
         }
         // spectral path: dw = (a/(HW)) modes(du); dR += dw conj(vh); dvh = R^H dw
-        k_to_bf16<<<grid1(act), 256, 0, s>>>(f->dv, f->db16, act, 1.f);
         GemmArgs g{};
         g.A = f->db16; g.B = f->Fx; g.C = f->Z;
         g.M = B * C * H; g.N = 2 * m; g.K = W;
@@ -1289,8 +1171,14 @@ static int fno_backward(mm_fno* f, int B, const float* x, const float* t) {
         FCU(gemm(g, 1, f->err, s));
         FCU(ydft(f, f->Z, B * C, f->dwr, f->dwi, 1.f / ((float)H * W), 1, s));
         const long long ro = (long long)l * C * C * nmode;
-        k_dR<<<grid1((long long)C * C * nmode), 256, 0, s>>>(f->dwr, f->dwi, f->vhr[l], f->vhi[l], C, nmode, B,
-                                                             f->g + f->oRr + ro, f->g + f->oRi + ro);
+        float *gre = f->g + f->oRr + ro, *gim = f->g + f->oRi + ro;
+        auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+        if (nmode % 4 == 0 && al(gre) && al(gim) && (long long)C * C * nmode < (1LL << 31))
+            k_dR4<<<grid1((long long)C * C * nmode / 4), 256, 0, s>>>(f->dwr, f->dwi, f->vhr[l], f->vhi[l], C, nmode,
+                                                                      B, gre, gim);
+        else
+            k_dR<<<grid1((long long)C * C * nmode), 256, 0, s>>>(f->dwr, f->dwi, f->vhr[l], f->vhi[l], C, nmode, B,
+                                                                 gre, gim);
         FCU(mode_inv(f, l, B, f->dwr, f->dwi, 1, s));
         GemmArgs g2{};
         g2.A = f->zb; g2.B = f->Gxa; g2.C = f->tmp;
@@ -1302,7 +1190,9 @@ static int fno_backward(mm_fno* f, int B, const float* x, const float* t) {
         f->dv = f->tmp;
         f->tmp = t2;
     }
-    if (!bw_tiled(f, B, 2, 0, f->dv, nullptr, x)) {
+    if (fused) {
+        FCU(back_part(f, 2, B, 0, x));
+    } else {
         k_outer_lift<<<dim3(gx, C * 5), 256, 0, s>>>(f->dv, C, x, H, W, B, f->g + f->oP);
         k_colsum<<<dim3(gx, C), 256, 0, s>>>(f->dv, C, np, B, f->g + f->op);
     }
