@@ -138,49 +138,84 @@ __device__ __forceinline__ void tc_epilogue(const GemmArgs& a, float* C, uint32_
     }
 }
 
-// Epilogue for a row-major C with 16-byte aligned rows: per 16-column
-// chunk the warp's 32 rows go through the warp's 32 x 17 float buffer `buf`
-// in shared memory; lane l then stores 4 columns of rows 8 i + l / 4.
+// Epilogue for a row-major C: per 32-column
+// chunk the warp's 32 rows go through the warp's 32 x 36 float buffer `buf`
+// in shared memory (rows 16-byte aligned and four banks apart); lane l then
+// stores 4 columns of rows 4 i + l / 8, so that a store instruction writes
+// whole 128-byte lines; where C's rows are not 16-byte aligned, one column of
+// each row in turn (128 contiguous bytes).
+constexpr int kTcBufRow = 36;
 template <int BN>
 __device__ __forceinline__ void tc_epilogue_rows(const GemmArgs& a, float* C, uint32_t tmem, int m0, int n0,
                                                  int warp, int lane, float* buf) {
+    const bool c_vec = a.scm % 4 == 0 && a.zC % 4 == 0 && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0;
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 16) {
-        uint32_t v[16];
+    for (int c0 = 0; c0 < BN; c0 += 32) {
+        uint32_t v[32];
         const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
         asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-            "[%16];"
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+              "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
+              "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
+              "=r"(v[30]), "=r"(v[31])
             : "r"(taddr)
             : "memory");
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int j = 0; j < 16; ++j) buf[lane * 17 + j] = __uint_as_float(v[j]);
+        for (int j = 0; j < 8; ++j)
+            *reinterpret_cast<uint4*>(buf + lane * kTcBufRow + 4 * j) =
+                make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int rr = 8 * i + (lane >> 2), cq = lane & 3;
-            const int row = m0 + warp * 32 + rr, col = n0 + c0 + 4 * cq;
-            const float* b = buf + rr * 17 + 4 * cq;
-            if (row < a.M) {
-                float* p = C + (long long)row * a.scm + col;
-                if (col + 3 < a.N) {
-                    float4 o = make_float4(a.alpha * b[0], a.alpha * b[1], a.alpha * b[2], a.alpha * b[3]);
-                    if (a.beta != 0.f) {
-                        const float4 q = *reinterpret_cast<const float4*>(p);
-                        o.x += a.beta * q.x;
-                        o.y += a.beta * q.y;
-                        o.z += a.beta * q.z;
-                        o.w += a.beta * q.w;
-                    }
-                    *reinterpret_cast<float4*>(p) = o;
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (col + j < a.N) p[j] = (a.beta != 0.f) ? a.beta * p[j] + a.alpha * b[j] : a.alpha * b[j];
+        if (!c_vec) {
+            const int col = n0 + c0 + lane;
+            const int nr = min(32, a.M - (m0 + warp * 32));
+            if (col < a.N) {
+                float* p = C + (long long)(m0 + warp * 32) * a.scm + col;
+#pragma unroll 8
+                for (int rr = 0; rr < nr; ++rr) {
+                    const float val = a.alpha * buf[rr * kTcBufRow + lane];
+                    p[(long long)rr * a.scm] = (a.beta != 0.f) ? a.beta * p[(long long)rr * a.scm] + val : val;
                 }
+            }
+            __syncwarp();
+            continue;
+        }
+        const int cq = lane & 7, col = n0 + c0 + 4 * cq;
+        if (col + 3 < a.N) {
+            // every old value of the chunk in flight before the first store
+            float4 q[8];
+            if (a.beta != 0.f) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int row = m0 + warp * 32 + 4 * i + (lane >> 3);
+                    if (row < a.M) q[i] = *reinterpret_cast<const float4*>(C + (long long)row * a.scm + col);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int rr = 4 * i + (lane >> 3), row = m0 + warp * 32 + rr;
+                if (row >= a.M) continue;
+                const float4 b = *reinterpret_cast<const float4*>(buf + rr * kTcBufRow + 4 * cq);
+                float4 o = make_float4(a.alpha * b.x, a.alpha * b.y, a.alpha * b.z, a.alpha * b.w);
+                if (a.beta != 0.f) {
+                    o.x += a.beta * q[i].x;
+                    o.y += a.beta * q[i].y;
+                    o.z += a.beta * q[i].z;
+                    o.w += a.beta * q[i].w;
+                }
+                *reinterpret_cast<float4*>(C + (long long)row * a.scm + col) = o;
+            }
+        } else {
+            for (int i = 0; i < 8; ++i) {
+                const int rr = 4 * i + (lane >> 3), row = m0 + warp * 32 + rr;
+                if (row >= a.M) continue;
+                const float* b = buf + rr * kTcBufRow + 4 * cq;
+                float* p = C + (long long)row * a.scm + col;
+                for (int j = 0; j < 4; ++j)
+                    if (col + j < a.N) p[j] = (a.beta != 0.f) ? a.beta * p[j] + a.alpha * b[j] : a.alpha * b[j];
             }
         }
         __syncwarp();
@@ -312,10 +347,12 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc(GemmArgs a) {
     }
 }
 
-// All of K resident (K a multiple of 16 up to kTcKFull, both operands
-// K-contiguous with 16-byte aligned rows): every 16-byte chunk of the A
+// All of K resident (1 <= K <= kTcKFull, both operands K-contiguous), K
+// rounded up to a multiple of 16 with zeros: every 16-byte chunk of the A
 // (128 x K) and B (BN x K) tiles is requested at once with cp.async (zero
-// fill outside M and N), then thread 0 issues the K / 16 MMAs back to back
+// fill outside M, N and K) where an operand's rows are 16-byte aligned and 8
+// divides K, else gathered element by element, eight to a chunk; then
+// thread 0 issues the K / 16 MMAs back to back
 // and commits them once.  A tile costs one memory latency and one MMA wait
 // instead of one of each per 32-wide K slice.  Tile layout: K-major core
 // matrices without swizzle, row r and chunk c (k = 8 c .. 8 c + 7) at
@@ -326,13 +363,42 @@ __device__ __forceinline__ void tc_cp16(uint32_t dst, const void* src, bool in) 
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
 
+// Rows r0 .. r0 + ROWS - 1 of a K-contiguous operand (row stride `rs`,
+// `rows` of them in all) into the tile at shared address dst.
+template <int ROWS>
+__device__ __forceinline__ void tc_load_rows(uint32_t dst, const __nv_bfloat16* __restrict__ P, int r0, int rows,
+                                             int K, int KC, long long rs, bool vec, uint32_t sbo) {
+    if (vec) {
+        for (int e = threadIdx.x; e < ROWS * KC; e += kTcThreads) {
+            const int r = e / KC, c = e - r * KC;
+            const bool in = r0 + r < rows && 8 * c < K;
+            tc_cp16(dst + (uint32_t)((r >> 3) * sbo + c * 128 + (r & 7) * 16),
+                    in ? (const void*)(P + (long long)(r0 + r) * rs + 8 * c) : (const void*)P, in);
+        }
+        return;
+    }
+    const unsigned short* p16 = reinterpret_cast<const unsigned short*>(P);
+#pragma unroll 2
+    for (int e = threadIdx.x; e < ROWS * KC; e += kTcThreads) {
+        const int r = e / KC, c = e - r * KC;
+        const unsigned short* p = p16 + (long long)(r0 + r) * rs + 8 * c;
+        unsigned h[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) h[j] = r0 + r < rows && 8 * c + j < K ? __ldg(p + j) : 0u;
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                         dst + (uint32_t)((r >> 3) * sbo + c * 128 + (r & 7) * 16)),
+                     "r"(h[0] | h[1] << 16), "r"(h[2] | h[3] << 16), "r"(h[4] | h[5] << 16), "r"(h[6] | h[7] << 16)
+                     : "memory");
+    }
+}
+
 template <int BN>
 __global__ void __launch_bounds__(kTcThreads) k_gemm_tc_kfull(GemmArgs a) {
     static_assert(BN % 16 == 0 && BN >= 32 && BN <= 256 && (BN & (BN - 1)) == 0, "MMA N and TMEM columns");
     extern __shared__ __align__(1024) unsigned char tc_smem[];
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
-    const int K = a.K, KC = K / 8;                        // 16-byte chunks per row
+    const int K = (a.K + 15) & ~15, KC = K / 8;           // 16-byte chunks per row
     const uint32_t As_s = (uint32_t)__cvta_generic_to_shared(tc_smem);
     const uint32_t Bs_s = As_s + (uint32_t)(kTcM * K * 2);
     const uint32_t sbo = (uint32_t)KC * 128;
@@ -350,18 +416,11 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc_kfull(GemmArgs a) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // the whole tile pair in flight before anything else
-    for (int e = threadIdx.x; e < kTcM * KC; e += kTcThreads) {
-        const int r = e / KC, c = e - r * KC;
-        const bool in = m0 + r < a.M;
-        tc_cp16(As_s + (uint32_t)((r >> 3) * sbo + c * 128 + (r & 7) * 16),
-                in ? (const void*)(A + (long long)(m0 + r) * a.sam + 8 * c) : (const void*)A, in);
-    }
-    for (int e = threadIdx.x; e < BN * KC; e += kTcThreads) {
-        const int n = e / KC, c = e - n * KC;
-        const bool in = n0 + n < a.N;
-        tc_cp16(Bs_s + (uint32_t)((n >> 3) * sbo + c * 128 + (n & 7) * 16),
-                in ? (const void*)(B + (long long)(n0 + n) * a.sbn + 8 * c) : (const void*)B, in);
-    }
+    auto vec = [&](const void* p, long long rs, long long z) {
+        return a.K % 8 == 0 && rs % 8 == 0 && z % 8 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+    };
+    tc_load_rows<kTcM>(As_s, A, m0, a.M, a.K, KC, a.sam, vec(a.A, a.sam, a.zA), sbo);
+    tc_load_rows<BN>(Bs_s, B, n0, a.N, a.K, KC, a.sbn, vec(a.B, a.sbn, a.zB), sbo);
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (warp == 0) {
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&tmem_base);
@@ -401,13 +460,11 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc_kfull(GemmArgs a) {
     if (!ok) {
         if (threadIdx.x == 0) atomicOr(a.err, 1);
         tc_wait(mbar_s, 0);                               // the MMAs in flight, bounded again
-    } else if (!a.atomic && a.scn == 1 && a.scm % 4 == 0 && a.zC % 4 == 0 &&
-               (reinterpret_cast<uintptr_t>(a.C) & 15) == 0) {
+    } else if (!a.atomic && a.scn == 1) {
         // row-major C: the operand tiles are free now; each warp passes its
-        // rows through 32 x 17 floats of them so that a store instruction
-        // writes 64 contiguous bytes of each of 8 rows
+        // rows through 32 x 36 floats of them
         tc_epilogue_rows<BN>(a, C, tmem, m0, n0, warp, lane,
-                             reinterpret_cast<float*>(tc_smem) + warp * 32 * 17);
+                             reinterpret_cast<float*>(tc_smem) + warp * 32 * kTcBufRow);
     } else {
         tc_epilogue<BN>(a, C, tmem, m0, n0, warp, lane, true);
     }
@@ -421,15 +478,17 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc_kfull(GemmArgs a) {
 
 // Dynamic shared memory of k_gemm_tc_kfull<BN> for a given K: the tiles,
 // padded like gemm_tc_smem so that at most 512 / BN CTAs share an SM.
+template <int BN> constexpr size_t gemm_tc_kfull_floor() {
+    constexpr size_t share = 227 * 1024 / (512 / BN) + 1024, buf = 4 * 32 * kTcBufRow * sizeof(float);   // epilogue
+    return share > buf ? share : buf;
+}
 template <int BN> inline size_t gemm_tc_kfull_smem(int K) {
-    const size_t tiles = (size_t)(kTcM + BN) * K * 2;
-    const size_t floor_ = 227 * 1024 / (512 / BN) + 1024;
-    return tiles > floor_ ? tiles : floor_;
+    const size_t tiles = (size_t)(kTcM + BN) * ((K + 15) & ~15) * 2;
+    return tiles > gemm_tc_kfull_floor<BN>() ? tiles : gemm_tc_kfull_floor<BN>();
 }
 template <int BN> constexpr size_t gemm_tc_kfull_smem_max() {
-    return (size_t)(kTcM + BN) * kTcKFull * 2 > 227 * 1024 / (512 / BN) + 1024
-               ? (size_t)(kTcM + BN) * kTcKFull * 2
-               : 227 * 1024 / (512 / BN) + 1024;
+    return (size_t)(kTcM + BN) * kTcKFull * 2 > gemm_tc_kfull_floor<BN>() ? (size_t)(kTcM + BN) * kTcKFull * 2
+                                                                           : gemm_tc_kfull_floor<BN>();
 }
 
 // Dynamic shared memory of k_gemm_tc<BN>: the two tiles, padded so that at
