@@ -49,11 +49,13 @@ namespace mmk {
 // plane blocks (measured per flushed step: 64x64x4 11.1 vs 11.9 us late,
 // 128x128x4 19.2 vs 15.4, 256x256x4 25.4 vs 25.4, 1024x1024x1 90.8 vs 92.9;
 // the field evaluations keep the late trigger, 23.2 vs 25.0 us at 256).
+// Also where planes and tiles together leave each SM one block (100 steps of
+// 32x32x1 454 us early against 478, 60 of 64x64x4 359 against 373).
 // MM_EARLY_TRIGGER=0/1 overrides the choice (for measurements).
-int fast_step_early_trigger(const Geom& g, int sms) {
+int fast_step_early_trigger(const Geom& g, const FastStepFns& f, int sms) {
     const char* e = getenv("MM_EARLY_TRIGGER");
     if (e && (e[0] == '0' || e[0] == '1') && e[1] == 0) return e[0] == '1';
-    return g.Hx > sms ? 1 : 0;
+    return g.Hx > sms || g.Hx + g.nz * (g.ny / f.rb) <= sms;
 }
 
 cudaError_t configure_step_kernels(const FastStepFns& f) {

@@ -392,7 +392,7 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
         if (c->has_fs) {
             int sms = 0;
             CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
-            c->fs.early = c->rag ? ragged_early_trigger(gf, c->fs, sms) : fast_step_early_trigger(gf, sms);
+            c->fs.early = c->rag ? ragged_early_trigger(gf, c->fs, sms) : fast_step_early_trigger(gf, c->fs, sms);
             if (!c->rag) encode_xstep_maps(g, &c->fs, c->Sh, c->S);   // per-thread copies where no map applies
         }
         if (c->has_persist) {

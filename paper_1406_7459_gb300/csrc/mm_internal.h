@@ -244,7 +244,7 @@ cudaError_t launch_step_pdl(const Geom& g, const FastStepFns& f, const LlgCoef& 
                             const float* M, float* Mout, int* flag, cudaStream_t s, bool pdl,
                             float* Mcopy = nullptr);
 cudaError_t configure_step_kernels(const FastStepFns& f);
-int fast_step_early_trigger(const Geom& g, int sms);
+int fast_step_early_trigger(const Geom& g, const FastStepFns& f, int sms);
 cudaError_t launch_step_a(const Geom& g, const FastStepFns& f, const float* Kd, const float2* S, float2* Sh,
                           int* flag, cudaStream_t s, bool pdl, int early);
 // The two-kernel evaluation of H_demag (mode kModeDemag, plain 2-D spectrum
