@@ -54,6 +54,9 @@ struct mm_ctx {
     double step_dt[2][2] = {{0, 0}, {0, 0}};
     unsigned long long step_ver[2][2] = {{0, 0}, {0, 0}};
     unsigned long long ver = 1;   // bumped when H_ext changes
+    int warm = 0;                 // steps launched directly with warm_dt, warm_ver (mm_step)
+    double warm_dt = 0;
+    unsigned long long warm_ver = 0;
     bool use_graphs = true;
     FastFns fast;              // compile-time kernels (when the grid has them)
     FastStepFns fs;            // two-kernel step (power-of-two grids)

@@ -648,6 +648,8 @@ static int enqueue_step(mm_ctx* c, int p, double dt, cudaStream_t s) {
 // from).  Inside one graph consecutive steps keep their programmatic
 // launch edges, so a step's first kernel starts while the previous one drains.
 constexpr int kGraphSteps = 16;
+// Steps of one dt that launch directly before graphs are captured.
+constexpr int kWarmSteps = 128;
 
 // Capture one step (kind 0) or kGraphSteps steps (kind 1) from parity p on
 // the private stream into a graph.
@@ -757,11 +759,19 @@ extern "C" int mm_step(mm_ctx* c, int n, double dt) {
     }
     for (int s = 0; s < n;) {
         const int p = c->cur;
-        // single steps of the two-kernel path launch directly: a flushed
-        // 256x256x4 step measured 23.2-23.5 us so against 24.7 us as a
-        // one-step graph; runs of kGraphSteps replay their graph (17.0
-        // against 17.3 us per L2-resident step launched one by one)
-        if (c->use_graphs && (n - s >= kGraphSteps || !c->has_fs)) {
+        // A context's first kWarmSteps steps of a dt launch directly: a graph
+        // of 16 steps takes ~130 us to capture and instantiate and gains 0.3
+        // us per step (a first block of 20 steps of 256x256x4 took 507 us with
+        // the capture and 390 so).  Then runs of kGraphSteps replay their
+        // graph, and the remaining single steps of the two-kernel path launch
+        // directly (a flushed 256x256x4 step measured 23.2-23.5 us so against
+        // 24.7 us as a one-step graph).
+        if (c->warm_dt != dt || c->warm_ver != c->ver) {
+            c->warm_dt = dt;
+            c->warm_ver = c->ver;
+            c->warm = 0;
+        }
+        if (c->use_graphs && c->warm >= kWarmSteps && (n - s >= kGraphSteps || !c->has_fs)) {
             const int kind = n - s >= kGraphSteps ? 1 : 0;
             if (!c->step_exec[kind][p] || c->step_dt[kind][p] != dt || c->step_ver[kind][p] != c->ver) {
                 rc = capture_step(c, kind, p, dt);
@@ -775,6 +785,7 @@ extern "C" int mm_step(mm_ctx* c, int n, double dt) {
             if (rc != MM_OK) return rc;
             c->cur = 1 - p;
             ++s;
+            if (c->warm < kWarmSteps) ++c->warm;
         }
     }
     return MM_OK;
