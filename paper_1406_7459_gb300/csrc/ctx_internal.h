@@ -94,10 +94,18 @@ cudaError_t form_spectrum(mm_ctx* c, const float* M, cudaStream_t s, float* Mcop
                           const XComb& comb = XComb{});
 // Whether a Runge-Kutta stage of this context is the plane pass and one
 // kernel (fused_stage) instead of a field evaluation and a stage update.
-// Not where the plane kernel runs more than 512 threads (512x512x4: 472 us per
-// RK4 step fused, 440 with the three-pass field evaluations).
+// On films up to kFusedCells: there a stage saves two launches and passes
+// (us per RK4 step, fused against field evaluations and stage updates:
+// 256x256x4 70 against 80, 600x400x1 115 against 127, 200x300x6 201 against
+// 205); on larger ones the stage kernel's registers cost more than the passes
+// (400x480x2 213 against 211, 620x640x1 198 against 193, 512x512x4 408 against
+// 390, 1000x1000x1 513 against 408).  Not where the plane kernel runs more
+// than 512 threads.  Thick samples gain throughout (100x80x20 145 against
+// 148, 160x120x20 229 against 241, 256x256x16 369 against 375; 200x160x20 423
+// against 417).
+constexpr int kFusedCells = 370000;
 inline bool fused_stages(const mm_ctx* c) {
-    return c->has_fs ? c->rag || c->fs.ta <= 512 : c->has_ss && (c->rag || c->l.fx);
+    return c->has_fs ? c->g.N <= kFusedCells && (c->rag || c->fs.ta <= 512) : c->has_ss && (c->rag || c->l.fx);
 }
 // One stage at the state Y whose x spectrum is in S: the slope's use per st
 // (mode kModeStage, which leaves the next state's spectrum in S, or kModeErr).

@@ -347,6 +347,180 @@ __global__ void __launch_bounds__(PlaneLayout<NY, NZ>::THREADS, (PlaneLayout<NY,
     if (!early_trigger) pdl_trigger();
 }
 
+// ------------------------------------------------- K_A of large planes --
+// The plane kernel where a plane's threads or its spectrum slice do not fit
+// k_plane_pdl (transform groups of a whole warp, NY >= 320, several layers):
+// a warp takes whole lines, one after the other, and both halves of a line in
+// turn, so that no barrier separates them and a thread has the registers of
+// a 32-point transform; the tensor spectrum is read from global memory.  The
+// forward halves go to the line's two regions as in k_plane_pdl; the inverse
+// leaves the even half's outputs in region 0 and adds them to the odd half's
+// on the way out.  One CTA per SM: bound by the issue of its twelve warps.
+// Per L2-resident step: 512x512x4 112 us with k_plane_pdl's 768 threads, 94
+// so; 512x512x8 210 with the split pass, 191 so; 512x1024x4 217 against 167.
+template <int NY, int NZ> struct BigPlane {
+    using A = PlaneLayout<NY, NZ>;
+    using F = Fft2<NY>;
+    static_assert(F::G == 32, "a transform group is a warp");
+    static constexpr int THREADS = 384, WARPS = THREADS / 32;
+    static constexpr int TW_OFF = 0, TA_OFF = 2 * NY, WORK_OFF = 3 * NY;
+    static constexpr size_t BYTES = sizeof(float2) * (WORK_OFF + A::NL * A::ZS);
+};
+
+template <int NY, int NZ, bool RAG = false>
+__global__ void __launch_bounds__(BigPlane<NY, NZ>::THREADS)
+    k_plane_big(const __grid_constant__ Geom g, const float* __restrict__ Kd, const float2* __restrict__ S,
+                float2* __restrict__ Sh, int* __restrict__ flag, int early_trigger) {
+    using Big = BigPlane<NY, NZ>;
+    using Lay = PlaneLayout<NY, NZ>;
+    using F = Fft2<NY>;
+    constexpr int P = F::P, Q = F::Q, LY = Lay::LY, ZS = Lay::ZS, NL = Lay::NL, HALF = Lay::HALF, T = Big::THREADS;
+    extern __shared__ __align__(16) float2 sm[];
+    __shared__ __align__(8) uint64_t bars[2];             // twiddles, S lines
+    float2* tw = sm + Big::TW_OFF;
+    float2* ta = sm + Big::TA_OFF;
+    float2* zb = sm + Big::WORK_OFF;
+    const int kx = blockIdx.x;
+    const uint32_t b_tw = smem_addr(&bars[0]), b_s = smem_addr(&bars[1]);
+    if (threadIdx.x == 0) {
+        mbar_init(b_tw, 1);
+        mbar_init(b_s, 1);
+        mbar_init_fence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        mbar_expect_tx(b_tw, LY * sizeof(float2));
+        bulk_g2s(smem_addr(tw), g.twy, LY * sizeof(float2), b_tw);
+    }
+    pdl_wait();
+    if (early_trigger) pdl_trigger();
+    if (threadIdx.x == 0) {
+        proxy_fence_global();                             // S came from ordinary stores
+        const float2* plane = S + (size_t)kx * NL * g.Jst;
+        const uint32_t ln = (uint32_t)((RAG ? g.Jst : NY) * sizeof(float2));
+        mbar_expect_tx(b_s, NL * ln);
+#pragma unroll 1
+        for (int l = 0; l < NL; ++l) bulk_g2s(smem_addr(zb + l * ZS), plane + (size_t)l * g.Jst, ln, b_s);
+    }
+    bool ok = mbar_wait(b_tw, 0);
+    if (ok) fill_ta<NY, Q, T>(ta, tw);
+    ok = mbar_wait(b_s, 0) && ok;
+    if (__syncthreads_or(!ok)) {
+        if (threadIdx.x == 0) {
+            atomicOr(flag, kFlagTimeout);
+            mbar_wait(b_tw, 0);                           // the copies in flight land first (bounded)
+            mbar_wait(b_s, 0);
+        }
+        __syncthreads();
+        return;
+    }
+    const int t = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // forward y of whole lines
+#pragma unroll 1
+    for (int l = warp; l < NL; l += Big::WARPS) {
+        float2* r0 = zb + l * ZS;
+        float2 v[P];
+        if (t < Q) {
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                if constexpr (RAG)
+                    v[q] = t + Q * q < g.Jst ? r0[t + Q * q] : make_float2(0.f, 0.f);
+                else
+                    v[q] = r0[t + Q * q];
+            }
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int h = 1; h >= 0; --h) {
+            float2* rf = r0 + h * HALF;
+            if (t < Q) {
+                float2 x[P];
+#pragma unroll
+                for (int q = 0; q < P; ++q) x[q] = v[q];
+                if (h) F::odd_input_tab(x, t, tw);
+                F::stepA_tab(x, t, ta, rf, false);
+            }
+            __syncwarp();
+            float2 w[Q];
+            if (t < P) F::stepB(w, t, rf, false);
+            __syncwarp();
+            if (t < P) {
+#pragma unroll
+                for (int q = 0; q < Q; ++q) rf[t + P * q] = w[q];
+            }
+        }
+    }
+    __syncthreads();
+    // z part of the convolution, one (ky) column per thread (plane_body)
+    const float* __restrict__ Kx = Kd + (size_t)kx * Lay::KT_FLOATS;
+#pragma unroll 1
+    for (int col = threadIdx.x; col < LY; col += T) {
+        const int hh = col / NY, mm = col - hh * NY;      // ky = 2 mm + hh
+        const int ky = 2 * mm + hh;
+        const int e = hh * HALF + mm;
+        int kyp = ky;
+        float sy = 1.f;
+        if (2 * ky > LY) { kyp = LY - ky; sy = -1.f; }
+        kyp = (kyp & 1) ? Lay::KY_EVEN + (kyp >> 1) : (kyp >> 1);
+        float d[NZ][6];
+#pragma unroll
+        for (int dz = 0; dz < NZ; ++dz)
+#pragma unroll
+            for (int c = 0; c < 6; ++c)
+                d[dz][c] = (c == 1 || c == 4 ? sy : 1.f) * __ldg(Kx + (dz * 6 + c) * Lay::HYP + kyp);
+        float2 m[3][NZ];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int k = 0; k < NZ; ++k) m[c][k] = zb[(c * NZ + k) * ZS + e];
+#pragma unroll
+        for (int k = 0; k < NZ; ++k) m[2][k] = make_float2(-m[2][k].y, m[2][k].x);   // i M_z
+        auto coef = [&](int dz, int c) -> float { return d[dz][c]; };
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            float2 hres[NZ];
+            zdirect_task<NZ>(m, coef, a, hres);
+#pragma unroll
+            for (int k = 0; k < NZ; ++k)
+                zb[(a * NZ + k) * ZS + e] = (a == 2) ? make_float2(hres[k].y, -hres[k].x) : hres[k];   // -i H_z'
+        }
+    }
+    __syncthreads();
+    // inverse y, pruned output
+    float2* outp = Sh + (size_t)kx * NL * g.Jst;
+#pragma unroll 1
+    for (int l = warp; l < NL; l += Big::WARPS) {
+        float2* r0 = zb + l * ZS;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            float2* ri = r0 + h * HALF;
+            float2 v[P];
+            if (t < Q) {
+#pragma unroll
+                for (int q = 0; q < P; ++q) v[q] = ri[t + Q * q];
+            }
+            __syncwarp();
+            if (t < Q) F::stepA_tab(v, t, ta, ri, true);
+            __syncwarp();
+            float2 w[Q];
+            if (t < P) {
+                F::stepB(w, t, ri, true);
+                if (h) F::odd_output_tab(w, t, tw);
+            }
+            __syncwarp();
+            if (t < P) {
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    const int n = t + P * q;
+                    if (h == 0) r0[n] = w[q];             // read back by this thread
+                    else if (!RAG || n < g.Jst) outp[(size_t)l * g.Jst + n] = cadd(r0[n], w[q]);
+                }
+            }
+        }
+    }
+    if (!early_trigger) pdl_trigger();
+}
+
 // ------------------------------------------------------------- K_B xstep --
 template <int N, int R> struct XstepLayout {
     static_assert(R == 2 || R == 4, "row pairs per tile: a pair shares one complex transform");

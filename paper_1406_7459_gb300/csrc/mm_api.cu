@@ -204,9 +204,10 @@ static int build_plan(mm_ctx* c) {
             c->fsplit.sz <= smem_cap)
             l.fs2 = &c->fsplit;
         FastStepFns& s = c->fs;
-        bool ok = fast_step_lookup_x(g.nx, &s);
-        ok = ok && (fast_step_lookup_plane_a(g.ny, g.nz, &s) || fast_step_lookup_plane_b(g.ny, g.nz, &s));
-        ok = ok && l.fx && !l.split && g.ny % s.rb == 0 && s.sa <= smem_cap && s.sb <= smem_cap;
+        const bool ok_x = fast_step_lookup_x(g.nx, &s);
+        bool ok = ok_x && (fast_step_lookup_plane_a(g.ny, g.nz, &s) || fast_step_lookup_plane_b(g.ny, g.nz, &s));
+        const bool big = ok_x && g.Hx >= kBigPlanes && fast_step_lookup_plane_big(g.ny, g.nz, &s);
+        ok = (ok || big) && l.fx && (!l.split || big) && g.ny % s.rb == 0 && s.sa <= smem_cap && s.sb <= smem_cap;
         // the x-step kernel indexes the spectrum and M with 32-bit offsets
         ok = ok && 3.0 * g.Hx * g.nz * g.Jst < (double)INT_MAX && 3.0 * g.N < (double)INT_MAX;
         c->has_fs = ok;
@@ -393,7 +394,7 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
             int sms = 0;
             CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
             c->fs.early = c->rag ? ragged_early_trigger(gf, c->fs, sms) : fast_step_early_trigger(gf, c->fs, sms);
-            if (!c->rag) encode_xstep_maps(g, &c->fs, c->Sh, c->S);   // per-thread copies where no map applies
+            if (!c->rag && !c->fs.big) encode_xstep_maps(g, &c->fs, c->Sh, c->S);   // per-thread copies where no map applies
         }
         if (c->has_persist) {
             bool usable = false;

@@ -191,6 +191,7 @@ struct FastStepFns {
     int early = 0;             // K_A triggers K_B right after its wait (fast_step_early_trigger)
     int ta = 0;
     size_t sa = 0;
+    bool big = false;          // ka is the large-plane kernel (one CTA per SM)
     // x-step kernels by Pass3Mode: demag field, effective field, Euler step
     void (*kb[3])(Geom, LlgCoef, const float2*, float2*, const float*, float*, int*, float*) = {nullptr, nullptr,
                                                                                                nullptr};
@@ -224,6 +225,10 @@ bool encode_xstep_maps(const Geom& g, FastStepFns* f, const float2* Sh, const fl
 bool fast_step_lookup_x(int nx, FastStepFns* f);
 bool fast_step_lookup_plane_a(int ny, int nz, FastStepFns* f);
 bool fast_step_lookup_plane_b(int ny, int nz, FastStepFns* f);
+bool fast_step_lookup_plane_big(int ny, int nz, FastStepFns* f);   // fast_step_plane_big.cu
+// Planes from which on the large-plane kernel (one CTA per SM) is used: one
+// for each SM.
+constexpr int kBigPlanes = 152;
 // Ragged films (ragged.cuh): the kernels and the carrier lengths NX >= nx,
 // NY >= ny; whether the plane kernel triggers the x-step early.
 bool ragged_lookup_x(int nx, FastStepFns* f, int* NX);

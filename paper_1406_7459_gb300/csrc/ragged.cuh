@@ -30,12 +30,31 @@ inline int ragged_len(int n) {
     return 0;
 }
 
-// Plane kernels exist where a plane's threads and shared memory fit.
+// k_plane_pdl exists where a plane's threads and shared memory fit, the
+// large-plane kernel for transform groups of a warp where its lines fit.
 template <int NY, int NZ> constexpr bool rag_plane_fits() {
     return PlaneLayout<NY, NZ>::THREADS <= 768 && PlaneLayout<NY, NZ>::BYTES <= 227 * 1024;
 }
+template <int NY, int NZ> constexpr bool big_plane_fits() {
+    if constexpr (Fft2<NY>::G == 32) return BigPlane<NY, NZ>::BYTES <= 226 * 1024;
+    else return false;
+}
 
-template <int NY, int NZ> bool rag_fill_plane(FastStepFns* f) {
+// many: the planes fill the SMs (kBigPlanes).  Then the large-plane kernel
+// takes the planes of more than 512 threads, whose registers spill in
+// k_plane_pdl, and those that do not fit it; fewer of them run better on
+// k_plane_pdl or on the split pass.
+template <int NY, int NZ> bool rag_fill_plane(bool many, FastStepFns* f) {
+    if constexpr (big_plane_fits<NY, NZ>() &&
+                  (PlaneLayout<NY, NZ>::THREADS > 512 || !rag_plane_fits<NY, NZ>())) {
+        if (many) {
+            f->ka = k_plane_big<NY, NZ, true>;
+            f->ta = BigPlane<NY, NZ>::THREADS;
+            f->sa = BigPlane<NY, NZ>::BYTES;
+            f->big = true;
+            return true;
+        }
+    }
     if constexpr (rag_plane_fits<NY, NZ>()) {
         f->ka = k_plane_pdl<NY, NZ, true>;
         f->ta = PlaneLayout<NY, NZ>::THREADS;
@@ -47,27 +66,27 @@ template <int NY, int NZ> bool rag_fill_plane(FastStepFns* f) {
 }
 
 // NZ layers, carrier NY, for the lengths of [0, 7) or [7, 14) of kRagLens
-template <int NZ> bool rag_lookup_plane_lo(int NY, FastStepFns* f) {
+template <int NZ> bool rag_lookup_plane_lo(int NY, bool many, FastStepFns* f) {
     switch (NY) {
-        case 16: return rag_fill_plane<16, NZ>(f);
-        case 32: return rag_fill_plane<32, NZ>(f);
-        case 48: return rag_fill_plane<48, NZ>(f);
-        case 64: return rag_fill_plane<64, NZ>(f);
-        case 96: return rag_fill_plane<96, NZ>(f);
-        case 128: return rag_fill_plane<128, NZ>(f);
-        case 192: return rag_fill_plane<192, NZ>(f);
+        case 16: return rag_fill_plane<16, NZ>(many, f);
+        case 32: return rag_fill_plane<32, NZ>(many, f);
+        case 48: return rag_fill_plane<48, NZ>(many, f);
+        case 64: return rag_fill_plane<64, NZ>(many, f);
+        case 96: return rag_fill_plane<96, NZ>(many, f);
+        case 128: return rag_fill_plane<128, NZ>(many, f);
+        case 192: return rag_fill_plane<192, NZ>(many, f);
         default: return false;
     }
 }
-template <int NZ> bool rag_lookup_plane_hi(int NY, FastStepFns* f) {
+template <int NZ> bool rag_lookup_plane_hi(int NY, bool many, FastStepFns* f) {
     switch (NY) {
-        case 256: return rag_fill_plane<256, NZ>(f);
-        case 320: return rag_fill_plane<320, NZ>(f);
-        case 384: return rag_fill_plane<384, NZ>(f);
-        case 512: return rag_fill_plane<512, NZ>(f);
-        case 640: return rag_fill_plane<640, NZ>(f);
-        case 768: return rag_fill_plane<768, NZ>(f);
-        case 1024: return rag_fill_plane<1024, NZ>(f);
+        case 256: return rag_fill_plane<256, NZ>(many, f);
+        case 320: return rag_fill_plane<320, NZ>(many, f);
+        case 384: return rag_fill_plane<384, NZ>(many, f);
+        case 512: return rag_fill_plane<512, NZ>(many, f);
+        case 640: return rag_fill_plane<640, NZ>(many, f);
+        case 768: return rag_fill_plane<768, NZ>(many, f);
+        case 1024: return rag_fill_plane<1024, NZ>(many, f);
         default: return false;
     }
 }

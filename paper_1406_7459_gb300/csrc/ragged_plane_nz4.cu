@@ -3,8 +3,8 @@
 
 namespace mmk {
 
-bool ragged_lookup_plane_nz4(int NY, FastStepFns* f) {
-    return rag_lookup_plane_lo<4>(NY, f) || rag_lookup_plane_hi<4>(NY, f);
+bool ragged_lookup_plane_nz4(int NY, bool many, FastStepFns* f) {
+    return rag_lookup_plane_lo<4>(NY, many, f) || rag_lookup_plane_hi<4>(NY, many, f);
 }
 
 }  // namespace mmk

@@ -3,8 +3,8 @@
 
 namespace mmk {
 
-bool ragged_lookup_plane_nz8(int NY, FastStepFns* f) {
-    return rag_lookup_plane_lo<8>(NY, f) || rag_lookup_plane_hi<8>(NY, f);
+bool ragged_lookup_plane_nz8(int NY, bool many, FastStepFns* f) {
+    return rag_lookup_plane_lo<8>(NY, many, f) || rag_lookup_plane_hi<8>(NY, many, f);
 }
 
 }  // namespace mmk

@@ -8,14 +8,14 @@ bool ragged_lookup_x_a(int N, FastStepFns* f);
 bool ragged_lookup_x_b(int N, FastStepFns* f);
 bool ragged_lookup_x_c(int N, FastStepFns* f);
 bool ragged_lookup_x_d(int N, FastStepFns* f);
-bool ragged_lookup_plane_nz1(int NY, FastStepFns* f);
-bool ragged_lookup_plane_nz2(int NY, FastStepFns* f);
-bool ragged_lookup_plane_nz3(int NY, FastStepFns* f);
-bool ragged_lookup_plane_nz4(int NY, FastStepFns* f);
-bool ragged_lookup_plane_nz5(int NY, FastStepFns* f);
-bool ragged_lookup_plane_nz6(int NY, FastStepFns* f);
-bool ragged_lookup_plane_nz7(int NY, FastStepFns* f);
-bool ragged_lookup_plane_nz8(int NY, FastStepFns* f);
+bool ragged_lookup_plane_nz1(int NY, bool many, FastStepFns* f);
+bool ragged_lookup_plane_nz2(int NY, bool many, FastStepFns* f);
+bool ragged_lookup_plane_nz3(int NY, bool many, FastStepFns* f);
+bool ragged_lookup_plane_nz4(int NY, bool many, FastStepFns* f);
+bool ragged_lookup_plane_nz5(int NY, bool many, FastStepFns* f);
+bool ragged_lookup_plane_nz6(int NY, bool many, FastStepFns* f);
+bool ragged_lookup_plane_nz7(int NY, bool many, FastStepFns* f);
+bool ragged_lookup_plane_nz8(int NY, bool many, FastStepFns* f);
 
 bool ragged_lookup_x(int nx, FastStepFns* f, int* NX) {
     *NX = ragged_len(nx);
@@ -25,16 +25,17 @@ bool ragged_lookup_x(int nx, FastStepFns* f, int* NX) {
 
 bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY) {
     *NY = ragged_len(ny);
+    const bool many = ragged_len(nx) + 1 >= kBigPlanes;
     bool ok = false;
     switch (nz) {
-        case 1: ok = ragged_lookup_plane_nz1(*NY, f); break;
-        case 2: ok = ragged_lookup_plane_nz2(*NY, f); break;
-        case 3: ok = ragged_lookup_plane_nz3(*NY, f); break;
-        case 4: ok = ragged_lookup_plane_nz4(*NY, f); break;
-        case 5: ok = ragged_lookup_plane_nz5(*NY, f); break;
-        case 6: ok = ragged_lookup_plane_nz6(*NY, f); break;
-        case 7: ok = ragged_lookup_plane_nz7(*NY, f); break;
-        case 8: ok = ragged_lookup_plane_nz8(*NY, f); break;
+        case 1: ok = ragged_lookup_plane_nz1(*NY, many, f); break;
+        case 2: ok = ragged_lookup_plane_nz2(*NY, many, f); break;
+        case 3: ok = ragged_lookup_plane_nz3(*NY, many, f); break;
+        case 4: ok = ragged_lookup_plane_nz4(*NY, many, f); break;
+        case 5: ok = ragged_lookup_plane_nz5(*NY, many, f); break;
+        case 6: ok = ragged_lookup_plane_nz6(*NY, many, f); break;
+        case 7: ok = ragged_lookup_plane_nz7(*NY, many, f); break;
+        case 8: ok = ragged_lookup_plane_nz8(*NY, many, f); break;
         default: break;
     }
     return ok && ragged_lookup_x(nx, f, NX);

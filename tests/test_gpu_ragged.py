@@ -68,6 +68,42 @@ def test_ragged_film_fields_and_steps(grid):
     assert rel_l2(host(out) - M64, ref - M64) < 1e-4
 
 
+# planes of the large-plane kernel: each of its line lengths at its first and
+# last line count, the fewest planes that take it, and the power-of-two ones
+BIG = [(129, 257, 5), (130, 320, 8), (129, 321, 3), (130, 384, 7), (129, 385, 4), (129, 511, 8), (131, 513, 3),
+       (129, 640, 6), (129, 641, 5), (130, 768, 3), (129, 769, 3), (129, 1023, 4), (256, 512, 4), (256, 512, 8),
+       (256, 1024, 4)]
+
+
+@pytest.mark.parametrize("grid", BIG)
+def test_large_planes_field_and_steps(grid):
+    """Field, Euler steps and a Heun step of films whose planes one block takes
+    a line per warp at a time: two kernels, and the oracle's values."""
+    from paper_1406_7459_gb300 import mm
+    cell, Hext, dt = (4e-9, 3e-9, 5e-9), (1e4, -5e3, 2e3), 2e-14
+    M = inputs.random_unit_m(grid, MS, seed=sum(grid))
+    ctx = mm.mm_create(grid, cell, MS, A_EX, 2e4, 0.2, GAMMA)
+    assert mm.mm_plan_info(ctx)[1] == 2
+    mm.mm_set_field(ctx, Hext)
+    Md = torch.from_numpy(M.reshape(-1)).cuda()
+    out = torch.full_like(Md, float("nan"))
+    Kt, Lp = oracle_spectrum(grid, cell)
+    M64 = M.astype(np.float64)
+    mm.mm_demag_field(ctx, Md, out)
+    Hd = D.demag_fft(M64, Kt, Lp)
+    got = out.cpu().numpy().reshape(Hd.shape)
+    assert rel_l2(got, Hd) < 1e-5 and rel_max(got, Hd) < 1e-5
+    mm.mm_set_m(ctx, Md)
+    mm.mm_step(ctx, 2, dt)
+    mm.mm_set_integrator(ctx, "heun")
+    mm.mm_step(ctx, 1, dt)
+    mm.mm_get_m(ctx, out)
+    mm.mm_sync(ctx)
+    args = (cell, MS, A_EX, 2e4, 0.2, GAMMA, Hext, Kt, Lp)
+    ref = L.run_rk(L.run_euler(M64, 2, dt, *args), 1, dt, "heun", *args)
+    assert rel_l2(out.cpu().numpy().reshape(ref.shape) - M64, ref - M64) < 1e-4
+
+
 def test_ragged_spectrum_is_formed_on_demand():
     """The stored-spectrum entry points of a ragged film, whose steps do not
     read that spectrum: the same padded lengths and values as the oracle's,
