@@ -110,10 +110,13 @@ int mm_destroy(mm_ctx *ctx);
 /*
  * mm_set_integrator -- choose the time stepper of mm_step.  Forward Euler
  * (Table 1 caption) is the default and runs as the two-kernel step on
- * power-of-two grids.  Heun and classic RK4 go beyond the paper: each stage
- * evaluates H_eff of the stage state with the same three demag/field passes,
- * stage states are not renormalised, the new state is renormalised to
- * |M| = Ms.  They allocate two extra 3*N float32 buffers on first use.
+ * films.  Heun and classic RK4 go beyond the paper: each stage evaluates
+ * H_eff of the stage state, either with the three demag/field passes and a
+ * stage update or, on films up to 370000 cells and on thick samples, with the
+ * stage update and the next stage's x transform fused into the last of them
+ * (the same arithmetic); stage states are not renormalised, the new state is
+ * renormalised to |M| = Ms.  They allocate two extra 3*N float32 buffers on
+ * first use.
  * Returns MM_EINVAL for an unknown method, MM_ENOMEM on allocation failure.
  */
 int mm_set_integrator(mm_ctx *ctx, int method);
@@ -123,7 +126,8 @@ int mm_set_integrator(mm_ctx *ctx, int method);
  * M with the embedded Dormand-Prince RK5(4) pair and step-size control
  * (beyond the paper, whose scheme is forward Euler, Table 1 caption).
  * Every stage evaluates H_eff of its (plain, not renormalised) stage state
- * with the three demag/field passes; the fifth-order state is renormalised
+ * (with the stage fused into the x kernel where mm_set_integrator says so);
+ * the fifth-order state is renormalised
  * to |M| = Ms; the seventh stage is the right-hand side at that state and
  * is reused as the first stage of the next step.  The error of a trial step
  * is err = max over cells |dt sum_i e_i k_i| / Ms (e: fifth- minus fourth-
@@ -191,8 +195,11 @@ int mm_effective_field(mm_ctx *ctx, const float *M_dev, float *H_dev);
  * + inverse y/z; inverse x C2R fused with exchange, anisotropy, Zeeman, LLG,
  * Euler and renormalisation); the update kernel also forms the next step's
  * x R2C, so a film step is two kernels (on power-of-two films the exchange
- * stencil rides in the tensor spectrum) and a thick sample's four; steps are
- * replayed from CUDA graphs of 16 steps (the remainder one step each).
+ * stencil rides in the tensor spectrum) and a thick sample's four.  Sides
+ * that are no powers of two up to 1023 are carried in the next compile-time
+ * transform length.  The first 128 steps of a dt are launched directly; from
+ * then on steps are replayed from CUDA graphs of 16 (the remainder one step
+ * each).
  * On the square power-of-two films the persistent step is built for
  * (64, 128, 256 wide with nz = 4; 256 x 256 with nz = 1 or 2) the two
  * kernels' work can instead run as one cooperative launch for up to 1024
@@ -301,7 +308,9 @@ int mm_tensor_octant(mm_ctx *ctx, double *out);
  * divided by Lx*Ly*Lz (the inverse-FFT normalisation is folded in), on the
  * octant 0..L/2 of each axis: out holds (Lx/2+1)*(Lz/2+1)*(Ly/2+1)*6 floats
  * laid out [kx][kz][ky][component].  Host or device.  Synchronises.
- * Diagnostic; not on the per-step path.
+ * Diagnostic; not on the per-step path: where the steps read another form of
+ * the spectrum (films with a side that is no power of two), this one is formed
+ * by the first call that wants it.
  */
 int mm_kernel_spectrum(mm_ctx *ctx, float *out);
 
@@ -325,13 +334,15 @@ int mm_time_passes(mm_ctx *ctx, int reps, double dt, void *flush, unsigned long 
  * size slowness on launch overhead, which batching removes).  Sample s has
  * its own grid (nz <= 4), cell, material, field and tensor spectrum; every
  * call of mm_batch_step advances all samples by forward-Euler steps of the
- * same dt, with two batched kernels per step (the plane pass; the update,
- * which also forms the next step's x spectra) replayed from a CUDA graph
- * after one x transform of a new state, or (mm_batch_set_path
- * MM_STEP_PERSISTENT) as one cooperative launch for up to 1024 steps whose
- * blocks take (sample, tile) items from a work queue per pass, the passes
- * separated by bounded grid barriers (same arithmetic); that launch is
- * captured in a CUDA graph and replayed while its arguments stay the same.
+ * same dt, with the plane pass and then the update, which also forms the
+ * next step's x spectra, after one x transform of a new state.  Samples
+ * whose sides fit the compile-time transform lengths are grouped into a few
+ * classes of kernel (mm_batch_autotune's shapes apply to the others); eight
+ * steps are launched directly, later ones replayed from a CUDA graph.  Or
+ * (mm_batch_set_path MM_STEP_PERSISTENT) one cooperative launch runs up to
+ * 1024 steps: its blocks take (sample, tile) items from a work queue per pass,
+ * the passes separated by bounded grid barriers (same arithmetic); that launch
+ * is captured in a CUDA graph and replayed while its arguments stay the same.
  * M arrays of a batch are the samples' SoA blocks back to back (sample s
  * starts at float offset sum_{t<s} 3 N_t).
  * ------------------------------------------------------------------------ */
@@ -368,9 +379,11 @@ int mm_batch_launch_form(const mm_batch *b);
  * steps of size dt, keep the fastest, and restore the state (tuning does not
  * advance the samples): first the rows per CTA of the x passes and the
  * threads per CTA (12 candidates), then, with those, the kx planes per CTA
- * of the plane pass (1, 2, 4, 8).  choice (may be NULL): {rows pass 1, rows
- * pass 3, threads, planes per CTA}; ms_out (may be NULL): 16 floats, mean ms
- * per step of each candidate in that order.  Synchronises.
+ * of the plane pass (1, 2, 4, 8).  They shape the general kernels: samples on
+ * the compile-time classes run the same under every candidate.  choice (may
+ * be NULL): {rows pass 1, rows pass 3, threads, planes per CTA}; ms_out (may
+ * be NULL): 16 floats, mean ms per step of each candidate in that order.
+ * Synchronises.
  */
 int mm_batch_autotune(mm_batch *b, double dt, int choice[4], float *ms_out);
 

@@ -364,30 +364,33 @@ __device__ __forceinline__ void tc_cp16(uint32_t dst, const void* src, bool in) 
 }
 
 // Rows r0 .. r0 + ROWS - 1 of a K-contiguous operand (row stride `rs`,
-// `rows` of them in all) into the tile at shared address dst.
+// `rows` of them in all) into the tile at shared address dst.  Chunk e of the
+// tile as it is laid out goes to thread e: a warp fills 512 consecutive bytes
+// of shared memory and reads eight rows of 64 bytes; a warp on one row of 512
+// bytes would fill chunks 128 bytes apart, all in the same four banks
+// (65536 x 32 x 256, bound by the load latency of its two waves of CTAs: 18.9
+// us so, 18.75 with the order here).
 template <int ROWS>
 __device__ __forceinline__ void tc_load_rows(uint32_t dst, const __nv_bfloat16* __restrict__ P, int r0, int rows,
-                                             int K, int KC, long long rs, bool vec, uint32_t sbo) {
+                                             int K, int KC, long long rs, bool vec) {
     if (vec) {
         for (int e = threadIdx.x; e < ROWS * KC; e += kTcThreads) {
-            const int r = e / KC, c = e - r * KC;
+            const int q = e >> 3, g = q / KC, r = 8 * g + (e & 7), c = q - g * KC;
             const bool in = r0 + r < rows && 8 * c < K;
-            tc_cp16(dst + (uint32_t)((r >> 3) * sbo + c * 128 + (r & 7) * 16),
-                    in ? (const void*)(P + (long long)(r0 + r) * rs + 8 * c) : (const void*)P, in);
+            tc_cp16(dst + 16u * e, in ? (const void*)(P + (long long)(r0 + r) * rs + 8 * c) : (const void*)P, in);
         }
         return;
     }
     const unsigned short* p16 = reinterpret_cast<const unsigned short*>(P);
 #pragma unroll 2
     for (int e = threadIdx.x; e < ROWS * KC; e += kTcThreads) {
-        const int r = e / KC, c = e - r * KC;
+        const int q = e >> 3, g = q / KC, r = 8 * g + (e & 7), c = q - g * KC;
         const unsigned short* p = p16 + (long long)(r0 + r) * rs + 8 * c;
         unsigned h[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) h[j] = r0 + r < rows && 8 * c + j < K ? __ldg(p + j) : 0u;
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
-                         dst + (uint32_t)((r >> 3) * sbo + c * 128 + (r & 7) * 16)),
-                     "r"(h[0] | h[1] << 16), "r"(h[2] | h[3] << 16), "r"(h[4] | h[5] << 16), "r"(h[6] | h[7] << 16)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + 16u * e), "r"(h[0] | h[1] << 16),
+                     "r"(h[2] | h[3] << 16), "r"(h[4] | h[5] << 16), "r"(h[6] | h[7] << 16)
                      : "memory");
     }
 }
@@ -419,8 +422,8 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc_kfull(GemmArgs a) {
     auto vec = [&](const void* p, long long rs, long long z) {
         return a.K % 8 == 0 && rs % 8 == 0 && z % 8 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
     };
-    tc_load_rows<kTcM>(As_s, A, m0, a.M, a.K, KC, a.sam, vec(a.A, a.sam, a.zA), sbo);
-    tc_load_rows<BN>(Bs_s, B, n0, a.N, a.K, KC, a.sbn, vec(a.B, a.sbn, a.zB), sbo);
+    tc_load_rows<kTcM>(As_s, A, m0, a.M, a.K, KC, a.sam, vec(a.A, a.sam, a.zA));
+    tc_load_rows<BN>(Bs_s, B, n0, a.N, a.K, KC, a.sbn, vec(a.B, a.sbn, a.zB));
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (warp == 0) {
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&tmem_base);
@@ -477,9 +480,13 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc_kfull(GemmArgs a) {
 }
 
 // Dynamic shared memory of k_gemm_tc_kfull<BN> for a given K: the tiles,
-// padded like gemm_tc_smem so that at most 512 / BN CTAs share an SM.
+// padded so that no more than 512 / BN CTAs share an SM's 512 TMEM columns
+// (of its 228 KB, 1 KB goes to each CTA beside its own).  For BN = 128 that
+// is four CTAs, where a share of 1 / 4 of the SM left room for three: 65536 x
+// 256 x 32, bound by the epilogue's stores, 25.8 us with three and 24.6 with
+// four.
 template <int BN> constexpr size_t gemm_tc_kfull_floor() {
-    constexpr size_t share = 227 * 1024 / (512 / BN) + 1024, buf = 4 * 32 * kTcBufRow * sizeof(float);   // epilogue
+    constexpr size_t share = 228 * 1024 / (512 / BN + 1), buf = 4 * 32 * kTcBufRow * sizeof(float);   // epilogue
     return share > buf ? share : buf;
 }
 template <int BN> inline size_t gemm_tc_kfull_smem(int K) {
