@@ -13,6 +13,8 @@
 // accumulator in tensor memory, gemm_tc.cuh); the small complex transforms along y and the per-mode
 // channel mix run as FP32 kernels.  Parameters live as an FP32 master copy
 // (Adam moments beside it) and a BF16 copy for the GEMMs.
+#include <algorithm>
+
 #include <cuda_bf16.h>
 #include <cuda_pipeline.h>
 #include <cuda_runtime.h>
@@ -93,7 +95,7 @@ static cudaError_t gemm(GemmArgs g, int batch, int* err, cudaStream_t s, bool pd
 __global__ void k_ydft_blk(const float* __restrict__ A, int ldA, int H, int m, const float* __restrict__ Fre,
                            const float* __restrict__ Fim, int ny_out, float* __restrict__ ore,
                            float* __restrict__ oim, float scale, int double_kx, int S);
-constexpr int kYdftThreads = 256;
+constexpr int kYdftThreads = 256, kYdftBlocks = 512;
 constexpr size_t kYdftSmemMax = 200 * 1024;
 
 static cudaError_t gemm_configure() {
@@ -557,8 +559,10 @@ __device__ __forceinline__ float gelu_as(float x) {
 // 16-byte shared reads feeds 4 OC multiply-adds (two pixels per
 // instruction), and reads and writes its u, v' as whole pixel quads.  PROJ
 // (the last layer): no activation, and the projection y[b][j][p] = sum_o
-// Q[j][o] v'[b][o][p] + q[j] (3 outputs) summed over the channel groups
-// through shared memory, so that v' is not stored unless TRAIN.
+// Q[j][o] v'[b][o][p] + q[j] (3 outputs) from the tile's v' in shared
+// memory, in SG partial sums, so that v' is not stored unless TRAIN and every
+// tile shape gives the same bits (a last bit of y turns up as BF16 roundings
+// of the whole backward pass).
 // Small films take 64-pixel tiles with as many threads, each with fewer
 // channels, so that every SM has work (mix_launch_t).
 template <int CW> struct MixSmall {
@@ -572,9 +576,10 @@ __global__ void __launch_bounds__(T) k_mix_bias_act(float* __restrict__ u, const
                                                       const float* __restrict__ qb, float* __restrict__ yout) {
     constexpr int GR = CW / OC, QUADS = T / GR, TP = 4 * QUADS;
     constexpr int TRIPS = CW * QUADS / T;
+    constexpr int SG = CW <= 32 ? 4 : 8;                   // partial sums of the projection, one order for all tiles
     __shared__ __align__(16) float Wt[CW * CW];            // [c][o]
     __shared__ __align__(16) uint2 vs[CW * QUADS];         // v, four pixels per element
-    __shared__ __align__(16) float ps[PROJ ? 3 * GR * TP : 4];
+    __shared__ __align__(16) float ps[PROJ ? CW * TP : 4];  // v' of the tile
     pdl_wait();
     pdl_trigger();
     for (int i = threadIdx.x; i < CW * CW; i += T) Wt[(i % CW) * CW + i / CW] = Wl[i];
@@ -641,8 +646,6 @@ __global__ void __launch_bounds__(T) k_mix_bias_act(float* __restrict__ u, const
                 hi[j] = fma2(ww, d, hi[j]);
             }
         }
-        float4 y[3];
-        if constexpr (PROJ) y[0] = y[1] = y[2] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int j = 0; j < OC; ++j) {
             const float4 s = make_float4(lo[j].x, lo[j].y, hi[j].x, hi[j].y);
@@ -664,27 +667,23 @@ __global__ void __launch_bounds__(T) k_mix_bias_act(float* __restrict__ u, const
                     if (p + 3 < np) r[3] = __float2bfloat16(g.w);
                 }
             }
-            if constexpr (PROJ) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const float q = __ldg(Q + k * CW + o0 + j);
-                    y[k].x = fmaf(q, g.x, y[k].x);
-                    y[k].y = fmaf(q, g.y, y[k].y);
-                    y[k].z = fmaf(q, g.z, y[k].z);
-                    y[k].w = fmaf(q, g.w, y[k].w);
-                }
-            }
+            if constexpr (PROJ) *reinterpret_cast<float4*>(ps + (o0 + j) * TP + 4 * qd) = g;
         }
         if constexpr (PROJ) {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) *reinterpret_cast<float4*>(ps + (k * GR + og) * TP + 4 * qd) = y[k];
             __syncthreads();
             const long long p0 = (tile - (long long)b * tpb) * TP;
             for (int e = threadIdx.x; e < 3 * TP; e += T) {
                 const int k = e / TP, i = e % TP;
                 if (p0 + i >= np) continue;
                 float s = __ldg(qb + k);
-                for (int g = 0; g < GR; ++g) s += ps[(k * GR + g) * TP + i];
+#pragma unroll
+                for (int g = 0; g < SG; ++g) {
+                    float t = 0.f;
+#pragma unroll
+                    for (int o = g * (CW / SG); o < (g + 1) * (CW / SG); ++o)
+                        t = fmaf(__ldg(Q + k * CW + o), ps[o * TP + i], t);
+                    s += t;
+                }
                 yout[((long long)b * 3 + k) * np + p0 + i] = s;
             }
         }
@@ -1053,7 +1052,7 @@ static cudaError_t mode_inv_batch(const mm_fno* f, int l, int B, const float* vr
     const int C = f->C, m = f->m, nmode = 2 * m * m;
     if (B < 4 || m % 4 != 0) return mode_inv(f, l, B, vr, vi, conjT, s, true);
     const long long ro = (long long)l * C * C * nmode;
-    cudaError_t e = launch_k(k_mode_mix, dim3((nmode + 31) / 32, C), 128, 0, s, true, vr, vi,
+    cudaError_t e = launch_k(k_mode_mix, dim3((nmode + 31) / 32, C, (B + kMixNB - 1) / kMixNB), 128, 0, s, true, vr, vi,
                              (const float*)(f->w + f->oRr + ro), (const float*)(f->w + f->oRi + ro), C, nmode, B,
                              conjT, f->wmr, f->wmi);
     if (e != cudaSuccess) return e;
@@ -1068,15 +1067,25 @@ static cudaError_t mode_inv_batch(const mm_fno* f, int l, int B, const float* vr
 static cudaError_t ydft(const mm_fno* f, const float* A, int BC, float* ore, float* oim, float scale, int double_kx,
                         cudaStream_t s, bool pdl = false) {
     const int m = f->m, H = f->H, ny = 2 * m;
-    // iy groups per slab: enough blocks to spread over the SMs
+    // iy groups per slab and y shares per output; then, with the same shares
+    // (the order of the sums), smaller groups of fewer threads up to
+    // kYdftBlocks blocks, which fill the SMs evenly: 256 x 256, width 32, 16
+    // modes, one forward pass 161 us with the first split alone and 157 with
+    // 512 blocks, loss and gradients at batch 8 1733 us with 256 blocks of 256
+    // threads, 1648 with 512 of 128 and 1681 with 1024 of 64.
     int G = 1;
     while (BC * G < 128 && ny % (2 * G) == 0 && ny / (2 * G) >= 4) G *= 2;
-    const int NT = (ny / G) * ((m + 3) / 4);
+    int NT = (ny / G) * ((m + 3) / 4);
     int S = kYdftThreads / NT;
     S = S < 1 ? 1 : (S > 8 ? 8 : S);
+    while (BC * G < kYdftBlocks && ny % (2 * G) == 0 && NT * S >= 128) {
+        G *= 2;
+        NT /= 2;
+    }
+    const int threads = std::min(kYdftThreads, (NT * S + 31) / 32 * 32);
     const size_t smem = sizeof(float) * ((((size_t)H * 2 * m + 3) & ~(size_t)3) + (size_t)S * NT * 8);
     if (smem <= kYdftSmemMax)
-        return launch_k(k_ydft_blk, dim3(BC, G), kYdftThreads, smem, s, pdl, A, 2 * m, H, m, (const float*)f->Fyre,
+        return launch_k(k_ydft_blk, dim3(BC, G), threads, smem, s, pdl, A, 2 * m, H, m, (const float*)f->Fyre,
                         (const float*)f->Fyim, ny, ore, oim, scale, double_kx, S);
     else
         k_ydft<<<grid1((long long)BC * ny * m), 256, 0, s>>>(A, 2 * m, H, m, f->Fyre, f->Fyim, ny, BC, ore, oim, scale,

@@ -58,6 +58,16 @@ def test_fno_forward_and_gradients_match_fp64_oracle(case):
         assert rel_l2(gd[name], gref[name]) < 5e-2, name
 
 
+# batches: samples that do not fill the mode mix's groups, y transforms split
+# over blocks of whole and of partial warps, and not split at all
+BATCH_CASES = [(40, 36, 16, 8, 2, 5), (48, 40, 32, 4, 1, 9), (64, 64, 8, 16, 1, 4), (32, 70, 16, 12, 1, 6)]
+
+
+@pytest.mark.parametrize("case", BATCH_CASES, ids=["x".join(map(str, c)) for c in BATCH_CASES])
+def test_fno_batches_match_fp64_oracle(case):
+    test_fno_forward_and_gradients_match_fp64_oracle(case)
+
+
 def test_fno_forward_at_the_surrogate_size():
     """The surrogate's network at full size (256 x 256 film, width 32, 16 x 16
     modes, 4 layers; batch 2) against the FP64 oracle forward pass, with the
