@@ -79,8 +79,11 @@ __device__ __forceinline__ void any_pass1(const RagDesc& d, int tile, int par) {
 // tiles, which also form the next step's x spectra in place: a tile reads
 // exactly the spectrum entries it writes.  The state goes M[par0] ->
 // M[par0 ^ 1] -> ...  A grid-barrier wait that runs out of polls, or a copy
-// wait that gives up, sets kFlagTimeout.
-__global__ void __launch_bounds__(kRagBatchThreads, 2)
+// wait that gives up, sets kFlagTimeout.  Bound by the latency of a tile
+// (queue, copies, barriers), so four blocks share an SM although their 64
+// registers spill: 512 samples of up to 256 x 64 x 2 cells take 1.37 ms per
+// step with two blocks, 1.05 with three and 0.95 with four.
+__global__ void __launch_bounds__(kRagBatchThreads, 4)
     k_batch_persist(const BatchDesc* __restrict__ d, const RagDesc* __restrict__ rd, BatchPass q1, BatchPass q2,
                     BatchPass q3, int ns, int par0, int nsteps, float dt, int first_x, int* __restrict__ flag,
                     GridBar* __restrict__ gb, long long limit) {

@@ -14,8 +14,8 @@
 // transforms with one exchange.  Bound by the latency of two single-wave
 // kernels on small films and by shared memory and the FP32 pipes on large
 // ones, like the power-of-two step.  Per L2-resident Euler step, general
-// kernels against these: 200x60x3 25 against 9.6 us, 600x400x1 field
-// evaluation and stage 55 against 34 us.
+// kernels against these: 200x60x3 25 against 9.6 us, an RK4 step of
+// 600x400x1 222 against 115.
 #pragma once
 #include "fast_step.cuh"
 
