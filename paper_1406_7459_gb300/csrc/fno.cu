@@ -1010,6 +1010,13 @@ static bool mix_tail(mm_fno* f, int l, int B, bool train, float* y, cudaStream_t
     }
 }
 
+// Whether the mode mix reads four modes at a time (and adds the channels as
+// eight partial sums).
+static bool mode_quads(int nmode, const float* Rr, const float* Ri, const float* vr, const float* vi) {
+    auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    return nmode % 16 == 0 && al(Rr) && al(Ri) && al(vr) && al(vi);
+}
+
 // Mode mix + inverse y (k_mode_inv) of B samples from (vr, vi) into f->zb
 // with the R of layer l (conjT: its adjoint): clusters of YS blocks per
 // (b, o), YS chosen to spread over the SMs.
@@ -1019,8 +1026,7 @@ static cudaError_t mode_inv(const mm_fno* f, int l, int B, const float* vr, cons
     const long long ro = (long long)l * C * C * nmode;
     const float* Rr = f->w + f->oRr + ro;
     const float* Ri = f->w + f->oRi + ro;
-    auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-    const bool vec4 = nmode % 16 == 0 && al(Rr) && al(Ri) && al(vr) && al(vi);
+    const bool vec4 = mode_quads(nmode, Rr, Ri, vr, vi);
     int YS = 1;
     while (B * C * YS < 152 && YS < 8 && H / (2 * YS) >= 8 && nmode % (2 * YS) == 0 &&
            (!vec4 || (nmode / (2 * YS)) % 16 == 0))
@@ -1050,8 +1056,9 @@ static cudaError_t mode_inv(const mm_fno* f, int l, int B, const float* vr, cons
 static cudaError_t mode_inv_batch(const mm_fno* f, int l, int B, const float* vr, const float* vi, int conjT,
                                   cudaStream_t s) {
     const int C = f->C, m = f->m, nmode = 2 * m * m;
-    if (B < 4 || m % 4 != 0) return mode_inv(f, l, B, vr, vi, conjT, s, true);
     const long long ro = (long long)l * C * C * nmode;
+    if (B < 4 || m % 4 != 0 || C % 2 != 0 || !mode_quads(nmode, f->w + f->oRr + ro, f->w + f->oRi + ro, vr, vi))
+        return mode_inv(f, l, B, vr, vi, conjT, s, true);
     cudaError_t e = launch_k(k_mode_mix, dim3((nmode + 31) / 32, C, (B + kMixNB - 1) / kMixNB), 128, 0, s, true, vr, vi,
                              (const float*)(f->w + f->oRr + ro), (const float*)(f->w + f->oRi + ro), C, nmode, B,
                              conjT, f->wmr, f->wmi);

@@ -456,10 +456,11 @@ __global__ void __launch_bounds__(256) k_back_reduce(BackJobs q) {
 
 // Batches: the per-mode channel mix,
 //   w[b][o][md] = sum_c R[c][o][md] vh[b][c][md]  (conjT: conj(R[o][c][md])),
-// a block per (32 modes, o, kMixNB samples), a quarter of the channels per
-// warp, the samples in registers so that one read of R serves them all (loads
-// past the batch are clamped, so that they all issue together), the quarters
-// summed through shared memory.  Bound by the latency of its loads from L2:
+// a block per (32 modes, o, kMixNB samples), the channels 2 w and 2 w + 1
+// modulo 8 to warp w (C even), the samples in registers so that one read of R
+// serves them all (loads past the batch are clamped, so that they all issue
+// together).  The eight partial sums are added in k_mode_inv's order, for the
+// same bits ahead of the BF16 rounding.  Bound by the latency of its loads from L2:
 // loss and gradients at 256 x 256, width 32, 16 modes, batch 8 take 1733 us
 // with all eight samples in one block, 1640 with four in each of two.
 constexpr int kMixNB = 4;
@@ -472,28 +473,31 @@ __global__ void __launch_bounds__(128) k_mode_mix(const float* __restrict__ vr, 
     pdl_trigger();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o = blockIdx.y, b0 = blockIdx.z * kMixNB;
     const int md = blockIdx.x * 32 + lane, mc = min(md, nmode - 1);
-    const int cq = (C + 3) / 4, c1 = min(C, (warp + 1) * cq);
     const float sgn = conjT ? -1.f : 1.f;
     const long long xs = (long long)C * nmode;            // one sample's modes
-    float sr[kMixNB], si[kMixNB];
+    float sr[2][kMixNB], si[2][kMixNB];
 #pragma unroll
-    for (int k = 0; k < kMixNB; ++k) sr[k] = si[k] = 0.f;
-#pragma unroll 4
-    for (int c = warp * cq; c < c1; ++c) {
+    for (int k = 0; k < kMixNB; ++k) sr[0][k] = sr[1][k] = si[0][k] = si[1][k] = 0.f;
+    auto add = [&](int c, float (&ar)[kMixNB], float (&ai)[kMixNB]) {
         const long long ri = (conjT ? (long long)o * C + c : (long long)c * C + o) * nmode + mc;
         const float rr = __ldg(Rre + ri), rm = sgn * __ldg(Rim + ri);
 #pragma unroll
         for (int k = 0; k < kMixNB; ++k) {
             const long long xi = min(b0 + k, B - 1) * xs + (long long)c * nmode + mc;
             const float xr = __ldg(vr + xi), xm = __ldg(vi + xi);
-            sr[k] += rr * xr - rm * xm;
-            si[k] += rr * xm + rm * xr;
+            ar[k] += rr * xr - rm * xm;
+            ai[k] += rr * xm + rm * xr;
         }
+    };
+#pragma unroll 2
+    for (int c = 2 * warp; c + 1 < C; c += 8) {
+        add(c, sr[0], si[0]);
+        add(c + 1, sr[1], si[1]);
     }
 #pragma unroll
     for (int k = 0; k < kMixNB; ++k) {
-        red[warp][2 * k][lane] = sr[k];
-        red[warp][2 * k + 1][lane] = si[k];
+        red[warp][2 * k][lane] = sr[0][k] + sr[1][k];
+        red[warp][2 * k + 1][lane] = si[0][k] + si[1][k];
     }
     __syncthreads();
     for (int e = warp; e < 2 * kMixNB; e += 4) {
