@@ -1052,7 +1052,8 @@ static cudaError_t mode_inv(const mm_fno* f, int l, int B, const float* vr, cons
 // The same for a training batch: R read once for all samples (k_mode_mix),
 // then the inverse y transform.  From four samples on: the fused kernel's
 // blocks each read R again (a training batch's gradients at batch 8, width
-// 32, 16 modes, 256 x 256: 1.83 ms with the fused kernel, 1.70 so).
+// 32, 16 modes, 256 x 256: 1.83 ms with the fused kernel, 1.58 so, the y
+// transforms' finer blocks included).
 static cudaError_t mode_inv_batch(const mm_fno* f, int l, int B, const float* vr, const float* vi, int conjT,
                                   cudaStream_t s) {
     const int C = f->C, m = f->m, nmode = 2 * m * m;
