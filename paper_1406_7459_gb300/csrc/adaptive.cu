@@ -47,6 +47,7 @@ static int dp_step_fused(mm_ctx* c, const DpPtrs& kp, const LlgCoef& cf, const f
     float* Y[2] = {c->Mst, c->H};
     auto args = [&](const double* w, int stage, float* out) {
         StageArgs st{};
+        st.kind = kStageDp;
         st.base = M;
         st.kout = kp.k[stage - 1];
         for (int j = 0; j < stage - 1; ++j)

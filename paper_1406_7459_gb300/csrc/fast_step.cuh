@@ -816,7 +816,7 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
         } else if constexpr (MODE == kModeStage) {
             float f[3], n[3];
             llg_rhs_fixed(cf, m, hh, f);
-            if (st->acc) {
+            if (st->kind == kStageRk) {
 #pragma unroll
                 for (int cc = 0; cc < 3; ++cc) {
                     const float a = fmaf(st->wf, f[cc], sc->a[u][cc]);
@@ -982,7 +982,7 @@ __device__ __forceinline__ void load_rag_cells(const Geom& g, const LlgCoef& cf,
 template <int N, int R, int T, bool RAG>
 __device__ __forceinline__ void load_stage_cells(const Geom& g, const StageArgs& st, int tile,
                                                  StageCells<(R * N + T - 1) / T>& sc) {
-    if (!st.acc) return;
+    if (st.kind != kStageRk) return;
     const int ntj = (RAG ? g.Jr : g.ny) / R;
     const int k = tile / ntj, j0 = (tile % ntj) * R;
     const int nx = RAG ? g.nx : N, Nc = g.N;

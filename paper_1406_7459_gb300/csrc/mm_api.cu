@@ -474,10 +474,12 @@ extern "C" int mm_set_integrator(mm_ctx* c, int method) {
     if (!c) return fail(MM_EINVAL, "null context");
     if (method != MM_INTEGRATOR_EULER && method != MM_INTEGRATOR_HEUN && method != MM_INTEGRATOR_RK4)
         return fail(MM_EINVAL, "unknown integrator %d", method);
-    if (method != MM_INTEGRATOR_EULER && !c->Mst) {
+    if (method != MM_INTEGRATOR_EULER) {
+        // each on its own: an adaptive run allocates Mst alone, and an earlier
+        // call may have stopped between the two
         const size_t n = 3 * (size_t)c->g.N;
-        CU(cudaMalloc(&c->Mst, sizeof(float) * n));
-        CU(cudaMalloc(&c->acc, sizeof(float) * n));
+        if (!c->Mst) CU(cudaMalloc(&c->Mst, sizeof(float) * n));
+        if (!c->acc) CU(cudaMalloc(&c->acc, sizeof(float) * n));
     }
     if (method != c->method) {
         c->method = method;
@@ -592,12 +594,14 @@ static int enqueue_rk_step(mm_ctx* c, int p, double dt, cudaStream_t s) {
     const float* av = ns == 2 ? heun_a : rk4_a;
     const float* bv = ns == 2 ? heun_b : rk4_b;
     const LlgCoef cf = make_coef(c, dt);
+    if (!c->Mst || !c->acc) return fail(MM_EINVAL, "no stage buffers");   // mm_set_integrator allocates both
     if (fused_stages(c)) {
         // S holds the x spectrum of M[p]; every stage leaves the next
         // state's, the last one M[1 - p]'s.  The stage states alternate
         // between two buffers (H is free here).
         for (int q = 0; q < ns; ++q) {
             StageArgs st{};
+            st.kind = kStageRk;
             st.base = c->Mbuf[p];
             st.acc = c->acc;
             st.wf = bv[q];

@@ -109,12 +109,14 @@ struct Launch {
 enum Pass3Mode { kModeDemag = 0, kModeHeff = 1, kModeStep = 2, kModeStepX = 3, kModeStage = 4, kModeErr = 5 };
 
 // What a stage does with its slope f = f(Y) (each pointer 3 N floats).
-//   acc set (Heun, RK4): a = wf f (+ acc unless first); the next state is
+//   kStageRk (Heun, RK4): a = wf f (+ acc unless first); the next state is
 //     base + s f, or on the last stage base + dt a renormalised to Ms.
-//   else (Dormand-Prince): f -> kout; a = wf f + sum_j w_j k_j; the next
+//   kStageDp (Dormand-Prince): f -> kout; a = wf f + sum_j w_j k_j; the next
 //     state is base + dt a, renormalised when last; kModeErr: err = max over
 //     cells of |dt a| / Ms, folded into *err.
+enum StageKind { kStageRk, kStageDp };
 struct StageArgs {
+    StageKind kind;
     const float* base;
     float* acc;
     float* kout;

@@ -1,0 +1,50 @@
+"""Sequences of calls on one context or batch, where one call leaves state that
+the next one uses: the integrators one after the other, a field changed with
+steps in flight, long persistent launches.  Tolerances are those of the step
+tests: 1e-4 of what the steps change against the FP64 oracle, bit equality
+between two forms of the same arithmetic."""
+import numpy as np
+import pytest
+
+from oracle import llg as L
+from paper_1406_7459_gb300 import inputs
+from tests._helpers import oracle_spectrum, rel_l2
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+MS, A_EX, GAMMA = 8.6e5, 1.3e-11, inputs.GAMMA0
+CELL, HEXT = (4e-9, 3e-9, 5e-9), (1e4, -5e3, 2e3)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+
+
+@pytest.mark.parametrize("method", ["heun", "rk4"])
+@pytest.mark.parametrize("grid", [(20, 12, 3), (32, 32, 2), (700, 540, 1), (1100, 6, 1)])
+def test_runge_kutta_after_an_adaptive_run(method, grid):
+    """An adaptive run allocates the stage state alone; Heun and RK4 also need
+    the sum of their slopes.  Fused stages (ragged and power-of-two), a film
+    above the fused stages' size and the general kernels."""
+    from paper_1406_7459_gb300 import mm
+    M = np.ascontiguousarray(inputs.perturbed_m(grid, MS, seed=3, amplitude=0.3), np.float32)
+    ctx = mm.mm_create(grid, CELL, MS, A_EX, 1e4, 0.2, GAMMA)
+    mm.mm_set_field(ctx, HEXT)
+    Md = torch.from_numpy(M.reshape(-1)).cuda()
+    mm.mm_set_m(ctx, Md)
+    done, _, _ = mm.mm_run_adaptive(ctx, 1e-14, 1e-14, 1.0, 4)
+    assert done
+    mid = torch.empty_like(Md)
+    mm.mm_get_m(ctx, mid)
+    mm.mm_set_integrator(ctx, method)
+    mm.mm_step(ctx, 2, 2e-14)
+    out = torch.empty_like(Md)
+    mm.mm_get_m(ctx, out)
+    mm.mm_sync(ctx)
+    Kt, Lp = oracle_spectrum(grid, CELL)
+    m64 = mid.cpu().numpy().reshape(M.shape).astype(np.float64)
+    ref = L.run_rk(m64, 2, 2e-14, method, CELL, MS, A_EX, 1e4, 0.2, GAMMA, HEXT, Kt, Lp)
+    assert rel_l2(out.cpu().numpy().reshape(M.shape) - m64, ref - m64) < 1e-4
