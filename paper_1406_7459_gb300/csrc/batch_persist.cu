@@ -11,10 +11,10 @@ template <int NY, int NZ> __device__ __noinline__ bool plane_item(const RagDesc&
     return rag_plane_tile<NY, NZ, kRagBatchThreads>(d, tile, flag);
 }
 template <int N> __device__ __noinline__ void xstep_item(const RagDesc& d, int tile, int par, float dt, int* flag) {
-    rag_xstep_tile<N, kRagBatchThreads>(d, tile, par, dt, flag);
+    rag_xstep_tile<N, kRagBatchThreads, true>(d, tile, par, dt, flag);
 }
 template <int N> __device__ __noinline__ void pass1_item(const RagDesc& d, int tile, int par) {
-    rag_pass1_tile<N, kRagBatchThreads>(d, tile, par);
+    rag_pass1_tile<N, kRagBatchThreads, true>(d, tile, par);
 }
 
 __device__ __forceinline__ bool any_plane(const RagDesc& d, int tile, int* flag) {
@@ -78,9 +78,10 @@ __device__ __forceinline__ void any_pass1(const RagDesc& d, int tile, int par) {
 // already those of that state), queue 1 the plane tiles, queue 2 the update
 // tiles, which also form the next step's x spectra in place: a tile reads
 // exactly the spectrum entries it writes.  The state goes M[par0] ->
-// M[par0 ^ 1] -> ...  A grid-barrier wait that runs out of polls, or a copy
-// wait that gives up, sets kFlagTimeout.  Bound by the latency of a tile
-// (queue, copies, barriers), so four blocks share an SM although their 64
+// M[par0 ^ 1] -> ..., so every load of M is an ordinary one (load_m).  A
+// grid-barrier wait that runs out of polls, or a copy wait that gives up,
+// sets kFlagTimeout.  Bound by the latency of a tile (queue, copies,
+// barriers), so four blocks share an SM although their 64
 // registers spill: 512 samples of up to 256 x 64 x 2 cells take 1.37 ms per
 // step with two blocks, 1.05 with three and 0.95 with four.
 __global__ void __launch_bounds__(kRagBatchThreads, 4)
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(kRagBatchThreads, 4)
             i -= q1.n_items;
             const int s = find_sample(q1.pre, ns, i);
             const BatchDesc& b = d[s];
-            pass1_body(b.g, b.r1, b.r1 / 2, par0 ? b.M1 : b.M0, b.S, i - __ldg(q1.pre + s));
+            pass1_body<true>(b.g, b.r1, b.r1 / 2, par0 ? b.M1 : b.M0, b.S, i - __ldg(q1.pre + s));
         }
         ok = grid_sync(gb, bar++, limit);
     }
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(kRagBatchThreads, 4)
             const BatchDesc& b = d[s];
             LlgCoef cf = b.cf;
             cf.dt = dt;
-            pass3_body<kModeStepX>(b.g, b.r3, 3 * b.r3 / 2, cf, b.S, par ? b.M1 : b.M0, par ? b.M0 : b.M1, flag,
+            pass3_body<kModeStepX, true>(b.g, b.r3, 3 * b.r3 / 2, cf, b.S, par ? b.M1 : b.M0, par ? b.M0 : b.M1, flag,
                                    i - __ldg(q3.pre + s), b.S);
         }
         if (st + 1 < nsteps) ok = grid_sync(gb, bar++, limit);

@@ -98,8 +98,8 @@ __global__ void __launch_bounds__(R * Fft2<N>::G) k_pass1_fast(Geom g, const flo
 // and the zero rows' spectra (up to Jr) are written like the others.
 // T: the block size (threads past the R G of the transforms only help with
 // the copies and the split).
-template <int N, int R, int T, bool RAG, bool COMB = false>
-__device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float* __restrict__ M,
+template <int N, int R, int T, bool RAG, bool COMB = false, bool OWN = false>
+__device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float* M,
                                            float2* __restrict__ S, float* __restrict__ Mcopy,
                                            const XComb& xc = XComb{}) {
     using F = Fft2<N>;
@@ -142,9 +142,9 @@ __device__ __forceinline__ void pass1_rows(const Geom& g, int tile, const float*
         for (int q = 0; q < P; ++q) {
             const int j = t + Q * q;
             if constexpr (RAG)
-                v[q] = make_float2(j < na ? __ldg(ra + j) : 0.f, j < nb ? __ldg(rb + j) : 0.f);
+                v[q] = make_float2(j < na ? load_m<OWN>(ra + j) : 0.f, j < nb ? load_m<OWN>(rb + j) : 0.f);
             else
-                v[q] = make_float2(__ldg(ra + j), __ldg(rb + j));
+                v[q] = make_float2(load_m<OWN>(ra + j), load_m<OWN>(rb + j));
         }
         if constexpr (COMB) {                              // M + dt (w K), e.g. a stage state
             const float* ka = xc.K + (ra - M);

@@ -938,9 +938,10 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
 // registers; the tile's cells past nx and ny are zeroed in Mt (the update
 // writes the others).  Run before the wait for the plane kernel, which does
 // not write M, so the 7-point loads overlap it.
-template <int N, int R, int T>
-__device__ __forceinline__ void load_rag_cells(const Geom& g, const LlgCoef& cf, int tile, const float* __restrict__ M,
-                                               float* Mt, RagCells<(R * N + T - 1) / T>& rc) {
+// OWN: the launch itself rewrites M between two of its barriers (load_m).
+template <int N, int R, int T, bool OWN = false>
+__device__ __forceinline__ void load_rag_cells(const Geom& g, const LlgCoef& cf, int tile, const float* M, float* Mt,
+                                               RagCells<(R * N + T - 1) / T>& rc) {
     const int ntj = g.Jr / R;
     const int k = tile / ntj, j0 = (tile % ntj) * R;
     const int nx = g.nx, Nc = g.N, plane_xy = nx * g.ny;
@@ -961,12 +962,13 @@ __device__ __forceinline__ void load_rag_cells(const Geom& g, const LlgCoef& cf,
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const float* Mc = M + (size_t)c * Nc;
-            const float m0 = __ldg(Mc + cell);
+            const float m0 = load_m<OWN>(Mc + cell);
             // contractions written out: the single and the batched kernel
             // round alike
-            float lap = __fmul_rn(fmaf(-2.f, m0, __ldg(Mc + xp)) + __ldg(Mc + xm), cf.idx2);
-            lap = fmaf(fmaf(-2.f, m0, __ldg(Mc + yp)) + __ldg(Mc + ym), cf.idy2, lap);
-            if (g.nz > 1) lap = fmaf(fmaf(-2.f, m0, __ldg(Mc + zp)) + __ldg(Mc + zm), cf.idz2, lap);
+            float lap = __fmul_rn(fmaf(-2.f, m0, load_m<OWN>(Mc + xp)) + load_m<OWN>(Mc + xm), cf.idx2);
+            lap = fmaf(fmaf(-2.f, m0, load_m<OWN>(Mc + yp)) + load_m<OWN>(Mc + ym), cf.idy2, lap);
+            if (g.nz > 1)
+                lap = fmaf(fmaf(-2.f, m0, load_m<OWN>(Mc + zp)) + load_m<OWN>(Mc + zm), cf.idz2, lap);
             rc.m[u][c] = m0;
             rc.ex[u][c] = __fmul_rn(cf.pexch, lap);
         }

@@ -130,6 +130,15 @@ struct StageArgs {
     unsigned* err;
 };
 
+// A cell of M.  OWN: the kernel's own blocks rewrite M between two grid barriers
+// of the launch, so the load must not go through the read-only path (whose
+// lines no barrier makes stale); else M does not change while the kernel
+// runs.
+template <bool OWN> __device__ __forceinline__ float load_m(const float* p) {
+    if constexpr (OWN) return *p;
+    else return __ldg(p);
+}
+
 // Planning helpers (mm_api.cu), shared with the batched driver.
 int plan_padded_length(int n);
 int plan_ragged_len(int n);        // carrier length of a ragged side, or 0 (ragged_select.cu)

@@ -8,8 +8,9 @@
 namespace mmk {
 
 // ---------------------------------------------------------------- pass 1 --
-__device__ __forceinline__ void pass1_body(const Geom& g, int R, int group, const float* __restrict__ M,
-                                           float2* __restrict__ S, int tile) {
+template <bool OWN = false>                                // load_m
+__device__ __forceinline__ void pass1_body(const Geom& g, int R, int group, const float* M, float2* __restrict__ S,
+                                           int tile) {
     extern __shared__ float2 sm[];
     const int lstride = padded_len(g.Lx);
     const int ntj = (g.ny + R - 1) / R;
@@ -26,7 +27,7 @@ __device__ __forceinline__ void pass1_body(const Geom& g, int R, int group, cons
         const int r = wl.q;
         const int i = wl.r;
         const int j = j0 + r;
-        const float v = (j < g.ny) ? __ldg(Mc + (size_t)j * g.nx + i) : 0.f;
+        const float v = (j < g.ny) ? load_m<OWN>(Mc + (size_t)j * g.nx + i) : 0.f;
         reinterpret_cast<float*>(sm + (r >> 1) * lstride + padi(i))[r & 1] = v;
     }
     fft_lines(sm, sm + (R / 2) * lstride, lstride, R / 2, group, g.px, g.twx, g.nx, false);
@@ -50,9 +51,9 @@ __device__ __forceinline__ void pass1_body(const Geom& g, int R, int group, cons
 }
 
 // ---------------------------------------------------------------- pass 3 --
-template <int MODE>
+template <int MODE, bool OWN = false>
 __device__ __forceinline__ void pass3_body(const Geom& g, int R, int group, const LlgCoef& cf,
-                                           const float2* S, const float* __restrict__ M,
+                                           const float2* S, const float* M,
                                            float* __restrict__ out, int* __restrict__ flag, int tile,
                                            float2* Snext = nullptr) {
     extern __shared__ float2 sm[];
@@ -122,10 +123,10 @@ __device__ __forceinline__ void pass3_body(const Geom& g, int R, int group, cons
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const float* Mc = M + c * N;
-            const float m0 = __ldg(Mc + cell);
-            const float lap = (__ldg(Mc + xp) - 2.f * m0 + __ldg(Mc + xm)) * cf.idx2 +
-                              (__ldg(Mc + yp) - 2.f * m0 + __ldg(Mc + ym)) * cf.idy2 +
-                              (__ldg(Mc + zp) - 2.f * m0 + __ldg(Mc + zm)) * cf.idz2;
+            const float m0 = load_m<OWN>(Mc + cell);
+            const float lap = (load_m<OWN>(Mc + xp) - 2.f * m0 + load_m<OWN>(Mc + xm)) * cf.idx2 +
+                              (load_m<OWN>(Mc + yp) - 2.f * m0 + load_m<OWN>(Mc + ym)) * cf.idy2 +
+                              (load_m<OWN>(Mc + zp) - 2.f * m0 + load_m<OWN>(Mc + zm)) * cf.idz2;
             m[c] = m0;
             h[c] = hd[c] + cf.pexch * lap;
         }

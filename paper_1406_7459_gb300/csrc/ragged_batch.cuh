@@ -108,7 +108,8 @@ __device__ __forceinline__ bool rag_plane_tile(const RagDesc& d, int kx, int* __
 
 // x tile `tile` of a sample: the Euler step of its rows from M[par] to
 // M[par ^ 1], and their next spectrum.
-template <int N, int T>
+// OWN (load_m): the persistent launch, whose steps swap M[0] and M[1].
+template <int N, int T, bool OWN>
 __device__ __forceinline__ void rag_xstep_tile(const RagDesc& d, int tile, int par, float dt, int* __restrict__ flag) {
     constexpr int R = rag_rows<N>();
     using Lay = XstepLayout<N, R>;
@@ -129,7 +130,7 @@ __device__ __forceinline__ void rag_xstep_tile(const RagDesc& d, int tile, int p
     __pipeline_commit();
     const float* M = d.M[par];
     RagCells<(R * N + T - 1) / T> rc;
-    load_rag_cells<N, R, T>(g, cf, tile, M, Mt, rc);
+    load_rag_cells<N, R, T, OWN>(g, cf, tile, M, Mt, rc);
     xstep_body<N, R, kModeStep, T, true>(g, cf, tile, tw, ta, Mt, sb, wk, d.S, d.S, d.M[par ^ 1], flag, nullptr,
                                          XTma{}, &rc);
     __syncthreads();
@@ -138,10 +139,10 @@ __device__ __forceinline__ void rag_xstep_tile(const RagDesc& d, int tile, int p
 // Row transform of 4 rows (tile) of M[par] into S, one row group per tile
 // as in k_pass1_rag<N, 4>.
 constexpr int kRagRows1 = 4;
-template <int N, int T>
+template <int N, int T, bool OWN>
 __device__ __forceinline__ void rag_pass1_tile(const RagDesc& d, int tile, int par) {
     const Geom g = rag_geom(d);
-    pass1_rows<N, kRagRows1, T, true>(g, tile, d.M[par], d.S, nullptr);
+    pass1_rows<N, kRagRows1, T, true, false, OWN>(g, tile, d.M[par], d.S, nullptr);
     __syncthreads();
 }
 
@@ -157,14 +158,14 @@ __global__ void __launch_bounds__(XstepLayout<N, rag_rows<N>()>::THREADS)
     k_rag_batch_xstep(const RagDesc* __restrict__ d, const RagItem* __restrict__ items, int par, float dt,
                       int* __restrict__ flag) {
     const RagItem it = items[blockIdx.x];
-    rag_xstep_tile<N, XstepLayout<N, rag_rows<N>()>::THREADS>(d[it.s], it.tile, par, dt, flag);
+    rag_xstep_tile<N, XstepLayout<N, rag_rows<N>()>::THREADS, false>(d[it.s], it.tile, par, dt, flag);
 }
 
 template <int N>
 __global__ void __launch_bounds__(kRagRows1 * Fft2<N>::G)
     k_rag_batch_pass1(const RagDesc* __restrict__ d, const RagItem* __restrict__ items, int par) {
     const RagItem it = items[blockIdx.x];
-    rag_pass1_tile<N, kRagRows1 * Fft2<N>::G>(d[it.s], it.tile, par);
+    rag_pass1_tile<N, kRagRows1 * Fft2<N>::G, false>(d[it.s], it.tile, par);
 }
 
 // Kernels of one plane class / x class (batch.cu).

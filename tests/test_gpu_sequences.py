@@ -48,3 +48,39 @@ def test_runge_kutta_after_an_adaptive_run(method, grid):
     m64 = mid.cpu().numpy().reshape(M.shape).astype(np.float64)
     ref = L.run_rk(m64, 2, 2e-14, method, CELL, MS, A_EX, 1e4, 0.2, GAMMA, HEXT, Kt, Lp)
     assert rel_l2(out.cpu().numpy().reshape(M.shape) - m64, ref - m64) < 1e-4
+
+
+def _batch(grids, stream=None):
+    from paper_1406_7459_gb300 import mm
+    n = len(grids)
+    b = mm.mm_batch_create(grids, [CELL] * n, [MS] * n, [A_EX] * n, [1e4] * n, [0.2] * n, [GAMMA] * n, stream=stream)
+    mm.mm_batch_set_field(b, [HEXT] * n)
+    M = np.concatenate([inputs.random_unit_m(g, MS, 20 + i).reshape(-1) for i, g in enumerate(grids)])
+    mm.mm_batch_set_m(b, torch.from_numpy(M).cuda())
+    return b
+
+
+def _batch_state(b):
+    from paper_1406_7459_gb300 import mm
+    out = torch.empty(b.total, device="cuda")
+    mm.mm_batch_get_m(b, out)
+    mm.mm_batch_sync(b)
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("grids", [[(33, 17, 2), (16, 48, 1), (100, 30, 2), (200, 64, 1), (64, 64, 4)],
+                                   [(257, 12, 1), (20, 65, 3)], [(40, 40, 1), (12, 257, 1)]],
+                         ids=["classes", "general", "mixed"])
+def test_long_persistent_launch_is_bitwise_the_batched_kernels(grids):
+    """One launch of 48 steps rewrites each state buffer 24 times between its
+    barriers; the batched kernels read a buffer that no running kernel
+    writes."""
+    from paper_1406_7459_gb300 import mm
+    got = []
+    for path in (mm.MM_STEP_GRAPH, mm.MM_STEP_PERSISTENT):
+        b = _batch(grids)
+        mm.mm_batch_set_path(b, path)
+        mm.mm_batch_step(b, 48, 5e-14)
+        got.append(_batch_state(b))
+    assert np.all(np.isfinite(got[0]))
+    assert np.array_equal(got[0], got[1])
