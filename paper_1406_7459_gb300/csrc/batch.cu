@@ -222,9 +222,12 @@ static int batch_layout(mm_batch* b) {
         BCU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_persist_fn(), kRagBatchThreads, ps));
         b->pgrid = per_sm * sms;
     }
-    BCU(cudaMemcpy(b->d_rag, b->rag.data(), sizeof(RagDesc) * b->ns, cudaMemcpyHostToDevice));
-    BCU(cudaMemcpy(b->d_desc, b->desc.data(), sizeof(BatchDesc) * b->ns, cudaMemcpyHostToDevice));
-    BCU(cudaMemcpy(b->d_pre, pre.data(), sizeof(int) * pre.size(), cudaMemcpyHostToDevice));
+    // on the batch's stream, behind the steps in flight that read the old
+    // tables (the legacy stream waits for no non-blocking one)
+    BCU(cudaMemcpyAsync(b->d_rag, b->rag.data(), sizeof(RagDesc) * b->ns, cudaMemcpyHostToDevice, b->stream));
+    BCU(cudaMemcpyAsync(b->d_desc, b->desc.data(), sizeof(BatchDesc) * b->ns, cudaMemcpyHostToDevice, b->stream));
+    BCU(cudaMemcpyAsync(b->d_pre, pre.data(), sizeof(int) * pre.size(), cudaMemcpyHostToDevice, b->stream));
+    BCU(cudaStreamSynchronize(b->stream));      // before the host tables change or go
     b->ver++;
     return MM_OK;
 }
@@ -368,7 +371,8 @@ static int batch_items(mm_batch* b) {
             b->rag_smem = std::max(b->rag_smem, f.smem);
         }
     BCU(cudaMalloc(&b->d_items, sizeof(RagItem) * (items.empty() ? 1 : items.size())));
-    BCU(cudaMemcpy(b->d_items, items.data(), sizeof(RagItem) * items.size(), cudaMemcpyHostToDevice));
+    BCU(cudaMemcpyAsync(b->d_items, items.data(), sizeof(RagItem) * items.size(), cudaMemcpyHostToDevice, b->stream));
+    BCU(cudaStreamSynchronize(b->stream));
     return MM_OK;
 }
 

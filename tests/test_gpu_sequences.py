@@ -56,7 +56,9 @@ def _batch(grids, stream=None):
     b = mm.mm_batch_create(grids, [CELL] * n, [MS] * n, [A_EX] * n, [1e4] * n, [0.2] * n, [GAMMA] * n, stream=stream)
     mm.mm_batch_set_field(b, [HEXT] * n)
     M = np.concatenate([inputs.random_unit_m(g, MS, 20 + i).reshape(-1) for i, g in enumerate(grids)])
-    mm.mm_batch_set_m(b, torch.from_numpy(M).cuda())
+    Md = torch.from_numpy(M).cuda()
+    torch.cuda.synchronize()
+    mm.mm_batch_set_m(b, Md)
     return b
 
 
@@ -81,6 +83,31 @@ def test_long_persistent_launch_is_bitwise_the_batched_kernels(grids):
         b = _batch(grids)
         mm.mm_batch_set_path(b, path)
         mm.mm_batch_step(b, 48, 5e-14)
+        got.append(_batch_state(b))
+    assert np.all(np.isfinite(got[0]))
+    assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("path", ["graph", "persistent"])
+@pytest.mark.parametrize("general", [False, True])
+def test_batch_field_change_behind_steps_in_flight(path, general):
+    """mm_batch_step returns with its kernels in flight; on a stream that the
+    legacy stream does not wait for, a field set right after it must reach
+    the later steps only."""
+    from paper_1406_7459_gb300 import mm
+    grids = [(400, 40, 2)] * 24 if general else [(256, 64, 2)] * 60
+    got = []
+    for wait in (True, False):
+        side = torch.cuda.Stream()
+        b = _batch(grids, side)
+        if path == "persistent":
+            mm.mm_batch_set_path(b, mm.MM_STEP_PERSISTENT)
+        for n, k in ((60, -1.0), (20, 0.5)):
+            mm.mm_batch_step(b, n, 5e-14)
+            if wait:
+                side.synchronize()
+            mm.mm_batch_set_field(b, [tuple(k * h for h in HEXT)] * len(grids))
+        mm.mm_batch_step(b, 3, 5e-14)
         got.append(_batch_state(b))
     assert np.all(np.isfinite(got[0]))
     assert np.array_equal(got[0], got[1])
