@@ -542,17 +542,26 @@ int mmk::fused_stage(mm_ctx* c, int mode, const float* Y, const StageArgs& st, c
     return MM_OK;
 }
 
+// Whether a field evaluation of a context with the two-kernel step takes the
+// step's plane kernel and the field-only variant of its x-step kernel.  On
+// power-of-two films these read the spectrum with the exchange stencil folded
+// in.  Where a plane takes 768 threads (256 and 512 rows, many layers) or the
+// large-plane kernel in their place, the three passes serve the field, with
+// the stencil of Eq. (4) on M itself: k_plane_pdl is starved of registers
+// there, and the exchange field keeps the rounding of neighbouring differences (on
+// 256x512x4, 10 % perturbation, rms 4e-8 Ms against 5e-7 folded).  Planes that
+// the three passes would have to split have the folded spectrum either way.
+static bool two_kernel_field(const mm_ctx* c) {
+    return c->has_fs && (c->rag || c->l.split || (!c->fs.big && c->fs.ta <= 512));
+}
+
 // The three-pass evaluation on the spectrum workspace S (which also holds
 // the two-kernel step's spectrum, so it invalidates a pending one).
 int mmk::run_passes(mm_ctx* c, int mode, const float* M, float* out, double dt, cudaStream_t s) {
     const LlgCoef cf = make_coef(c, dt);
     c->spec_valid = false;
     CU(form_spectrum(c, M, s));
-    if (c->has_fs && (c->rag || c->fs.ta <= 512) && (mode == kModeDemag || mode == kModeHeff)) {
-        // power-of-two films: the step's plane kernel and the field-only
-        // variant of its x-step kernel (where the plane kernel runs at most
-        // 512 threads: larger ones are register-starved, and the three-pass
-        // plane kernel serves them better)
+    if (two_kernel_field(c) && (mode == kModeDemag || mode == kModeHeff)) {
         CU(launch_field_pdl(c->gf, c->fs, cf, mode, mode == kModeDemag ? c->gf.Kd0 : c->gf.Kd, c->S, c->Sh, M, out,
                             c->flag, s));
         return MM_OK;
