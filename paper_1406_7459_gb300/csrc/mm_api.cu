@@ -394,7 +394,9 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
             int sms = 0;
             CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
             c->fs.early = c->rag ? ragged_early_trigger(gf, c->fs, sms) : fast_step_early_trigger(gf, c->fs, sms);
-            if (!c->rag && !c->fs.big) encode_xstep_maps(g, &c->fs, c->Sh, c->S);   // per-thread copies where no map applies
+            // per-thread copies where no map applies (the maps concern the x
+            // kernel alone; wide spectrum rows of split planes have none)
+            if (!c->rag && !c->l.split) encode_xstep_maps(g, &c->fs, c->Sh, c->S);
         }
         if (c->has_persist) {
             bool usable = false;
