@@ -596,7 +596,8 @@ template <int T> __device__ __forceinline__ void block_err_max(float e, unsigned
 }
 
 // A thread's cells of a ragged x-step tile (its trips of the field loop):
-// M and the exchange field of Eq. (4), formed before the spectrum arrives.
+// M and the Laplacian of Eq. (4), formed before the spectrum arrives (the
+// exchange field is added to H_d in one rounding).
 template <int CPT> struct RagCells {
     float m[CPT][3], ex[CPT][3];
 };
@@ -774,7 +775,7 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc) {
                 m[cc] = rc->m[u][cc];
-                hh[cc] = hd[cc] + rc->ex[u][cc];
+                hh[cc] = fmaf(cf.pexch, rc->ex[u][cc], hd[cc]);
             }
         } else {
             const float bnd = bz + cf.pexch * ((float)((i == 0) + (i == N - 1)) * cf.idx2 +
@@ -970,7 +971,7 @@ __device__ __forceinline__ void load_rag_cells(const Geom& g, const LlgCoef& cf,
             if (g.nz > 1)
                 lap = fmaf(fmaf(-2.f, m0, load_m<OWN>(Mc + zp)) + load_m<OWN>(Mc + zm), cf.idz2, lap);
             rc.m[u][c] = m0;
-            rc.ex[u][c] = __fmul_rn(cf.pexch, lap);
+            rc.ex[u][c] = lap;
         }
     }
 }

@@ -41,3 +41,35 @@ def test_exchange_is_the_stencil_of_neighbouring_differences(grid):
     bound = 2.0 ** -24 * (np.abs(he).max() + 10 * np.abs(ex).max() + 6 * w * np.abs(M[1:]).max())
     print("largest error %.2e Ms, bound %.2e Ms" % (np.abs(he - hd - ex).max() / MS, bound / MS))
     assert np.abs(he - hd - ex).max() <= bound
+
+
+@pytest.mark.parametrize("grid", [(40, 36, 3), (129, 385, 4), (33, 50, 1), (20, 18, 11)])
+def test_ragged_exchange_is_added_in_one_rounding(grid):
+    """H_eff = fl(H_d + pexch lap), lap by FP32 multiply-adds.  The multiply-adds
+    are evaluated here in FP64 and rounded once more, which is the same but for
+    ties of the second rounding (one in 2^29 and fewer); a separately
+    rounded product would differ in a quarter of the cells."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1406_7459_gb300 import mm
+    M = inputs.random_unit_m(grid, MS, seed=2)
+    ctx = mm.mm_create(grid, CELL, MS, A_EX, 0.0, 0.1, GAMMA)
+    Md = torch.from_numpy(M.reshape(-1)).cuda()
+    hd, he = torch.empty_like(Md), torch.empty_like(Md)
+    mm.mm_demag_field(ctx, Md, hd)
+    mm.mm_effective_field(ctx, Md, he)
+    mm.mm_sync(ctx)
+    hd, he = (t.cpu().numpy().reshape(M.shape) for t in (hd, he))
+
+    def fma(a, b, c):
+        return (a.astype(np.float64) * np.float64(b) + c).astype(np.float32)
+
+    w, d2 = np.float32(2 * A_EX / (4e-7 * np.pi * MS * MS)), np.float32(1 / CELL[0] ** 2)
+    P = np.pad(M, ((0, 0), (1, 1), (1, 1), (1, 1)), mode="edge")
+    lap = np.float32(0)
+    for axis in (3, 2, 1) if grid[2] > 1 else (3, 2):
+        lo, hi = [slice(1, -1)] * 3, [slice(1, -1)] * 3
+        lo[axis - 1], hi[axis - 1] = slice(0, -2), slice(2, None)
+        second = fma(M, -2.0, P[(slice(None), *hi)]) + P[(slice(None), *lo)]
+        lap = fma(second, d2, lap)
+    assert np.mean(fma(lap, w, hd) != he) < 1e-3
