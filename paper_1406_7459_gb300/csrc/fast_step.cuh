@@ -576,6 +576,13 @@ __device__ __forceinline__ void llg_rhs_fixed(const LlgCoef& cf, const float (&m
     f[2] = fmaf(cf.c1, p2, __fmul_rn(cf.c2, q2));
 }
 
+// |n|^2 with the squares added from z to x: the easy axis is x, so the largest
+// square usually enters last, unrounded, and the sum rounds once at its size
+// (renormalising a state within 10 % of x: rms 4.2e-8 so, 4.6e-8 from x to z).
+__device__ __forceinline__ float norm2_fixed(float n0, float n1, float n2) {
+    return fmaf(n0, n0, fmaf(n1, n1, __fmul_rn(n2, n2)));
+}
+
 // a += sum_j w_j k_j of one cell.
 __device__ __forceinline__ void add_slopes(const StageArgs& st, size_t cell, size_t n, float (&a)[3]) {
 #pragma unroll
@@ -835,8 +842,7 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
 #pragma unroll
                 for (int cc = 0; cc < 3; ++cc) n[cc] = fmaf(cf.dt, a[cc], __ldg(st->base + cc * Nc + cell));
             }
-            const float s =
-                st->last ? cf.Ms / sqrtf(fmaf(n[2], n[2], fmaf(n[1], n[1], __fmul_rn(n[0], n[0])))) : 1.f;
+            const float s = st->last ? cf.Ms / sqrtf(norm2_fixed(n[0], n[1], n[2])) : 1.f;
             o0 = __fmul_rn(n[0], s);
             o1 = __fmul_rn(n[1], s);
             o2 = __fmul_rn(n[2], s);
@@ -845,7 +851,7 @@ __device__ __forceinline__ void xstep_body(const Geom& g, const LlgCoef& cf, int
             float f[3];
             llg_rhs_fixed(cf, m, hh, f);
             const float n0 = fmaf(cf.dt, f[0], m[0]), n1 = fmaf(cf.dt, f[1], m[1]), n2 = fmaf(cf.dt, f[2], m[2]);
-            const float s = cf.Ms / sqrtf(fmaf(n2, n2, fmaf(n1, n1, __fmul_rn(n0, n0))));
+            const float s = cf.Ms / sqrtf(norm2_fixed(n0, n1, n2));
             o0 = __fmul_rn(n0, s);
             o1 = __fmul_rn(n1, s);
             o2 = __fmul_rn(n2, s);
