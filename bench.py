@@ -655,7 +655,8 @@ def run_batch(args, rank, ws):
     path_ms, forms = {}, {}
     for name, path in (("graph", mm.MM_STEP_GRAPH), ("persistent", mm.MM_STEP_PERSISTENT)):
         mm.mm_batch_set_path(b, path)
-        mm.mm_batch_step(b, max(args.warmup, 3), dt)
+        # past the steps that launch directly and the capture of both parities
+        mm.mm_batch_step(b, max(args.warmup, 12), dt)
         barrier(ws)
         torch.cuda.synchronize()
         e0.record()
@@ -666,7 +667,8 @@ def run_batch(args, rank, ws):
         mm.mm_batch_sync(b)
         path_ms[name] = max_over_ranks(e0.elapsed_time(e1) / K, ws)
         forms[name] = {0: "batched kernels replayed from a CUDA graph", 1: "one cooperative launch replayed from a CUDA graph",
-                       2: "one cooperative launch issued directly"}.get(mm.mm_batch_launch_form(b), "?")
+                       2: "one cooperative launch issued directly",
+                       3: "batched kernels launched directly"}.get(mm.mm_batch_launch_form(b), "?")
     batch_ms = path_ms["graph"]
     by = batch_bytes([s["grid"] for s in samples])
     by = {k: sum_over_ranks(float(v), ws) for k, v in by.items()}

@@ -211,6 +211,15 @@ int mm_effective_field(mm_ctx *ctx, const float *M_dev, float *H_dev);
 int mm_step(mm_ctx *ctx, int n, double dt);
 
 /*
+ * mm_step_form -- how the steps of the last mm_step or mm_step_host call ran:
+ * the sum of MM_FORM_DIRECT (kernels launched one by one), MM_FORM_GRAPH
+ * (replayed from a CUDA graph) and MM_FORM_PERSISTENT (one cooperative
+ * launch) for the forms it used; -1 for NULL or before any step.
+ */
+enum { MM_FORM_DIRECT = 1, MM_FORM_GRAPH = 2, MM_FORM_PERSISTENT = 4 };
+int mm_step_form(const mm_ctx *ctx);
+
+/*
  * mm_step_host -- n steps (n >= 0, dt > 0) from a state held in host
  * memory, with the result written back to host memory: the same result as
  * mm_set_m(M_in), mm_step(n, dt), mm_get_m(M_out), bit for bit, with one
@@ -369,10 +378,12 @@ int mm_batch_set_path(mm_batch *b, int path);
  * up (default 2^20; 0: at once, to exercise the timeout path).  polls >= 0. */
 int mm_batch_set_wait_limit(mm_batch *b, long long polls);
 long long mm_batch_cells(const mm_batch *b);              /* total cells, or -1 */
-/* How the last mm_batch_step ran: 0 the graph step, 1 the persistent launch
- * replayed from a CUDA graph (captured once per set of launch arguments), 2
- * the persistent launch issued directly (the runtime refused its capture);
- * -1 for NULL or before any step. */
+/* How the last step of the last mm_batch_step ran: 0 the batched kernels
+ * replayed from a CUDA graph, 1 the persistent launch replayed from a CUDA
+ * graph (captured once per set of launch arguments), 2 the persistent launch
+ * issued directly (the runtime refused its capture), 3 the batched kernels
+ * launched directly (the first steps of a dt); -1 for NULL or before any
+ * step. */
 int mm_batch_launch_form(const mm_batch *b);
 /*
  * mm_batch_autotune -- time the candidate tile shapes on this batch with

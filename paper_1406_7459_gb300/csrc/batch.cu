@@ -698,7 +698,7 @@ extern "C" int mm_batch_step(mm_batch* b, int n, double dt) {
             int rc = batch_enqueue(b, p, dt, b->stream);
             if (rc != MM_OK) return rc;
             ++b->warm;
-            b->form = 0;
+            b->form = 3;
             b->par = 1 - p;
             continue;
         }

@@ -58,6 +58,7 @@ struct mm_ctx {
     double warm_dt = 0;
     unsigned long long warm_ver = 0;
     bool use_graphs = true;
+    int form = -1;                // mm_step_form of the last run of steps
     FastFns fast;              // compile-time kernels (when the grid has them)
     FastStepFns fs;            // two-kernel step (power-of-two grids)
     FastSplitFns fsplit;       // compile-time split pass 2 (thick power-of-two samples)

@@ -762,7 +762,9 @@ extern "C" int mm_step(mm_ctx* c, int n, double dt) {
     if (n == 0) return MM_OK;
     int rc = ensure_spectrum(c);
     if (rc != MM_OK) return rc;
+    c->form = 0;
     if (uses_persist(c)) {
+        c->form = MM_FORM_PERSISTENT;
         // n steps per launch (in chunks, so that one launch stays short)
         const LlgCoef cf = make_coef(c, dt);
         for (int s = 0; s < n;) {
@@ -796,11 +798,13 @@ extern "C" int mm_step(mm_ctx* c, int n, double dt) {
                 if (rc != MM_OK) return rc;
             }
             CU(cudaGraphLaunch(c->step_exec[kind][p], c->stream));
+            c->form |= MM_FORM_GRAPH;
             if (!kind) c->cur = 1 - p;
             s += kind ? kGraphSteps : 1;
         } else {
             rc = enqueue_step(c, p, dt, c->stream);
             if (rc != MM_OK) return rc;
+            c->form |= MM_FORM_DIRECT;
             c->cur = 1 - p;
             ++s;
             if (c->warm < kWarmSteps) ++c->warm;
@@ -808,6 +812,8 @@ extern "C" int mm_step(mm_ctx* c, int n, double dt) {
     }
     return MM_OK;
 }
+
+extern "C" int mm_step_form(const mm_ctx* c) { return c ? c->form : -1; }
 
 // A host buffer's address as kernels may use it: page-locked memory mapped
 // into the device's address space, or, where the device reaches pageable
@@ -872,6 +878,7 @@ extern "C" int mm_step_host(mm_ctx* c, const float* M_in, int n, double dt, floa
     float* cp = in == c->Mbuf[c->cur] ? nullptr : c->Mbuf[c->cur];
     CU(form_spectrum(c, in, c->stream, cp));
     const LlgCoef cf = make_coef(c, dt);
+    c->form = MM_FORM_DIRECT;
     int p = c->cur;
     for (int s = 0; s < n; ++s) {
         const float* Mn = c->Mbuf[p];

@@ -26,6 +26,9 @@ MM_ELIMIT = -7
 MM_STEP_AUTO = 0
 MM_STEP_GRAPH = 1
 MM_STEP_PERSISTENT = 2
+MM_FORM_DIRECT = 1
+MM_FORM_GRAPH = 2
+MM_FORM_PERSISTENT = 4
 MM_TILED_GATHER = 1
 MM_TILED_SCATTER = 2
 
@@ -46,6 +49,7 @@ _PROTOS = {
     "mm_demag_field": (_c_int, [_vp, _vp, _vp]),
     "mm_effective_field": (_c_int, [_vp, _vp, _vp]),
     "mm_step": (_c_int, [_vp, _c_int, _c_double]),
+    "mm_step_form": (_c_int, [_vp]),
     "mm_step_host": (_c_int, [_vp, _vp, _c_int, _c_double, _vp]),
     "mm_set_step_path": (_c_int, [_vp, _c_int]),
     "mm_get_step_path": (_c_int, [_vp]),
@@ -212,6 +216,12 @@ def mm_effective_field(ctx, M, H):
 
 def mm_step(ctx, n, dt):
     _check(lib().mm_step(ctx.handle, int(n), float(dt)))
+
+
+def mm_step_form(ctx):
+    """Forms in which the last run of steps was launched: the sum of
+    MM_FORM_DIRECT, MM_FORM_GRAPH and MM_FORM_PERSISTENT; -1 before any step."""
+    return int(lib().mm_step_form(ctx.handle))
 
 
 def mm_step_host(ctx, M_in, n, dt, M_out):
@@ -381,8 +391,9 @@ def mm_batch_cells(b):
 
 
 def mm_batch_launch_form(b):
-    """0: graph step; 1: persistent launch replayed from a graph; 2: persistent
-    launch issued directly; -1 before any step."""
+    """0: batched kernels replayed from a graph; 1: persistent launch replayed
+    from a graph; 2: persistent launch issued directly; 3: batched kernels
+    launched directly; -1 before any step."""
     return int(lib().mm_batch_launch_form(b.handle))
 
 
