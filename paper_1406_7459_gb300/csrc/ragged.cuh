@@ -6,7 +6,15 @@
 // length >= 2n - 1 gives the exact linear convolution (Sec. 2), so the rows
 // and lines are zero past the sample and the outputs past it are dropped.
 // Lengths between the powers of two (3 and 5 times a power of two) keep the
-// waste of a carried side below a half, and below a third above 256.
+// waste of a carried side of more than 8 cells below a half, and below a third
+// above 256.  Shorter sides, single rows and columns among them, are carried in 16
+// all the same: what they waste is less than the general kernels' barriers
+// cost (per L2-resident Euler step, general kernels against these: 600x1x1
+// 18.5 against 13.1 us, 1x200x2 15.9 against 6.0, 5x5x5 14.9 against 4.9,
+// 1x1x100 16.6 against 14.6, 2x2x1 7.6 against 4.0).  The nearest are single
+// columns of one layer, whose general kernels transform nothing along x: 1x32x1 4.1
+// against 4.4, 1x64x1 4.4 against 4.5, 1x128x1 4.9 against 4.7, and an RK4
+// step of them 25 against 17.
 //
 // The general mixed-radix kernels transform the whole padded line in three
 // or four shared-memory stages with a block barrier, an index computation
