@@ -145,10 +145,11 @@ __device__ __forceinline__ void tc_epilogue(const GemmArgs& a, float* C, uint32_
 // whole 128-byte lines; where C's rows are not 16-byte aligned, one column of
 // each row in turn (128 contiguous bytes).
 constexpr int kTcBufRow = 36;
-template <int BN>
+template <int BN, bool VEC>
 __device__ __forceinline__ void tc_epilogue_rows(const GemmArgs& a, float* C, uint32_t tmem, int m0, int n0,
                                                  int warp, int lane, float* buf) {
-    const bool c_vec = a.scm % 4 == 0 && a.zC % 4 == 0 && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0;
+    const bool c_vec =
+        VEC || (a.scm % 4 == 0 && a.zC % 4 == 0 && (reinterpret_cast<uintptr_t>(a.C) & 15) == 0);
 #pragma unroll 1
     for (int c0 = 0; c0 < BN; c0 += 32) {
         uint32_t v[32];
@@ -370,10 +371,10 @@ __device__ __forceinline__ void tc_cp16(uint32_t dst, const void* src, bool in) 
 // bytes would fill chunks 128 bytes apart, all in the same four banks
 // (65536 x 32 x 256, bound by the load latency of its two waves of CTAs: 18.9
 // us so, 18.75 with the order here).
-template <int ROWS>
+template <int ROWS, bool VEC>
 __device__ __forceinline__ void tc_load_rows(uint32_t dst, const __nv_bfloat16* __restrict__ P, int r0, int rows,
                                              int K, int KC, long long rs, bool vec) {
-    if (vec) {
+    if (VEC || vec) {
         for (int e = threadIdx.x; e < ROWS * KC; e += kTcThreads) {
             const int q = e >> 3, g = q / KC, r = 8 * g + (e & 7), c = q - g * KC;
             const bool in = r0 + r < rows && 8 * c < K;
@@ -395,7 +396,7 @@ __device__ __forceinline__ void tc_load_rows(uint32_t dst, const __nv_bfloat16* 
     }
 }
 
-template <int BN>
+template <int BN, bool VEC>
 __global__ void __launch_bounds__(kTcThreads) k_gemm_tc_kfull(GemmArgs a) {
     static_assert(BN % 16 == 0 && BN >= 32 && BN <= 256 && (BN & (BN - 1)) == 0, "MMA N and TMEM columns");
     extern __shared__ __align__(1024) unsigned char tc_smem[];
@@ -422,8 +423,8 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc_kfull(GemmArgs a) {
     auto vec = [&](const void* p, long long rs, long long z) {
         return a.K % 8 == 0 && rs % 8 == 0 && z % 8 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
     };
-    tc_load_rows<kTcM>(As_s, A, m0, a.M, a.K, KC, a.sam, vec(a.A, a.sam, a.zA));
-    tc_load_rows<BN>(Bs_s, B, n0, a.N, a.K, KC, a.sbn, vec(a.B, a.sbn, a.zB));
+    tc_load_rows<kTcM, VEC>(As_s, A, m0, a.M, a.K, KC, a.sam, vec(a.A, a.sam, a.zA));
+    tc_load_rows<BN, VEC>(Bs_s, B, n0, a.N, a.K, KC, a.sbn, vec(a.B, a.sbn, a.zB));
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (warp == 0) {
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&tmem_base);
@@ -463,10 +464,10 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc_kfull(GemmArgs a) {
     if (!ok) {
         if (threadIdx.x == 0) atomicOr(a.err, 1);
         tc_wait(mbar_s, 0);                               // the MMAs in flight, bounded again
-    } else if (!a.atomic && a.scn == 1) {
+    } else if (VEC || (!a.atomic && a.scn == 1)) {
         // row-major C: the operand tiles are free now; each warp passes its
         // rows through 32 x 36 floats of them
-        tc_epilogue_rows<BN>(a, C, tmem, m0, n0, warp, lane,
+        tc_epilogue_rows<BN, VEC>(a, C, tmem, m0, n0, warp, lane,
                              reinterpret_cast<float*>(tc_smem) + warp * 32 * kTcBufRow);
     } else {
         tc_epilogue<BN>(a, C, tmem, m0, n0, warp, lane, true);
