@@ -193,6 +193,11 @@ __global__ void k_ydft(const float* __restrict__ A, int ldA, int H, int m, const
 // NT S takes the quad q = w % NT (iy = iy0 + q / mq, kx = 4 (q % mq) .. + 3)
 // over the y share w / NT, and the S shares of each output are summed in
 // order through shared memory.
+// It triggers its successor when the sums are formed: triggered at its start,
+// the clusters of k_mode_inv take their places while the other blocks of this
+// kernel still wait for theirs, and pile up on a few SMs (one forward pass of
+// 128 x 128, width 32, 16 modes, batch 2: 141 us triggered at the start, 130
+// so; 256 x 256, batch 2, 211 and 195).
 __global__ void __launch_bounds__(kYdftThreads)
     k_ydft_blk(const float* __restrict__ A, int ldA, int H, int m, const float* __restrict__ Fre,
                const float* __restrict__ Fim, int ny_out, float* __restrict__ ore, float* __restrict__ oim,
@@ -204,7 +209,6 @@ __global__ void __launch_bounds__(kYdftThreads)
     float* part = ys + (((size_t)H * m2 + 3) & ~(size_t)3);   // [share][quad][4 re, 4 im]
     const float* a = A + (size_t)bc * H * ldA;
     pdl_wait();
-    pdl_trigger();
     if (ldA == m2 && ((H * m2) & 3) == 0 && (reinterpret_cast<uintptr_t>(a) & 15) == 0) {
         for (int i = threadIdx.x; i < H * m2 / 4; i += blockDim.x)
             __pipeline_memcpy_async(sa + 4 * i, a + 4 * i, 16);
@@ -282,6 +286,7 @@ __global__ void __launch_bounds__(kYdftThreads)
             p[4 + j] = si[j];
         }
     }
+    pdl_trigger();
     __syncthreads();
     for (int o = threadIdx.x; o < nyb * m; o += blockDim.x) {
         const int il = o / m, kx = o - il * m;
