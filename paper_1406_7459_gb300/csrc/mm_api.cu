@@ -65,6 +65,37 @@ static bool make_axis_plan(int L, AxisPlan* p) {
     return n == 1 && p->nst <= kMaxStages;
 }
 
+// Whether a sample with a ragged nx steps faster on the general x passes than
+// in the carrier length NX.  Only where ny and nz are powers of two, so that
+// the y and z passes are compile-time ones on either route; a carried x then
+// pays in its planes (NX + 1 of them) and gains in its rows alone.  It loses where
+// the sample is large enough to be bound by throughput and
+//   - NX exceeds half the padded length by a quarter or more (a side just above
+//     a carrier): 387x128x8 55.5 us per Euler step on the general passes, 66.8
+//     carried; 773x64x16 110 and 135; 147x512x8 73 and 83; 193x256x16 94 and 101;
+//   - NX is 768 or above, whose update kernel spills: 643x128x8 102 and 127,
+//     768x512x2 100 and 112;
+//   - the planes are 128 rows of eight layers (768 threads): 275x128x8 47 and 52.
+// Of 1560 such samples from 64k carried cells on, 109 were more than 2 % slower
+// carried and up to 33 %; with these lines 26 are, by up to 9 % (32 rows of
+// eight layers, 128 layers), and 3 of the others lose 3 to 5 %.
+static bool general_x_faster(const Geom& g, const Launch& l) {
+    if (!l.fp && !l.fs2) return false;
+    const int NX = plan_ragged_len(g.nx);
+    const long long cells = (long long)NX * g.ny * g.nz, k512 = 512 * 1024;
+    const bool thick = g.nz >= 16, rows128 = g.nz == 8 && g.ny == 128;
+    const bool quarter = 8LL * NX >= 5LL * g.Lx, eighth = 40LL * NX >= 23LL * g.Lx;   // 2 NX / Lx >= 1.25, 1.15
+    if (NX == 768) return (thick && 4 * cells >= 3 * k512) || (g.nz == 8 && g.ny >= 128) || (g.nz >= 2 && g.ny >= 512);
+    if (NX == 320) return rows128;
+    if (NX == 1024 && quarter) return cells >= k512 && !(g.ny == 1024 && g.nz == 1);
+    if (NX == 512 && quarter) return cells >= k512 && (g.nz >= 8 || (g.nz >= 2 && cells >= 2 * k512));
+    if (NX >= 512 && eighth) return (thick && cells >= 2 * k512) || rows128;
+    if (NX >= 128 && NX <= 256 && quarter)
+        return (thick && cells >= k512) || (g.nz == 8 && g.ny >= 512) || (NX == 128 && g.nz == 4 && g.ny == 1024) ||
+               (NX == 192 && rows128);
+    return false;
+}
+
 // Ragged films: the two-kernel step on carrier lengths (ragged.cuh), its
 // geometry in c->gf.  False, with c unchanged but for c->fs and c->gf, where
 // no kernels exist for the size.
@@ -221,11 +252,12 @@ static int build_plan(mm_ctx* c) {
     c->gf = g;
     // without the compile-time power-of-two kernels (MM_NO_FAST=1) a context
     // takes the kernels that a batch takes for the same sample
-    c->rag = !c->has_fs && !c->has_ss && (allow_fast || ragged_batchable(g.nx, g.ny, g.nz)) && plan_ragged(c);
+    const bool carry = !c->has_fs && !c->has_ss && !general_x_faster(g, l);
+    c->rag = carry && (allow_fast || ragged_batchable(g.nx, g.ny, g.nz)) && plan_ragged(c);
     if (c->rag) {
         c->has_fs = true;
         c->has_persist = false;
-    } else if (allow_fast && !c->has_fs && !c->has_ss) {
+    } else if (allow_fast && carry) {
         c->gf = g;
         c->rag = c->has_ss = plan_ragged_split(c);
     }
