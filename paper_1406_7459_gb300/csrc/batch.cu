@@ -161,17 +161,6 @@ static LlgCoef batch_coef(const mm_batch* b, int s) {
     return f;
 }
 
-// Let a kernel have all the dynamic shared memory its static part leaves.
-// The attribute belongs to the kernel, not to a batch: every batch of the
-// process sets the same value, so that none takes it away from another.
-template <typename F> static cudaError_t allow_smem(F* k) {
-    cudaFuncAttributes at;
-    cudaError_t e = cudaFuncGetAttributes(&at, k);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(227 * 1024 - at.sharedSizeBytes));
-}
-
 // Tile counts, prefix tables, shared-memory sizes and descriptors for the
 // current shape choice (r1, r3, threads); uploads them.
 static int batch_layout(mm_batch* b) {

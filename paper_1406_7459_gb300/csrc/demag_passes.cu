@@ -54,22 +54,19 @@ cudaError_t configure_pass_kernels(const Geom& g, const Launch& l) {
             e = cudaFuncSetAttribute(l.fx->p3[m], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.fx->s3);
         if (e != cudaSuccess) return e;
     } else {
-        e = cudaFuncSetAttribute(k_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem1);
-        if (e != cudaSuccess) return e;
-        for (int m = 0; m < 4 && e == cudaSuccess; ++m)
-            e = cudaFuncSetAttribute(m == 0   ? k_pass3<kModeDemag>
-                                     : m == 1 ? k_pass3<kModeHeff>
-                                     : m == 2 ? k_pass3<kModeStep>
-                                              : k_pass3<kModeStepX>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem3);
+        e = allow_smem(k_pass1);
+        if (e == cudaSuccess) e = allow_smem(k_pass3<kModeDemag>);
+        if (e == cudaSuccess) e = allow_smem(k_pass3<kModeHeff>);
+        if (e == cudaSuccess) e = allow_smem(k_pass3<kModeStep>);
+        if (e == cudaSuccess) e = allow_smem(k_pass3<kModeStepX>);
         if (e != cudaSuccess) return e;
     }
     if (l.split && l.fs2) return configure_fast_split(*l.fs2);
-    if (l.split) return configure_split_kernels(g);
+    if (l.split) return configure_split_kernels();
     if (l.fp) return cudaFuncSetAttribute(l.fp->pl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.fp->s2);
     PlaneFn pf = plane_fn(g.Lz);
     if (!pf) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute(pf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem2);
+    return allow_smem(pf);
 }
 cudaError_t launch_pass1(const Geom& g, const Launch& l, const float* M, float2* S, cudaStream_t s, float* Mcopy,
                          const XComb& comb) {

@@ -130,6 +130,18 @@ struct StageArgs {
     unsigned* err;
 };
 
+// Let a kernel whose dynamic shared memory follows the sample's size have all
+// that its static part leaves.  The attribute belongs to the kernel, not to
+// a context or a batch: all of the process set the same value, so that none
+// takes it away from another.
+template <typename F> inline cudaError_t allow_smem(F* k) {
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, k);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(227 * 1024 - at.sharedSizeBytes));
+}
+
 // A cell of M.  OWN: the kernel's own blocks rewrite M between two grid barriers
 // of the launch, so the load must not go through the read-only path (whose
 // lines no barrier makes stale); else M does not change while the kernel
@@ -303,7 +315,7 @@ cudaError_t launch_step_b(const Geom& g, const FastStepFns& f, const LlgCoef& c,
 
 // Pass 2 for thick samples (split_kernels.cu); the spectrum row stride is Ly.
 cudaError_t launch_split_plane(const Geom& g, float2* S, cudaStream_t s);
-cudaError_t configure_split_kernels(const Geom& g);
+cudaError_t configure_split_kernels();
 size_t split_smem_y(const Geom& g);
 size_t split_smem_z(const Geom& g);
 

@@ -100,10 +100,9 @@ size_t split_smem_y(const Geom& g) {
 }
 size_t split_smem_z(const Geom& g) { return (size_t)2 * 3 * split_chunk(g) * padded_len(g.Lz) * sizeof(float2); }
 
-cudaError_t configure_split_kernels(const Geom& g) {
-    cudaError_t e = cudaFuncSetAttribute(k_yfft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_smem_y(g));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_zconv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_smem_z(g));
+cudaError_t configure_split_kernels() {
+    const cudaError_t e = allow_smem(k_yfft);
+    return e == cudaSuccess ? allow_smem(k_zconv) : e;
 }
 
 cudaError_t launch_split_plane(const Geom& g, float2* S, cudaStream_t s) {

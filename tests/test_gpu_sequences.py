@@ -111,3 +111,28 @@ def test_batch_field_change_behind_steps_in_flight(path, general):
         got.append(_batch_state(b))
     assert np.all(np.isfinite(got[0]))
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("first,second", [((1100, 40, 4), (1030, 3, 4)), ((1100, 24, 12), (1040, 3, 9))])
+def test_general_contexts_of_different_sizes_alive_together(first, second):
+    """The general kernels' shared memory follows the sample; a context created
+    later with shorter lines leaves an earlier one its own."""
+    from paper_1406_7459_gb300 import mm
+
+    def make(grid):
+        ctx = mm.mm_create(grid, CELL, MS, A_EX, 1e4, 0.2, GAMMA)
+        mm.mm_set_m(ctx, torch.from_numpy(inputs.random_unit_m(grid, MS, 5).reshape(-1)).cuda())
+        return ctx
+
+    got = []
+    for shared in (False, True):
+        ctx = make(first)
+        other = make(second) if shared else None
+        if shared:
+            mm.mm_step(other, 1, 2e-14)
+        mm.mm_step(ctx, 2, 2e-14)
+        out = torch.empty(3 * ctx.N, device="cuda")
+        mm.mm_get_m(ctx, out)
+        mm.mm_sync(ctx)
+        got.append(out)
+    assert torch.isfinite(got[0]).all() and torch.equal(got[0], got[1])
