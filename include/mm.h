@@ -197,9 +197,11 @@ int mm_effective_field(mm_ctx *ctx, const float *M_dev, float *H_dev);
  * x R2C, so a film step is two kernels (on power-of-two films the exchange
  * stencil rides in the tensor spectrum) and a thick sample's four.  Sides
  * that are no powers of two up to 1023 are carried in the next compile-time
- * transform length.  The first 128 steps of a dt are launched directly; from
- * then on steps are replayed from CUDA graphs of 16 (the remainder one step
- * each).
+ * transform length, unless nx alone is none and carrying it would cost more
+ * than the general x passes.  The first 128 steps of a dt are launched
+ * directly; from then on steps are replayed from CUDA graphs of 16, the
+ * remainder launched directly (Runge-Kutta steps on the general kernels: the
+ * first 8 directly, then also one-step graphs).
  * On the square power-of-two films the persistent step is built for
  * (64, 128, 256 wide with nz = 4; 256 x 256 with nz = 1 or 2) the two
  * kernels' work can instead run as one cooperative launch for up to 1024
@@ -224,7 +226,7 @@ int mm_step_form(const mm_ctx *ctx);
  * memory, with the result written back to host memory: the same result as
  * mm_set_m(M_in), mm_step(n, dt), mm_get_m(M_out), bit for bit, with one
  * synchronisation.  M_in, M_out: 3*N float32 in host memory (they may be
- * the same buffer).  On the power-of-two films' Euler step (graph path),
+ * the same buffer).  On the films' two-kernel Euler step (graph path),
  * the kernels themselves read M_in and write M_out over the host link
  * (no staging copies) when the buffers are page-locked, or pageable on a
  * device with coherent access to pageable host memory; otherwise the data

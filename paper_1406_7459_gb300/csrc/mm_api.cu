@@ -698,8 +698,9 @@ static int enqueue_step(mm_ctx* c, int p, double dt, cudaStream_t s) {
 // from).  Inside one graph consecutive steps keep their programmatic
 // launch edges, so a step's first kernel starts while the previous one drains.
 constexpr int kGraphSteps = 16;
-// Steps of one dt that launch directly before graphs are captured.
-constexpr int kWarmSteps = 128;
+// Steps of one dt that launch directly before graphs are captured; the fewer
+// for steps whose launches a graph shortens (graph_steps).
+constexpr int kWarmSteps = 128, kWarmLong = 8;
 
 // Capture one step (kind 0) or kGraphSteps steps (kind 1) from parity p on
 // the private stream into a graph.
@@ -787,6 +788,14 @@ extern "C" int mm_set_wait_limit(mm_ctx* c, long long polls) {
     return MM_OK;
 }
 
+// Whether single steps replay a graph: Runge-Kutta steps on the general
+// kernels, a dozen and more launches without programmatic chains between the
+// stages (set, five RK4 steps and get of 643x16x32 1379 us as one-step graphs,
+// 1430 launched directly; of 1100x6x1 930 and 959).
+static bool graph_steps(const mm_ctx* c) {
+    return !c->has_fs && c->method != MM_INTEGRATOR_EULER && !fused_stages(c);
+}
+
 extern "C" int mm_step(mm_ctx* c, int n, double dt) {
     if (!c) return fail(MM_EINVAL, "null context");
     if (n < 0) return fail(MM_EINVAL, "n must be >= 0");
@@ -815,15 +824,18 @@ extern "C" int mm_step(mm_ctx* c, int n, double dt) {
         // of 16 steps takes ~130 us to capture and instantiate and gains 0.3
         // us per step (a first block of 20 steps of 256x256x4 took 507 us with
         // the capture and 390 so).  Then runs of kGraphSteps replay their
-        // graph, and the remaining single steps of the two-kernel path launch
-        // directly (a flushed 256x256x4 step measured 23.2-23.5 us so against
-        // 24.7 us as a one-step graph).
+        // graph, and the remaining single steps launch directly: their kernels
+        // are chained by programmatic launches, which a graph of one step
+        // breaks at each end (a flushed 256x256x4 step 23.2-23.5 us against
+        // 24.7 as a one-step graph; set, five steps and get of 64x64x16 75
+        // against 94, of 1100x40x4 438 against 453).
         if (c->warm_dt != dt || c->warm_ver != c->ver) {
             c->warm_dt = dt;
             c->warm_ver = c->ver;
             c->warm = 0;
         }
-        if (c->use_graphs && c->warm >= kWarmSteps && (n - s >= kGraphSteps || !c->has_fs)) {
+        const bool single = graph_steps(c);
+        if (c->use_graphs && c->warm >= (single ? kWarmLong : kWarmSteps) && (n - s >= kGraphSteps || single)) {
             const int kind = n - s >= kGraphSteps ? 1 : 0;
             if (!c->step_exec[kind][p] || c->step_dt[kind][p] != dt || c->step_ver[kind][p] != c->ver) {
                 rc = capture_step(c, kind, p, dt);

@@ -22,8 +22,8 @@ def _gpu():
 
 
 # ragged film, ragged block, power-of-two film and block, planes of the
-# large-plane kernel (both kinds), general kernels (their single steps are
-# graphs too); Runge-Kutta stages fused and unfused
+# large-plane kernel (both kinds), general kernels (whose single Runge-Kutta
+# steps are graphs too); Runge-Kutta stages fused and unfused
 RUNS = [((20, 12, 3), "euler"), ((19, 22, 11), "euler"), ((32, 32, 2), "euler"), ((32, 32, 32), "euler"),
         ((256, 512, 4), "euler"), ((129, 385, 4), "euler"), ((1100, 6, 1), "euler"), ((20, 12, 3), "rk4"),
         ((32, 32, 2), "heun"), ((19, 22, 11), "rk4"), ((700, 540, 1), "rk4"), ((1100, 6, 1), "heun")]
