@@ -60,11 +60,11 @@ struct mm_ctx {
     bool use_graphs = true;
     int form = -1;                // mm_step_form of the last run of steps
     FastFns fast;              // compile-time kernels (when the grid has them)
-    FastStepFns fs;            // two-kernel step (power-of-two grids)
-    FastSplitFns fsplit;       // compile-time split pass 2 (thick power-of-two samples)
+    FastStepFns fs;            // two-kernel step (films on compile-time lengths)
+    FastSplitFns fsplit;       // compile-time split pass 2 (thick samples)
     bool has_fs = false;
     bool rag = false;          // has_fs or has_ss through the ragged kernels; Kt is formed on demand
-    bool has_ss = false;       // thick power-of-two samples: split pass 2 + the x-step kernel
+    bool has_ss = false;       // thick samples: compile-time split pass 2 + the x-step kernel
     bool has_gx = false;       // generic x passes: the step's pass 3 also forms the next x spectrum
     float* Kt_ex = nullptr;    // has_ss: tensor spectrum with the exchange stencil folded in (ragged: plain,
                                // on the carrier lengths)

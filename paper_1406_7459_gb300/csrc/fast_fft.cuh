@@ -1,4 +1,5 @@
-// fast_fft.cuh -- compile-time-sized FFT pieces for power-of-two grids.
+// fast_fft.cuh -- compile-time-sized FFT pieces: powers of two and the carrier
+// lengths between them (ragged.cuh).
 //
 // The zero-padded transforms of the demag convolution (Sec. 2, steps (1)-(5);
 // Sec. 3, Eqs. (14)-(16)) have padded length L = 2n on an axis of n cells

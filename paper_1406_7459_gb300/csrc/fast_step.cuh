@@ -1,13 +1,14 @@
-// fast_step.cuh -- the two-kernel Euler step for power-of-two grids.
+// fast_step.cuh -- the two-kernel Euler step of films: power-of-two sides, and
+// ragged ones in their carrier lengths (RAG; ragged.cuh).
 //
 // Step n (spectrum S of M^n already formed):
 //   K_A  k_plane_pdl   per kx plane: y FFT, the z part of the convolution
 //                      as a direct sum over the nz layers with the (x, y)
 //                      tensor spectrum of each z offset (exact, and cheaper
 //                      than a length-2nz transform pair for nz <= 8), the
-//                      tensor product (Eq. (15)), inverse y; S -> Sh.  The
-//                      zero-padded exchange stencil of Eq. (4) rides in the
-//                      same spectrum.
+//                      tensor product (Eq. (15)), inverse y; S -> Sh.  On
+//                      power-of-two films the zero-padded exchange stencil of
+//                      Eq. (4) rides in the same spectrum.
 //   K_B  k_xstep_pdl   per (layer, row pair): inverse x C2R (Eq. (16)), the
 //                      field and LLG update of Eqs. (2)-(6) with the Euler
 //                      step and renormalisation, and then the forward x R2C

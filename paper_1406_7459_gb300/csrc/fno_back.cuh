@@ -8,7 +8,7 @@
 // (0.3 GB); the activation's derivative, the BF16 copy, the weight gradient
 // and the channel map as separate kernels moved 0.77 GB.  Measured there: a
 // layer 97 us against 269 in the four kernels, the head 25 against 140, the
-// lift's gradient 20 against 71, loss and gradients in all 2.88 -> 1.58 ms.
+// lift's gradient 20 against 71, loss and gradients in all 2.87 -> 1.55 ms.
 // A layer is bound by instruction issue (erf and exp of the derivative) next
 // to HBM.
 #pragma once
@@ -462,10 +462,9 @@ __global__ void __launch_bounds__(256) k_back_reduce(BackJobs q) {
 // together).  The eight partial sums are added in k_mode_inv's order, for the
 // same bits ahead of the BF16 rounding.  Bound by the latency of its loads from L2:
 // loss and gradients at 256 x 256, width 32, 16 modes, batch 8 took 1733 us
-// with all eight samples in one block, 1640 with four in each of two (the
-// channels in contiguous quarters; 1529 with the finer y transform, 1583 in
-// this order of the sums; unrolled over all channels of a warp, so that its
-// loads issue together, 1607 -> 1572 in a run of its own).
+// with all eight samples in one block and 1640 with four in each of two; then
+// 1607 with a warp's channels one after the other and 1572 unrolled over
+// them, so that its loads issue together (each pair from one run).
 constexpr int kMixNB = 4;
 __global__ void __launch_bounds__(128) k_mode_mix(const float* __restrict__ vr, const float* __restrict__ vi,
                                                   const float* __restrict__ Rre, const float* __restrict__ Rim, int C,

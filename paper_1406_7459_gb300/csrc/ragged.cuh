@@ -22,8 +22,8 @@
 // transforms with one exchange.  Bound by the latency of two single-wave
 // kernels on small films and by shared memory and the FP32 pipes on large
 // ones, like the power-of-two step.  Per L2-resident Euler step, general
-// kernels against these: 200x60x3 25 against 9.6 us, an RK4 step of
-// 600x400x1 222 against 115.
+// kernels against these: 200x60x3 22.0 against 9.5 us, 300x300x3 52.8 against
+// 42.9, 1000x1000x1 174.6 against 105.1, an RK4 step of it 756 against 405.
 #pragma once
 #include "fast_step.cuh"
 
@@ -83,8 +83,12 @@ template <int NY, int NZ> constexpr bool big_plane_fits() {
 
 // many: the planes fill the SMs (kBigPlanes).  Then the large-plane kernel
 // takes the planes of more than 512 threads, whose registers spill in
-// k_plane_pdl, and those that do not fit it; fewer of them run better on
-// k_plane_pdl or on the split pass.
+// k_plane_pdl, and those that do not fit it.  With fewer planes these stay on
+// k_plane_pdl or on the split pass, which is the better side for the widest
+// planes (per L2-resident Euler step, as it is against the large-plane kernel:
+// 64x512x8 24.5 against 32.3 us, 20x400x6 15.5 against 26.1) but not for four
+// and five layers (128x512x4 25.8 against 21.6, 64x640x4 33.6 against 22.4,
+// 100x400x5 38.6 against 30.0).
 template <int NY, int NZ> bool rag_fill_plane(bool many, FastStepFns* f) {
     if constexpr (big_plane_fits<NY, NZ>() &&
                   (PlaneLayout<NY, NZ>::THREADS > 512 || !rag_plane_fits<NY, NZ>())) {
