@@ -513,7 +513,7 @@ extern "C" int mm_batch_create(mm_batch** out, int n, const int* grids, const do
             float* Ks = b->Kt + koff[s];
             if (e == cudaSuccess)
                 e = b->rag[s].xcls >= 0 ? tensor_spectrum(&grids[3 * s], L, Nd, nullptr, w1, w2, b->stream, Ks,
-                                                          ExchangeFold{}, nullptr, plan_ragged_gain(L))
+                                                          ExchangeFold{}, nullptr, true)
                                         : tensor_spectrum(&grids[3 * s], L, Nd, Ks, w1, w2, b->stream);
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);

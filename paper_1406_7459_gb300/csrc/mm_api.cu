@@ -456,11 +456,10 @@ extern "C" int mm_create(mm_ctx** out, const int grid[3], const double cell[3], 
         exf.idy2 = 1.0 / (c->cell[1] * c->cell[1]);
         exf.idz2 = 1.0 / (c->cell[2] * c->cell[2]);
         if (e == cudaSuccess && c->rag && c->has_ss)
-            e = tensor_spectrum(c->grid, L, Nd, c->Kt_ex, w1, w2, c->stream, nullptr, ExchangeFold{}, nullptr,
-                                plan_ragged_gain(L));
+            e = tensor_spectrum(c->grid, L, Nd, c->Kt_ex, w1, w2, c->stream, nullptr, ExchangeFold{}, nullptr, true);
         else if (e == cudaSuccess && c->rag)
             e = tensor_spectrum(c->grid, L, Nd, nullptr, w1, w2, c->stream, c->Kd0, ExchangeFold{}, nullptr,
-                                plan_ragged_gain(L));
+                                true);
         else if (e == cudaSuccess)
             e = tensor_spectrum(c->grid, L, Nd, c->Kt, w1, w2, c->stream, c->Kd, exf, c->Kd0);
         if (e == cudaSuccess && c->has_ss && !c->rag) {

@@ -156,7 +156,9 @@ template <bool OWN> __device__ __forceinline__ float load_m(const float* p) {
 // Planning helpers (mm_api.cu), shared with the batched driver.
 int plan_padded_length(int n);
 int plan_ragged_len(int n);        // carrier length of a ragged side, or 0 (ragged_select.cu)
-double plan_ragged_gain(const int L[3]);   // of the transforms there and back on padded carrier lengths
+// 1 / gain of the wavenumbers 0 .. L/2 of a padded carrier length's transforms
+// there and back (ragged_gain.cu); z: of the split pass's z columns.
+void ragged_inverse_gains(int L, bool z, double* out);
 bool plan_axis(int L, AxisPlan* p);
 void plan_twiddles(int L, float2* out);
 int set_error(int code, const char* msg);
@@ -365,11 +367,11 @@ struct ExchangeFold {
     int nx, ny, Lx, Ly;
     double pexch, idx2, idy2, idz2;
 };
-// (Kt_dev null: only the 2-D spectra).  The spectra are divided by `gain`, that
-// of the transforms that will use them.
+// (Kt_dev null: only the 2-D spectra).  carried: spectra for the transforms on
+// carrier lengths, divided by their gains.
 cudaError_t tensor_spectrum(const int grid[3], const int L[3], const double* N_dev, float* Kt_dev,
                             double* work1, double* work2, cudaStream_t s, float* Kd_dev = nullptr,
-                            ExchangeFold ex = ExchangeFold{}, float* Kd0_dev = nullptr, double gain = 1.0);
+                            ExchangeFold ex = ExchangeFold{}, float* Kd0_dev = nullptr, bool carried = false);
 // Kt_ex = Kt plus the zero-padded 7-point exchange stencil's symbol on the
 // diagonal (the 3-D counterpart of the fold into Kd).
 cudaError_t tensor_fold_exchange3(const Geom& g, ExchangeFold ex, const float* Kt, float* Kt_ex, cudaStream_t s);

@@ -38,39 +38,6 @@ inline int ragged_len(int n) {
     return 0;
 }
 
-// Gain of a carrier length's padded transform and its inverse, minus one.  The
-// butterflies' FP32 constants and the table entries have moduli that are not
-// one (0.70710677 for sqrt(1/2), 0.9238795, 0.3826834 for the sixteenth of the
-// circle), and the nearest values of the few constants in the butterflies
-// happen to lie below: forward and back, a line loses this share of itself.
-// The values are the mean over the 2 N wavenumbers of inverse times forward,
-// carried out in FP64 with the constants of fft_device.cuh and fast_fft.cuh
-// as they are rounded (they spread by 1.4e-8 to 2.4e-8 over the wavenumbers).
-// The spectrum's normalisation makes up for it.  Without, H_demag of 100x80x20
-// was 1.5e-7 too small, as large as all its other rounding.
-inline double ragged_gain_minus_one(int N) {
-    switch (N) {
-        case 4: return -0.86e-8;
-        case 8: return -2.71e-8;
-        case 16: return -4.12e-8;
-        case 24: return -4.27e-8;
-        case 32: return -4.40e-8;
-        case 48: return -5.31e-8;
-        case 64: return -4.07e-8;
-        case 96: return -6.75e-8;
-        case 128: return -4.44e-8;
-        case 192: return -6.32e-8;
-        case 256: return -5.38e-8;
-        case 320: return -0.23e-8;
-        case 384: return -6.89e-8;
-        case 512: return -6.83e-8;
-        case 640: return -1.56e-8;
-        case 768: return -8.25e-8;
-        case 1024: return -8.68e-8;
-        default: return 0.0;                  // 1 and 2: no rounded constant
-    }
-}
-
 // k_plane_pdl exists where a plane's threads and shared memory fit, the
 // large-plane kernel for transform groups of a warp where its lines fit.
 template <int NY, int NZ> constexpr bool rag_plane_fits() {

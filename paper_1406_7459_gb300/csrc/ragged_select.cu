@@ -43,12 +43,6 @@ bool ragged_lookup(int nx, int ny, int nz, FastStepFns* f, int* NX, int* NY) {
 
 int plan_ragged_len(int n) { return ragged_len(n); }
 
-double plan_ragged_gain(const int L[3]) {
-    double g = 1.0;
-    for (int a = 0; a < 3; ++a) g *= 1.0 + ragged_gain_minus_one(L[a] / 2);
-    return g;
-}
-
 bool ragged_batchable(int nx, int ny, int nz) {
     return rag_x_class(ragged_len(nx)) >= 0 && rag_plane_class(ragged_len(ny), nz) >= 0;
 }

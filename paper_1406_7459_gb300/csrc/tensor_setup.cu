@@ -18,6 +18,7 @@
 // over the non-negative offsets and stored on the octant kx, ky, kz in
 // [0, L/2] in FP32, with the inverse-FFT factor 1/(Lx Ly Lz) folded in.
 #include <cmath>
+#include <vector>
 
 #include "mm_internal.h"
 
@@ -214,8 +215,8 @@ __global__ void k_ty(int ny, int nz, int Hx, int Ly, int Hy, const double* __res
 
 // Transform along z and pack: in[c][k][ky][kx] -> Kt[kx][kz][ky][c] (FP32),
 // K~ = -(sign) N~ / (Lx Ly Lz), sign = (-i)^2 = -1 for the off-diagonals.
-__global__ void k_tz(int nz, int Hx, int Hy, int Lz, int Hz, double scale, const double* __restrict__ in,
-                     float* __restrict__ Kt, const double2* __restrict__ cs) {
+__global__ void k_tz(int nz, int Hx, int Hy, int Lz, int Hz, double scale, const double* __restrict__ gain,
+                     const double* __restrict__ in, float* __restrict__ Kt, const double2* __restrict__ cs) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t total = (size_t)6 * Hx * Hy * Hz;
     if (t >= total) return;
@@ -235,6 +236,7 @@ __global__ void k_tz(int nz, int Hx, int Hy, int Lz, int Hz, double scale, const
         acc += src[k * kstride] * (odd ? v.y : v.x);
     }
     const bool offdiag = (c == 1 || c == 2 || c == 4);
+    if (gain) scale *= gain[kx] * gain[Hx + ky] * gain[Hx + Hy + kz];
     Kt[t] = (float)((offdiag ? scale : -scale) * (2.0 * acc));
 }
 
@@ -253,8 +255,8 @@ __global__ void k_tz(int nz, int Hx, int Hy, int Lz, int Hz, double scale, const
 // zero-padded 7-point stencil (its free-boundary remainder, M(i) times the
 // number of missing neighbours / delta^2, is added per cell by the update
 // kernel), so that the update needs no neighbour cells.
-__global__ void k_pack2d(int nz, int Hx, int Hy, int Hyp, double scale, const double* __restrict__ in,
-                         float* __restrict__ Kd, ExchangeFold ex) {
+__global__ void k_pack2d(int nz, int Hx, int Hy, int Hyp, double scale, const double* __restrict__ gain,
+                         const double* __restrict__ in, float* __restrict__ Kd, ExchangeFold ex) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t total = (size_t)6 * Hx * Hyp * nz;
     if (t >= total) return;
@@ -286,6 +288,7 @@ __global__ void k_pack2d(int nz, int Hx, int Hy, int Hyp, double scale, const do
         }
         e *= ex.pexch;
     }
+    if (gain) scale *= gain[kx] * gain[Hx + ky];
     Kd[t] = (float)(scale * (sg * v + e));
 }
 
@@ -358,12 +361,27 @@ size_t tensor_work_elems(const int grid[3], const int L[3]) {
 
 cudaError_t tensor_spectrum(const int grid[3], const int L[3], const double* N_dev, float* Kt_dev,
                             double* work1, double* work2, cudaStream_t s, float* Kd_dev, ExchangeFold ex,
-                            float* Kd0_dev, double gain) {
+                            float* Kd0_dev, bool carried) {
     const int nx = grid[0], ny = grid[1], nz = grid[2];
     const int Hx = L[0] / 2 + 1, Hy = L[1] / 2 + 1, Hz = L[2] / 2 + 1;
     double2* cs = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&cs, sizeof(double2) * (L[0] + L[1] + L[2]), s);
+    // the twiddles, then the inverse gains of the three axes
+    const int ntw = L[0] + L[1] + L[2], ng = Hx + Hy + Hz;
+    cudaError_t e = cudaMallocAsync((void**)&cs, sizeof(double2) * ntw + sizeof(double) * ng, s);
     if (e != cudaSuccess) return e;
+    double* gain = nullptr;
+    if (carried) {
+        std::vector<double> h(ng);
+        ragged_inverse_gains(L[0], false, h.data());
+        ragged_inverse_gains(L[1], false, h.data() + Hx);
+        ragged_inverse_gains(L[2], true, h.data() + Hx + Hy);
+        gain = reinterpret_cast<double*>(cs + ntw);
+        e = cudaMemcpyAsync(gain, h.data(), sizeof(double) * ng, cudaMemcpyHostToDevice, s);
+        if (e != cudaSuccess) {
+            cudaFreeAsync(cs, s);
+            return e;
+        }
+    }
     double2 *csx = cs, *csy = cs + L[0], *csz = cs + L[0] + L[1];
     const int T = 256;
     k_cos_sin<<<(L[0] + T - 1) / T, T, 0, s>>>(L[0], csx);
@@ -376,16 +394,16 @@ cudaError_t tensor_spectrum(const int grid[3], const int L[3], const double* N_d
     if (Kd_dev) {
         const int Hyp = kd_row(Hy);
         const size_t nd = (size_t)6 * Hx * Hyp * nz;
-        k_pack2d<<<(unsigned)((nd + T - 1) / T), T, 0, s>>>(nz, Hx, Hy, Hyp, 1.0 / (gain * L[0] * L[1]), work2,
-                                                            Kd_dev, ex);
+        k_pack2d<<<(unsigned)((nd + T - 1) / T), T, 0, s>>>(nz, Hx, Hy, Hyp, 1.0 / ((double)L[0] * L[1]), gain,
+                                                            work2, Kd_dev, ex);
         if (Kd0_dev)
-            k_pack2d<<<(unsigned)((nd + T - 1) / T), T, 0, s>>>(nz, Hx, Hy, Hyp, 1.0 / (gain * L[0] * L[1]), work2,
-                                                                Kd0_dev, ExchangeFold{});
+            k_pack2d<<<(unsigned)((nd + T - 1) / T), T, 0, s>>>(nz, Hx, Hy, Hyp, 1.0 / ((double)L[0] * L[1]),
+                                                                gain, work2, Kd0_dev, ExchangeFold{});
     }
     if (Kt_dev) {
         const size_t n3 = (size_t)6 * Hx * Hy * Hz;
-        const double scale = 1.0 / (gain * L[0] * L[1] * L[2]);
-        k_tz<<<(unsigned)((n3 + T - 1) / T), T, 0, s>>>(nz, Hx, Hy, L[2], Hz, scale, work2, Kt_dev, csz);
+        const double scale = 1.0 / ((double)L[0] * L[1] * L[2]);
+        k_tz<<<(unsigned)((n3 + T - 1) / T), T, 0, s>>>(nz, Hx, Hy, L[2], Hz, scale, gain, work2, Kt_dev, csz);
     }
     e = cudaGetLastError();
     cudaError_t e2 = cudaFreeAsync(cs, s);
